@@ -95,7 +95,7 @@ struct HostCase {
     // node's weight (1/2 or 1/4 for a node with u = 0 or v = 0, stored in two or four classes)
     std::vector<int> vcan, vcls;
     std::vector<double> vfac;
-    int k1b, k2b, k3b, k4b, ksb, ktb;
+    int k1b, k2b, k3b, k4b, ksb;
     int k4shape;
     int k1sep;                      // face sums by v-moments: no zero node, every sign class 1..32 u-nodes wide
     int pairs;                      // every sign class holds an even number of velocity blocks
@@ -272,9 +272,8 @@ void fill_host(HostCase& h, const hbugks_case& c)
             o[2] = W.T_mean + W.T_re * cs - W.T_im * sn;   // Eq. bc_temp
         }
     h.k2b = (h.nf * h.nt + 127) / 128;
-    h.k3b = (h.nc + K3_THREADS - 1) / K3_THREADS;
+    h.k3b = (h.nc + K3_CELLS - 1) / K3_CELLS;
     h.ksb = (h.nc + 127) / 128;
-    h.ktb = (h.nc * h.nt + KT_ITEMS - 1) / KT_ITEMS;
 }
 
 template <typename T>
@@ -293,6 +292,10 @@ void layout_case(Carver& cv, const HostCase& h, CaseDev<T>& d)
     for (int k = 0; k < 8; ++k) d.e[k] = 0.0;
     for (int dd = 1; dd <= h.nh; ++dd) d.e[dd] = ((dd & 1) ? -0.5 : 0.5) / sin(M_PI * dd / h.nt);   // Eq. D_explicit
     for (int k = 0; k < 8; ++k) d.et[k] = T(d.e[k]);
+    for (int k = 0; k < MAXNT; ++k) {
+        d.ct[k] = cos(2.0 * M_PI * k / h.nt);
+        d.snt[k] = sin(2.0 * M_PI * k / h.nt);
+    }
     d.spectral_implicit = h.src.phys.spectral_implicit;
     d.minv = cv.take<T>((size_t)h.nc * h.nt * h.nt);
     d.nslot = h.nslot;
@@ -348,7 +351,7 @@ void layout_case(Carver& cv, const HostCase& h, CaseDev<T>& d)
 
 // one kernel launch of the iteration covering every case it applies to
 struct LaunchSpec {
-    int kind;      // 0 K1 tile, 1 K2, 2 K3, 3 tables, 4 K4 tile, 5 steps
+    int kind;      // 0 K1 tile, 1 K2, 2 K3 (with the equilibrium tables), 4 K4 tile, 5 steps
     int shape;     // tile shape index (K1, K4)
     int table;     // block offset table index
     int total;     // total blocks
@@ -369,6 +372,7 @@ struct Impl {
     std::vector<int> off_host;
     std::vector<LaunchSpec> specs;   // in launch order (without the residual kernel)
     int k3_table = 0, steps_table = 0;
+    int max_nt = 1;                  // the largest N_T of the cases
     bool any_implicit = false;       // some case takes the spectral source at the new iterate
 };
 
@@ -411,6 +415,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
         HostCase& h = im.hc[k];
         fill_host(h, cases[k]);
         h.k4shape = pick_k4_shape<T>(h.nt);
+        im.max_nt = std::max(im.max_nt, h.nt);
         h.k1b = ((h.nx + K1_TX<T> - 1) / K1_TX<T>) * ((h.ny + K1_TY<T> - 1) / K1_TY<T>) * h.nt;
         set_k4_blocks(h);
     }
@@ -420,7 +425,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
     im.d_err = cv.take<int>(2);
     im.d_loop = cv.take<int>(2);
     im.d_tune_off = cv.take<int>(2);
-    // launch specs: K1 per shape, K2, K3, tables, K4 per shape; plus the step kernel (state setting only)
+    // launch specs: K1 per shape, K2, K3, K4 per shape; plus the step kernel (state setting only)
     im.specs.clear();
     auto add = [&](int kind, int shape) { im.specs.push_back(LaunchSpec{kind, shape, (int)im.specs.size(), 0, 0}); };
     add(0, 0);
@@ -428,7 +433,6 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
     add(1, 0);
     add(2, 0);
     im.k3_table = (int)im.specs.size() - 1;
-    add(3, 0);
     for (int sh = 0; sh < N_K4_SHAPES; ++sh) add(4, sh);
     add(5, 0);
     im.steps_table = (int)im.specs.size() - 1;
@@ -462,7 +466,6 @@ void fill_offsets(Impl<T>& im, int ncases)
                 case 0: nb = h.k1sep == sp.shape ? h.k1b : 0; smem = k1_smem_of<T>(); break;
                 case 1: nb = h.k2b; break;
                 case 2: nb = h.k3b; break;
-                case 3: nb = h.ktb; break;
                 case 4: if (h.k4shape == sp.shape) { nb = h.k4b; smem = std::max(smem, k4_smem_of<T>(sp.shape, h.nt)); } break;
                 case 5: nb = h.ksb; break;
             }
@@ -736,7 +739,7 @@ cudaError_t set_smem_attributes()
 
 // Kernel kinds reported by the profiler: 0 face moments, 1 face parameters, 2 macro update (with the
 // equilibrium tables), 3 micro update, 4 residual.
-inline int profile_slot(int kind) { return kind == 0 ? 0 : kind == 1 ? 1 : (kind == 2 || kind == 3) ? 2 : 3; }
+inline int profile_slot(int kind) { return kind == 0 ? 0 : kind == 1 ? 1 : kind == 2 ? 2 : 3; }
 
 // one iteration; with `ev` (2 events per kernel kind, 5 kinds) each kind is bracketed by an event pair
 template <typename T>
@@ -753,13 +756,16 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
             open_slot = slot;
         }
         Batch<T> b{im.d_cases, ncases, im.d_off + (size_t)sp.table * stride};
-        static const char* const names[5] = {"k1_cells", "k2_face_params", "k3_macro", "k_tables", "k4_cells"};
+        static const char* const names[5] = {"k1_cells", "k2_face_params", "k3_macro", "", "k4_cells"};
         Range r(names[sp.kind]);
         switch (sp.kind) {
             case 0: launch_k1<T>(sp.shape, sp.total, sp.smem, b, s); break;
             case 1: k2_face_params<T><<<sp.total, 128, 0, s>>>(b); break;
-            case 2: k3_macro<T><<<sp.total, K3_THREADS, 0, s>>>(b); break;
-            case 3: k_tables<T><<<sp.total, KT_ITEMS, 0, s>>>(b); break;
+            case 2: {
+                Range rt("k_tables");          // the same launch writes the equilibrium tables
+                k3_macro<T><<<sp.total, k3_threads(im.max_nt), 0, s>>>(b);
+                break;
+            }
             case 4: launch_k4<T>(im.any_implicit, sp.shape, sp.total, sp.smem, b, s); break;
         }
     }
@@ -769,7 +775,7 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
     }
     {
         Range r("k5_finish");
-        k5_finish<T><<<ncases, 32, 0, s>>>(im.d_cases, ncases, im.d_off + (size_t)im.k3_table * stride);
+        k5_finish<T><<<ncases, K5_THREADS, 0, s>>>(im.d_cases, ncases, im.d_off + (size_t)im.k3_table * stride);
     }
     if (ev) cudaEventRecord(ev[9], s);
 }

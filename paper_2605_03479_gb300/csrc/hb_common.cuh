@@ -22,7 +22,7 @@ constexpr int NCM = 13;       // cell moments per (cell, level)
 constexpr int NP = 44;        // face parameters per (face, level), 16-byte aligned blocks
 constexpr int NCP = 36;       // cell parameters per (cell, level)
 constexpr int RING = 4096;    // residual history slots per case
-constexpr int K3_THREADS = 128;
+constexpr int K3_CELLS = 8;   // cells per CTA of the macro update
 constexpr int WCN = 18;       // per wall and level: Aw[13] (reflected-half raw moments, unit density), Dw, Gw[4]
 
 // ------------------------------------------------------------------ (h, b) pairs and packed arithmetic
@@ -97,6 +97,7 @@ struct CaseDev {
     int face_step;
     double omega, mu0, w_vss, pr, cfl, gam, umax, vmax, lam0;
     double e[8];                       // e_d = (-1)^d / (2 sin(pi d / N_T)), d = 1..N_H
+    double ct[MAXNT], snt[MAXNT];      // cos, sin(2 pi j / N_T)
     T et[8];                           // the same in the storage precision
     int spectral_implicit;             // spectral source at the new pseudo-time iterate
     T* minv;                           // [nc][nt][nt] inverse of diag(1 + dG/(2 tau_n^{k+1})) + dG omega E (implicit)
@@ -270,19 +271,35 @@ template <typename T> __device__ __forceinline__ T t_expm1(T x);
 template <> __device__ __forceinline__ double t_expm1<double>(double x) { return expm1(x); }
 template <> __device__ __forceinline__ float t_expm1<float>(float x) { return expm1f(x); }
 
+// 1 / x in double precision by Newton's iteration in its cubically convergent form r (1 + e + e^2), e = 1 - x r,
+// from the hardware's approximation (relative error about 2^-20, so e^3 lies below the last bit): 3 FMAs, within
+// 1 ulp, where a correctly rounded division costs 9.  An FP64 instruction occupies its scheduler for 64 cycles here,
+// so the per-cell and per-face arithmetic and the FP64 slopes pay for every one of them.  x = 0 or infinite gives NaN.
+__device__ __forceinline__ double rcp64(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 // primitive variables from W = (rho, rho U, rho V, rho E) with D + K = 3
 __device__ __forceinline__ void prim(const double* W, double& rho, double& U, double& V, double& lam)
 {
     rho = W[0];
-    U = W[1] / rho;
-    V = W[2] / rho;
-    lam = 0.75 * rho / (W[3] - 0.5 * rho * (U * U + V * V));
+    const double ir = rcp64(rho);
+    U = W[1] * ir;
+    V = W[2] * ir;
+    // fused as written, so that every kernel forms the same bits from the same W
+    lam = 0.75 * rho * rcp64(fma(-0.5 * rho, fma(U, U, V * V), W[3]));
 }
 
-// tau = mu/p, mu = mu0 (T/T0)^w, T/T0 = lam0/lam, p = rho/(2 lam)
-__device__ __forceinline__ double relax_time(double mu0, double w, double lam0, double rho, double lam)
+// tau = mu/p, mu = mu0 (T/T0)^w, T/T0 = lam0/lam, p = rho/(2 lam); ir = 1/rho, il0 = 1/lam0.  The power as
+// exp(-w log(lam/lam0)): both within a few ulp, for half the instructions of pow, whose extra digits of the
+// logarithm serve exponents far from the w = 0.5..1 of a viscosity law.
+__device__ __forceinline__ double relax_time(double mu0, double w, double il0, double ir, double lam)
 {
-    return mu0 * pow(lam0 / lam, w) * 2.0 * lam / rho;
+    return mu0 * exp(-w * log(lam * il0)) * 2.0 * lam * ir;
 }
 
 // Coefficients of Eq. C_coeffs: Taylor series in x = dG/tau below x = 1 (the printed forms cancel there),
@@ -360,15 +377,15 @@ __device__ inline void shakhov_poly(double s, double qx, double qy, double U, do
 // factor s (c.q)(2 lam |c|^2 - 4), s = (1 - Pr) 4 lam^2 / (5 rho), c = u - U, kept as its linear factor
 // L = s (c.q) and quadratic factor 2 lam |c|^2 - 4 (Eq. shakhov integrated over xi)
 template <typename T>
-__device__ inline void eq_cell(double rho, double U, double V, double lam, double lam0, double pr, double qx, double qy,
+__device__ inline void eq_cell(double rho, double U, double V, double lam, double il0, double pr, double qx, double qy,
                                T* o)
 {
-    const double r = rho * lam / lam0;
+    const double r = rho * lam * il0, i2l = 0.5 * rcp64(lam);
     o[E_RM1] = T(r - 1.0);
     o[E_R] = T(r);
-    o[E_I2L] = T(0.5 / lam);
-    o[E_DI2L] = T(0.5 / lam - 0.5 / lam0);
-    const double s = (1.0 - pr) * 4.0 * lam * lam / (5.0 * rho);
+    o[E_I2L] = T(i2l);
+    o[E_DI2L] = T(i2l - 0.5 * il0);
+    const double s = (1.0 - pr) * 0.8 * lam * lam * rcp64(rho);
     o[E_L] = T(-s * (qx * U + qy * V));
     o[E_L + 1] = T(s * qx);
     o[E_L + 2] = T(s * qy);

@@ -8,8 +8,9 @@
 //   K2 face_params  : per (face, level): interface Maxwellian, tau, dG_f (Eq. dt_face), C1..C5 (Eq. C_coeffs),
 //                     slopes a^L, a^R, a_t and A (compatibility), diffuse-wall density (Eq. rho_wall), the
 //                     macro flux (Eq. macro_flux) and the parameters the micro update needs
-//   K3 macro_update : per cell: W^{k+1} (Eq. fv_W with the spectral source), the collision coefficients of
-//                     Eq. fv_h, the next local step (Eqs. dt_hb, nu_conv) and the level-0 residual partials
+//   K3 macro_update : per (cell, level): W^{k+1} (Eq. fv_W with the spectral source), the collision coefficients
+//                     of Eq. fv_h, the equilibrium tables; per cell the next local step (Eqs. dt_hb, nu_conv) and
+//                     the level-0 residual partials
 //   K4 micro_update : per (cell, 32 velocities): interface micro fluxes (Eq. micro_flux), spectral source
 //                     across levels and the semi-implicit collision update (Eq. fv_h)
 //   K5 finish       : per case: residual (Eq. benchmark_residuals), convergence / divergence status
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(128) k2_face_params(Batch<T> B)
     prim(W0, rho0, U0, V0, lamf);
     double q0x, q0y;
     heat_flux_raw(Amix, U0, V0, q0x, q0y);
-    const double tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, rho0, lamf);
+    const double tau = relax_time(cd.mu0, cd.w_vss, rcp64(cd.lam0), rcp64(rho0), lamf);
 
     // ---- face step (Eq. dt_face) and time-integration weights (Eq. C_coeffs)
     const int cL = g.jL * cd.nx + g.iL, cR = g.jR * cd.nx + g.iR;
@@ -414,78 +415,22 @@ __global__ void __launch_bounds__(128) k2_face_params(Batch<T> B)
     }
 }
 
-// ------------------------------------------------------------------------------ separable Maxwellian tables
-
-// Tables of expm1(lam0 x^2 - lam (x - U)^2) over the 1-D velocity nodes, so that for a Maxwellian of density
-// rho: H - H_ref = H_ref [(r - 1) + r (ex + ey + ex ey)], r = rho lam / lam0.  The cell-level tables of W^k and
-// W^{k+1}: a CTA takes 128 cell-levels; each thread first forms the exponent coefficients of one of them in
-// FP64 (one thread per cell-level, so the slow FP64 divisions run on every lane), then each warp writes the
-// tables of 32 of them with its lanes over the nodes.  (The interface and wall tables are formed in
-// k2_face_params.)
-constexpr int KT_ITEMS = 128;   // cell-levels per CTA of k_tables (one per thread)
-
-template <typename T>
-__global__ void __launch_bounds__(KT_ITEMS) k_tables(Batch<T> B)
-{
-    const int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
-    if (!cd.st->active || *(volatile int*)cd.err) return;
-    __shared__ T coef[KT_ITEMS][2][5];
-    const int nt = cd.nt, nuv = cd.nu + cd.nv, nitems = cd.nc * nt;
-    const int first = (blockIdx.x - B.off[cs]) * KT_ITEMS;   // cell-level pairs first.., item = c * nt + n
-    const int p = cd.st->parity;
-    {
-        const int item = first + threadIdx.x;
-        if (item < nitems) {
-            for (int e = 0; e < 2; ++e) {
-                double rho, U, V, lam;
-                prim((e == 0 ? cd.W[p] : cd.W[p ^ 1]) + ((size_t)(item % nt) * cd.nc + item / nt) * 4, rho, U, V, lam);
-                T* q = coef[threadIdx.x][e];
-                q[0] = T(cd.lam0 - lam);
-                q[1] = T(2.0 * lam * U);
-                q[2] = T(lam * U * U);
-                q[3] = T(2.0 * lam * V);
-                q[4] = T(lam * V * V);
-            }
-        }
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int r = 0; r < 32; ++r) {
-        const int li = warp * 32 + r, item = first + li;
-        if (item >= nitems) break;
-        for (int e = 0; e < 2; ++e) {
-            const T* c = coef[li][e];
-            T* dst = cd.ctab + ((size_t)item * 2 + e) * nuv;
-            for (int k = lane; k < cd.nu; k += 32) {
-                const T x = cd.tu1[k];
-                dst[k] = t_expm1<T>(c[0] * x * x + c[1] * x - c[2]);
-            }
-            for (int k = lane; k < cd.nv; k += 32) {
-                const T y = cd.tv1[k];
-                dst[cd.nu + k] = t_expm1<T>(c[0] * y * y + c[3] * y - c[4]);
-            }
-        }
-    }
-}
-
 // ------------------------------------------------------------------------------ local pseudo-time step
+
+// nu_conv of one (cell, level) with the cell's 1/dx, 1/dy (Eq. nu_conv); k_steps and k3_macro form the same bits, so
+// a state that is set from a checkpoint continues exactly
+template <typename T>
+__device__ __forceinline__ double nu_conv(const CaseDev<T>& cd, double U, double V, double lam, double rdx, double rdy)
+{
+    const double cs = sqrt(0.5 * cd.gam * rcp64(lam));
+    return fma(fmax(fabs(cd.umax), fabs(U)) + cs, rdx, (fmax(fabs(cd.vmax), fabs(V)) + cs) * rdy);
+}
 
 // Eqs. dt_hb, nu_conv: dG_i = CFL / (max_n nu_conv,i,n + omega N_H)
 template <typename T>
-__device__ __forceinline__ double local_step(const CaseDev<T>& cd, const double* W, int c, int i, int j)
+__device__ __forceinline__ double local_step(const CaseDev<T>& cd, double numax)
 {
-    const double dx = 2.0 * cd.hx[i], dy = 2.0 * cd.hy[j];
-    double numax = 0.0;
-    for (int n = 0; n < cd.nt; ++n) {
-        double rho, U, V, lam;
-        prim(W + ((size_t)n * cd.nc + c) * 4, rho, U, V, lam);
-        double cs = sqrt(cd.gam / (2.0 * lam));
-        double ut = fmax(fabs(cd.umax), fabs(U)) + cs;
-        double vt = fmax(fabs(cd.vmax), fabs(V)) + cs;
-        numax = fmax(numax, (dy * ut + dx * vt) / (dx * dy));
-    }
-    return cd.cfl / (numax + cd.omega * cd.nh);
+    return cd.dt_fixed > 0.0 ? cd.dt_fixed : cd.cfl / fma(cd.omega, (double)cd.nh, numax);
 }
 
 template <typename T>
@@ -495,179 +440,236 @@ __global__ void k_steps(Batch<T> B)
     const CaseDev<T>& cd = B.cases[cs];
     int c = (blockIdx.x - B.off[cs]) * blockDim.x + threadIdx.x;
     if (c >= cd.nc) return;
-    cd.dG[c] = cd.dt_fixed > 0.0 ? cd.dt_fixed : local_step(cd, cd.W[cd.st->parity], c, c % cd.nx, c / cd.nx);
+    const double rdx = rcp64(2.0 * cd.hx[c % cd.nx]), rdy = rcp64(2.0 * cd.hy[c / cd.nx]);
+    double numax = 0.0;
+    for (int n = 0; n < cd.nt; ++n) {
+        double rho, U, V, lam;
+        prim(cd.W[cd.st->parity] + ((size_t)n * cd.nc + c) * 4, rho, U, V, lam);
+        numax = fmax(numax, nu_conv(cd, U, V, lam, rdx, rdy));
+    }
+    cd.dG[c] = local_step(cd, numax);
 }
 
 // ------------------------------------------------------------------------------ K3 macro update
 
-// A = diag(D) + dG omega E (D = 1 when null), E of Eq. D_explicit from the paired offsets e_d:
-// E_{n, n-d} = e_d, E_{n, n+d} = -e_d (levels cyclic)
-template <typename T>
-__device__ void spectral_matrix(const CaseDev<T>& cd, double dG, const double* D, double (&A)[MAXNT][MAXNT])
-{
-    const int nt = cd.nt;
-    for (int n = 0; n < nt; ++n)
-        for (int m = 0; m < nt; ++m) A[n][m] = n == m ? (D ? D[n] : 1.0) : 0.0;
-    for (int n = 0; n < nt; ++n)
-        for (int d = 1; d <= cd.nh; ++d) {
-            int nm = n - d; if (nm < 0) nm += nt;
-            int np = n + d; if (np >= nt) np -= nt;
-            A[n][nm] += dG * cd.omega * cd.e[d];
-            A[n][np] -= dG * cd.omega * cd.e[d];
-        }
-}
-
-// Solve A X = R in place for the columns of R (R becomes X), A destroyed: Gaussian elimination with partial
-// pivoting over the levels
-template <int NR>
-__device__ void solve_levels(int nt, double (&A)[MAXNT][MAXNT], double (&R)[MAXNT][NR])
-{
-    for (int k = 0; k < nt; ++k) {
-        int piv = k;
-        for (int i = k + 1; i < nt; ++i)
-            if (fabs(A[i][k]) > fabs(A[piv][k])) piv = i;
-        if (piv != k) {
-            for (int j = 0; j < nt; ++j) { const double t = A[k][j]; A[k][j] = A[piv][j]; A[piv][j] = t; }
-            for (int j = 0; j < NR; ++j) { const double t = R[k][j]; R[k][j] = R[piv][j]; R[piv][j] = t; }
-        }
-        for (int i = k + 1; i < nt; ++i) {
-            const double f = A[i][k] / A[k][k];
-            for (int j = k; j < nt; ++j) A[i][j] -= f * A[k][j];
-            for (int j = 0; j < NR; ++j) R[i][j] -= f * R[k][j];
-        }
-    }
-    for (int k = nt - 1; k >= 0; --k)
-        for (int j = 0; j < NR; ++j) {
-            double s = R[k][j];
-            for (int m = k + 1; m < nt; ++m) s -= A[k][m] * R[m][j];
-            R[k][j] = s / A[k][k];
-        }
-}
+// A CTA takes K3_CELLS cells on all their levels, in two halves of its warps: threads 0.. form W^k's primitive
+// variables, heat flux and relaxation time of one (cell, level) each, threads half.. the new W and those of W^{k+1};
+// they exchange what the other side needs through shared memory and each writes its equilibrium's parameters.  All
+// warps then write the expm1 tables of the CTA's equilibria.  Bound by FP64 instructions, and on small meshes by
+// the length of one thread's chain of them: the previous layout (a thread per cell running over its levels, then a
+// kernel of 128 cell-levels per CTA for the tables) left most of the chip idle.  Measured before -> now, both parts:
+// 115 -> 18 us (8x8 cells, N_T 3), 262 -> 57 us (64x64, N_T 7), 482 -> 255 us (128x128, N_T 11), 754 -> 49 us (32x32,
+// N_T 11, spectral source at the new iterate), 236 -> 36 us (32x32, N_T 3, FP64 tables).  8 cells per CTA give a
+// 32x32 mesh 128 CTAs and still fill three quarters of the lanes at N_T = 3.
+constexpr int K3_MAXTHREADS = 2 * ((MAXNT * K3_CELLS + 31) / 32) * 32;
+// warps of one half for nt levels, and threads of the launch for the largest nt of its cases (at least four warps,
+// one per scheduler, for the tables)
+__host__ __device__ constexpr int k3_half(int nt) { return (nt * K3_CELLS + 31) / 32 * 32; }
+__host__ __device__ constexpr int k3_threads(int nt) { return 2 * k3_half(nt) < 128 ? 128 : 2 * k3_half(nt); }
 
 template <typename T>
-__global__ void __launch_bounds__(K3_THREADS) k3_macro(Batch<T> B)
+__global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
 {
-    int cs = find_case(B.off, B.ncases, blockIdx.x);
+    const int cs = find_case(B.off, B.ncases, blockIdx.x);
     const CaseDev<T>& cd = B.cases[cs];
+    // uniform over the CTA: neither word changes while this kernel runs
     if (!cd.st->active || *(volatile int*)cd.err) return;
+    __shared__ T coef[K3_CELLS * MAXNT * 2][5];            // exponent coefficients of the tables, row (cell, level, e)
+    __shared__ double sq[MAXNT * K3_CELLS][2], stau[MAXNT * K3_CELLS], snu[MAXNT * K3_CELLS];
+    __shared__ double srhs[MAXNT * K3_CELLS][4], sinv[MAXNT * K3_CELLS];
+    __shared__ double sM[MAXNT][MAXNT][K3_CELLS];
     const int lb = blockIdx.x - B.off[cs];
-    const int c = lb * K3_THREADS + threadIdx.x;
-    const int nt = cd.nt, nc = cd.nc;
+    const int nt = cd.nt, nc = cd.nc, half = k3_half(nt);
+    const int role = (int)threadIdx.x / half;              // 0: W^k, 1: W^{k+1}, 2: helps with the tables only
+    const int r = (int)threadIdx.x - role * half;
+    const int n = r / K3_CELLS, ci = r % K3_CELLS, c = lb * K3_CELLS + ci;
+    const bool work = role < 2 && n < nt && c < nc;
     const int p = cd.st->parity;
-    double r2[4] = {0, 0, 0, 0};
-    if (c < nc) {
-        const int i = c % cd.nx, j = c / cd.nx;
-        const double* W = cd.W[p];
-        double* Wn = cd.W[p ^ 1];
-        const int fL = j * (cd.nx + 1) + i, fR = fL + 1, fB = cd.nfx + j * cd.nx + i, fT = fB + cd.nx;
-        const double dx = 2.0 * cd.hx[i], dy = 2.0 * cd.hy[j], area = dx * dy;
-        const double dG = cd.dG[c];
-        double Wc[MAXNT][4];
-        for (int n = 0; n < nt; ++n)
+    const bool implicit = cd.spectral_implicit != 0;
+    const double* W = cd.W[p];
+    double* Wn = cd.W[p ^ 1];
+    const double il0 = rcp64(cd.lam0);
+    const int i = work ? c % cd.nx : 0, j = work ? c / cd.nx : 0;
+    const double dx = 2.0 * cd.hx[i], dy = 2.0 * cd.hy[j], idx_ = rcp64(dx), idy = rcp64(dy);
+    const double dG = work ? cd.dG[c] : 0.0;
+    double rho = 1.0, U = 0.0, V = 0.0, lam = 1.0, tau = 1.0, qx = 0.0, qy = 0.0;
+    double Wc[4], wn[4];                                   // this thread's W^k, W^{k+1}
+    if (work) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) Wc[n][k] = W[((size_t)n * nc + c) * 4 + k];
-        const bool implicit = cd.spectral_implicit != 0;
-        double Wi[MAXNT][4];
-        if (implicit) {
-            // spectral source at the new iterate: (I + dG omega E) W^{k+1} = W^k - dG div F for every variable
-            double A[MAXNT][MAXNT];
-            spectral_matrix(cd, dG, nullptr, A);
-            for (int n = 0; n < nt; ++n) {
-                const double* FL = cd.fflux + ((size_t)fL * nt + n) * 4;
-                const double* FR = cd.fflux + ((size_t)fR * nt + n) * 4;
-                const double* FB = cd.fflux + ((size_t)fB * nt + n) * 4;
-                const double* FT = cd.fflux + ((size_t)fT * nt + n) * 4;
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    Wi[n][k] = Wc[n][k] - dG * (dy * (FR[k] - FL[k]) + dx * (FT[k] - FB[k])) / area;
-            }
-            solve_levels(nt, A, Wi);
-        }
-        double Dn[MAXNT];
-        for (int n = 0; n < nt; ++n) {
-            const double* FL = cd.fflux + ((size_t)fL * nt + n) * 4;
-            const double* FR = cd.fflux + ((size_t)fR * nt + n) * 4;
-            const double* FB = cd.fflux + ((size_t)fB * nt + n) * 4;
-            const double* FT = cd.fflux + ((size_t)fT * nt + n) * 4;
-            double wn[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (implicit) {
-                    wn[k] = Wi[n][k];
-                } else {
-                    double div = (dy * (FR[k] - FL[k]) + dx * (FT[k] - FB[k])) / area;
-                    double ew = 0.0;
-                    for (int d = 1; d <= cd.nh; ++d) {
-                        int nm = n - d; if (nm < 0) nm += nt;
-                        int np = n + d; if (np >= nt) np -= nt;
-                        ew += cd.e[d] * (Wc[nm][k] - Wc[np][k]);
-                    }
-                    wn[k] = Wc[n][k] - dG * (div + cd.omega * ew);
-                }
-                Wn[((size_t)n * nc + c) * 4 + k] = wn[k];
-            }
-            if (n == 0) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) { double d = wn[k] - Wc[0][k]; r2[k] = d * d; }
-            }
-            // collision coefficients of Eq. fv_h with h+ from W^k and W^{k+1} and the heat flux q^k
+        for (int k = 0; k < 4; ++k) Wc[k] = W[((size_t)n * nc + c) * 4 + k];
+        if (role == 0) {
             double A[13];
             const double* cm = cd.cmom + ((size_t)c * nt + n) * NCM;
 #pragma unroll
             for (int k = 0; k < 13; ++k) A[k] = cm[k] + cd.refmom[k];
-            double r0, U0, V0, l0, r1, U1, V1, l1, qx, qy;
-            prim(Wc[n], r0, U0, V0, l0);
-            prim(wn, r1, U1, V1, l1);
-            heat_flux_raw(A, U0, V0, qx, qy);
-            const double t0 = relax_time(cd.mu0, cd.w_vss, cd.lam0, r0, l0);
-            const double t1 = relax_time(cd.mu0, cd.w_vss, cd.lam0, r1, l1);
-            T* cp = cd.cpar + ((size_t)n * cd.nc + c) * NCP;
-            eq_cell(r0, U0, V0, l0, cd.lam0, cd.pr, qx, qy, cp + C_EQ0);
-            eq_cell(r1, U1, V1, l1, cd.lam0, cd.pr, qx, qy, cp + C_EQ1);
-            // explicit: the update of Eq. fv_h divided by D; implicit: its right-hand side, which the micro
-            // update then multiplies by minv across levels
-            const double D = 1.0 + 0.5 * dG / t1;
-            Dn[n] = D;
-            const double s_ = implicit ? 1.0 : D;
+            prim(Wc, rho, U, V, lam);
+            heat_flux_raw(A, U, V, qx, qy);
+            tau = relax_time(cd.mu0, cd.w_vss, il0, rcp64(rho), lam);
+            sq[r][0] = qx;
+            sq[r][1] = qy;
+        } else {
+            const int fL = j * (cd.nx + 1) + i, fB = cd.nfx + j * cd.nx + i;
+            const double* FL = cd.fflux + ((size_t)fL * nt + n) * 4;
+            const double* FR = FL + (size_t)nt * 4;
+            const double* FB = cd.fflux + ((size_t)fB * nt + n) * 4;
+            const double* FT = FB + (size_t)cd.nx * nt * 4;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double div = (FR[k] - FL[k]) * idx_ + (FT[k] - FB[k]) * idy;
+                if (implicit) {
+                    srhs[r][k] = Wc[k] - dG * div;
+                } else {
+                    double ew = 0.0;
+                    for (int d = 1; d <= cd.nh; ++d) {
+                        int nm = n - d; nm += nm < 0 ? nt : 0;
+                        int np = n + d; np -= np >= nt ? nt : 0;
+                        ew += cd.e[d] * (W[((size_t)nm * nc + c) * 4 + k] - W[((size_t)np * nc + c) * 4 + k]);
+                    }
+                    wn[k] = Wc[k] - dG * (div + cd.omega * ew);
+                }
+            }
+            if (implicit) {
+                // entry d = n of the inverse of the circulant I + a E, a = dG omega, whose eigenvalues are 1 + i a k:
+                // (1/N_T) [1 + 2 sum_k (cos(2 pi k d / N_T) + a k sin(2 pi k d / N_T)) / (1 + a^2 k^2)]
+                const double a = dG * cd.omega;
+                double s = 0.0;
+                for (int k = 1, m = n; k <= cd.nh; ++k, m += n) {
+                    if (m >= nt) m -= nt;
+                    const double ak = a * k;
+                    s += (cd.ct[m] + ak * cd.snt[m]) * rcp64(1.0 + ak * ak);
+                }
+                sinv[r] = (1.0 + 2.0 * s) / nt;
+            }
+        }
+    }
+    if (implicit) {
+        // spectral source at the new iterate: (I + dG omega E) W^{k+1} = W^k - dG div F for every variable
+        __syncthreads();
+        if (work && role == 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) wn[k] = 0.0;
+            for (int m = 0; m < nt; ++m) {
+                int d = n - m; d += d < 0 ? nt : 0;
+                const double g = sinv[d * K3_CELLS + ci];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) wn[k] += g * srhs[m * K3_CELLS + ci][k];
+            }
+        }
+    }
+    if (work && role == 1) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) Wn[((size_t)n * nc + c) * 4 + k] = wn[k];
+        prim(wn, rho, U, V, lam);
+        tau = relax_time(cd.mu0, cd.w_vss, il0, rcp64(rho), lam);
+        stau[r] = tau;
+        snu[r] = nu_conv(cd, U, V, lam, idx_, idy);        // for the next local step
+    }
+    if (role == 1 && r < 32) {
+        // level-0 residual partials of the CTA's cells (lanes 0..7 of the half's first warp)
+        double r2[4] = {0, 0, 0, 0};
+        if (work && n == 0)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) { const double d = wn[k] - Wc[k]; r2[k] = d * d; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+            for (int o = K3_CELLS / 2; o > 0; o >>= 1) r2[k] += __shfl_xor_sync(0xffffffffu, r2[k], o);
+        }
+        if (r == 0)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) cd.rpart[(size_t)lb * 4 + k] = r2[k];
+    }
+    __syncthreads();
+    if (work) {
+        T* cp = cd.cpar + ((size_t)n * nc + c) * NCP;
+        const int row = (ci * nt + n) * 2 + role;
+        coef[row][0] = T(cd.lam0 - lam);
+        coef[row][1] = T(2.0 * lam * U);
+        coef[row][2] = T(lam * U * U);
+        coef[row][3] = T(2.0 * lam * V);
+        coef[row][4] = T(lam * V * V);
+        if (role == 0) {
+            // collision coefficients of Eq. fv_h.  Explicit: the update divided by D; implicit: its right-hand side,
+            // which the micro update then multiplies by minv across levels
+            eq_cell(rho, U, V, lam, il0, cd.pr, qx, qy, cp + C_EQ0);
+            const double h0 = 0.5 * dG * rcp64(tau), h1 = 0.5 * dG * rcp64(stau[r]);
+            const double is = implicit ? 1.0 : rcp64(1.0 + h1);
             // kself, -kE, kp1, kp0, -kdx, -kdy, each stored twice (broadcast pairs for the (h, b) update)
-            const double kk[6] = {(1.0 - 0.5 * dG / t0) / s_, implicit ? 0.0 : -dG * cd.omega / D,
-                                  0.5 * dG / (t1 * s_), 0.5 * dG / (t0 * s_), -dG / (dx * s_), -dG / (dy * s_)};
+            const double kk[6] = {(1.0 - h0) * is, implicit ? 0.0 : -dG * cd.omega * is, h1 * is, h0 * is,
+                                  -dG * idx_ * is, -dG * idy * is};
 #pragma unroll
             for (int q = 0; q < 6; ++q) cp[C_K + 2 * q] = cp[C_K + 2 * q + 1] = T(kk[q]);
+        } else {
+            // h+ of W^{k+1} takes the heat flux q^k
+            eq_cell(rho, U, V, lam, il0, cd.pr, sq[r][0], sq[r][1], cp + C_EQ1);
+            if (n == 0) {
+                double numax = 0.0;
+                for (int m = 0; m < nt; ++m) numax = fmax(numax, snu[m * K3_CELLS + ci]);
+                cd.dG[c] = local_step(cd, numax);
+            }
         }
-        if (implicit) {
-            // inverse of diag(D_n) + dG omega E for the micro update of this cell (every velocity)
-            double A[MAXNT][MAXNT], X[MAXNT][MAXNT];
-            spectral_matrix(cd, dG, Dn, A);
-            for (int n = 0; n < nt; ++n)
-                for (int m = 0; m < nt; ++m) X[n][m] = n == m ? 1.0 : 0.0;
-            solve_levels(nt, A, X);
-            T* mo = cd.minv + (size_t)c * nt * nt;
-            for (int n = 0; n < nt; ++n)
-                for (int m = 0; m < nt; ++m) mo[n * nt + m] = T(X[n][m]);
-        }
-        cd.dG[c] = cd.dt_fixed > 0.0 ? cd.dt_fixed : local_step(cd, Wn, c, i, j);
     }
-    // deterministic block reduction of the level-0 residual partials
-    __shared__ double red[K3_THREADS][4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) red[threadIdx.x][k] = r2[k];
-    __syncthreads();
-    for (int s = K3_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) red[threadIdx.x][k] += red[threadIdx.x + s][k];
+    if (implicit) {
+        // inverse of diag(D_n) + dG omega E, D = 1 + dG/(2 tau^{k+1}), for the micro update of each cell (every
+        // velocity): Gauss-Jordan in place, a thread per row and cell and the two halves on alternate columns.  No
+        // pivoting is needed: E is skew-symmetric and D > 0, so the symmetric part is positive definite, and so is
+        // that of every Schur complement the elimination meets.
+        double D = 0.0;
+        if (work) {
+            D = 1.0 + 0.5 * dG * rcp64(stau[r]);
+            for (int m = role; m < nt; m += 2) {
+                int d = n - m; d += d < 0 ? nt : 0;        // E_{n, n-d} = e_d for d <= N_H, -e_{N_T - d} beyond
+                const double e = d == 0 ? 0.0 : d <= cd.nh ? cd.e[d] : -cd.e[nt - d];
+                sM[n][m][ci] = d == 0 ? D : dG * cd.omega * e;
+            }
+        }
         __syncthreads();
+        for (int k = 0; k < nt; ++k) {
+            double pv = 0.0, f = 0.0;
+            if (work) {
+                pv = rcp64(sM[k][k][ci]);
+                f = sM[n][k][ci] * pv;
+                if (n != k)
+                    for (int m = role; m < nt; m += 2)
+                        if (m != k) sM[n][m][ci] -= f * sM[k][m][ci];
+            }
+            __syncthreads();
+            if (work) {
+                if (n == k) {
+                    for (int m = role; m < nt; m += 2) sM[k][m][ci] = m == k ? pv : sM[k][m][ci] * pv;
+                } else if ((k & 1) == role) {
+                    sM[n][k][ci] = -f;
+                }
+            }
+            __syncthreads();
+        }
+        if (work) {
+            T* mo = cd.minv + (size_t)c * nt * nt + n * nt;
+            for (int m = role; m < nt; m += 2) mo[m] = T(sM[n][m][ci]);
+        }
     }
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) cd.rpart[lb * 4 + k] = red[0][k];
+    __syncthreads();
+    // tables of expm1(lam0 x^2 - lam (x - U)^2) over the 1-D velocity nodes, so that for a Maxwellian of density rho:
+    // H - H_ref = H_ref [(r - 1) + r (ex + ey + ex ey)], r = rho lam / lam0.  The CTA's rows are consecutive in memory.
+    const int nuv = cd.nu + cd.nv, rows = min(K3_CELLS, nc - lb * K3_CELLS) * nt * 2;
+    T* dst = cd.ctab + (size_t)lb * K3_CELLS * nt * 2 * nuv;
+    int row = (int)threadIdx.x / nuv, k = (int)threadIdx.x - row * nuv;
+    for (int q = threadIdx.x; row < rows; q += blockDim.x) {
+        const T* e = coef[row];
+        const bool isu = k < cd.nu;
+        const T x = isu ? cd.tu1[k] : cd.tv1[k - cd.nu];
+        dst[q] = t_expm1<T>(e[0] * x * x + (isu ? e[1] : e[3]) * x - (isu ? e[2] : e[4]));
+        k += blockDim.x;
+        while (k >= nuv) { k -= nuv; ++row; }
+    }
 }
 
 // ------------------------------------------------------------------------------ K5 residual / status
 
+constexpr int K5_THREADS = 128;
+
 template <typename T>
-__global__ void k5_finish(const CaseDev<T>* cases, int ncases, const int* k3off)
+__global__ void __launch_bounds__(K5_THREADS) k5_finish(const CaseDev<T>* cases, int ncases, const int* k3off)
 {
     int cs = blockIdx.x;
     if (cs >= ncases) return;
@@ -675,34 +677,35 @@ __global__ void k5_finish(const CaseDev<T>* cases, int ncases, const int* k3off)
     CaseStatus* st = cd.st;
     if (!st->active || *(volatile int*)cd.err) return;   // a failed wait leaves the iteration unfinished
     const int nb = k3off[cs + 1] - k3off[cs];
-    __shared__ double part[4][32];
-    const int lane = threadIdx.x;      // 32 threads
-    double s[4] = {0, 0, 0, 0};
-    for (int b = lane; b < nb; b += 32)
+    // thread t sums variable t & 3 of every 32nd partial; then a fixed tree over lanes and warps
+    __shared__ double part[K5_THREADS / 32][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double s = 0.0;
+    for (int b = threadIdx.x >> 2; b < nb; b += K5_THREADS / 4) s += cd.rpart[(size_t)b * 4 + (lane & 3)];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) s[k] += cd.rpart[b * 4 + k];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) part[k][lane] = s[k];
-    __syncwarp();
-    if (lane == 0) {
-        double R[4];
-        bool bad = false;
-        for (int k = 0; k < 4; ++k) {
-            double t = 0.0;
-            for (int l = 0; l < 32; ++l) t += part[k][l];
-            R[k] = sqrt(t / cd.nc);
-            if (!(R[k] <= 1e10)) bad = true;   // also catches NaN
-            st->last[k] = R[k];
-            cd.rhist[(st->iters % RING) * 4 + k] = R[k];
+    for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < 4) part[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+        // lanes 0..3: one variable each
+        const int k = lane & 3;
+        const double R = sqrt((part[0][k] + part[1][k] + part[2][k] + part[3][k]) / cd.nc);
+        const bool bad = __any_sync(0xffffffffu, !(R <= 1e10));   // also catches NaN
+        if (lane < 4) {
+            st->last[k] = R;
+            cd.rhist[(st->iters % RING) * 4 + k] = R;
         }
-        st->iters += 1;
-        st->iters_call += 1;
-        st->parity ^= 1;
-        if (bad) {
-            st->diverged = 1;
-            st->active = 0;
-        } else if (*cd.tol > 0.0 && st->iters >= 10 && R[0] <= *cd.tol) {
-            st->active = 0;
+        __syncwarp();
+        if (lane == 0) {
+            st->iters += 1;
+            st->iters_call += 1;
+            st->parity ^= 1;
+            if (bad) {
+                st->diverged = 1;
+                st->active = 0;
+            } else if (*cd.tol > 0.0 && st->iters >= 10 && R <= *cd.tol) {
+                st->active = 0;
+            }
         }
     }
 }
