@@ -22,28 +22,33 @@
 namespace hb {
 
 // van Leer limiter of a pair: 2 s1 s2 / (s1 + s2) where s1 s2 > 0, else 0.  Single precision: the limited slope
-// needs no correctly rounded division (approximate reciprocal, 2 ulp)
+// needs no correctly rounded division (approximate reciprocal, 2 ulp); double precision: rcp64
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// The arguments are twice the one-sided slopes, so that the limited slope 2 s1 s2 / (s1 + s2) is their product over
+// their sum.
 __device__ __forceinline__ float2 vleer2(float2 s1, float2 s2)
 {
     const float2 p = pmul(s1, s2);
     const float2 den = padd(s1, s2);
-    const float2 q = pmul(padd(p, p), make_float2(rcp_approx(den.x), rcp_approx(den.y)));
+    const float2 q = pmul(p, make_float2(rcp_approx(den.x), rcp_approx(den.y)));
     return make_float2(p.x > 0.f ? q.x : 0.f, p.y > 0.f ? q.y : 0.f);
 }
+// x > 0 from the high word, off the FP64 pipe (false for NaN; a positive denormal below 2^-1042 counts as zero)
+__device__ __forceinline__ bool pos64(double x) { return (unsigned)(__double2hiint(x) - 1) < 0x7ff00000u; }
 __device__ __forceinline__ double2 vleer2(double2 s1, double2 s2)
 {
     const double px = s1.x * s2.x, py = s1.y * s2.y;
-    return make_double2(px > 0.0 ? (px + px) / (s1.x + s2.x) : 0.0, py > 0.0 ? (py + py) / (s1.y + s2.y) : 0.0);
+    const double qx = px * rcp64(s1.x + s2.x), qy = py * rcp64(s1.y + s2.y);
+    return make_double2(pos64(px) ? qx : 0.0, pos64(py) ? qy : 0.0);
 }
 
-// Limited slope of (h, b) of a cell from its two neighbours along one axis, wm = 1/(x_i - x_{i-1}),
-// wp = 1/(x_{i+1} - x_i) (non-uniform spacing); a missing neighbour (wall) makes the available one-sided
+// Limited slope of (h, b) of a cell from its two neighbours along one axis, wm = 2/(x_i - x_{i-1}),
+// wp = 2/(x_{i+1} - x_i) (non-uniform spacing); a missing neighbour (wall) makes the available one-sided
 // difference the slope, a single cell along the axis has none
 template <typename V, typename T>
 __device__ __forceinline__ V slope2(V fm, V f0, V fp, T wm, T wp, bool has_m, bool has_p, bool several)
@@ -139,10 +144,20 @@ __device__ __forceinline__ T lane_totals(T (&v)[N], int lane)
 // A wall face takes 0..12 and 18..22 from the velocities moving into the wall only and 13..17 from all.
 // Half-face slots per (cell, level): 0 x-face of the u > 0 class (the right face), 1 u < 0 (left face),
 // 2 v > 0 (top face), 3 v < 0 (bottom face).
+// Every one of these sums is linear in f0, the slope s_x and the slope s_y of the cell (d0 = f0 +- h_x s_x at the
+// x-face, f0 +- h_y s_y at the y-face; u_n s_n + u_t s_t = u s_x + v s_y at both), with factors that are the same for
+// the whole sign class.  So a lane keeps moments of f0, s_x and s_y only and the face sums are formed from them when
+// the class changes: 47 sums per velocity instead of 59 and no reconstruction (the b sums need the weights 1, u, v of
+// f0; 1, u, v, u^2, uv of s_x; 1, u, v, uv, v^2 of s_y).
 // With SEP the case's velocity grid has no zero node and each sign class has 1, 2, 4, 8, 16 or 32 u-nodes, so a
 // lane sees the same u in every block of a class (blocks hold whole rows of the class, u fastest): every sum
 // w u^a v^b d factors into w_u u^a (the lane's) times sum over the lane's velocities of w_v v^b d, and the lane
-// keeps only those v-moments (34 sums instead of 59), multiplying by w_u u^a when the class changes.
+// keeps only those v-moments (20 sums: of f0 v^0..3 for h and v^0..1 for b, of s_x the same, of s_y v^0..4 and
+// v^0..2), multiplying by w_u u^a when the class changes.
+// Bound by FP64 instructions in FP64 (67 per velocity with SEP, the limiter's reciprocals included) and by
+// instruction issue in FP32.  Against 59 sums with the reconstruction formed per velocity and divisions in the
+// limiter: 36.98 -> 23.19 ms (twelve 64x64 cavities, 32x32 velocities, N_T 3, FP64, SEP), 18.22 -> 12.81 ms (64x64,
+// 48x48, N_T 7, FP64), 4.83 -> 4.19 ms (128x128, 64x64, N_T 11, FP32, SEP), 0.543 -> 0.518 ms (64x64, 48x48, FP32).
 template <typename T, int TX, int TY, int G, int S, bool SEP>
 __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8) ? 2 : 1) k1_cells(Batch<T> B)
 {
@@ -210,8 +225,8 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
 
     // the warp's cell: neighbours, spacings, half widths (uniform over the warp)
     const bool hm = i > 0, hp = i < nx - 1, vm = j > 0, vp = j < ny - 1, sx = nx > 1, sy = ny > 1;
-    const T wxm = valid && hm ? T(cd.rdx[i - 1]) : T(0), wxp = valid && hp ? T(cd.rdx[i]) : T(0);
-    const T wym = valid && vm ? T(cd.rdy[j - 1]) : T(0), wyp = valid && vp ? T(cd.rdy[j]) : T(0);
+    const T wxm = valid && hm ? T(2) * T(cd.rdx[i - 1]) : T(0), wxp = valid && hp ? T(2) * T(cd.rdx[i]) : T(0);
+    const T wym = valid && vm ? T(2) * T(cd.rdy[j - 1]) : T(0), wyp = valid && vp ? T(2) * T(cd.rdy[j]) : T(0);
     const T hxh = valid ? T(cd.hx[i]) : T(0), hyh = valid ? T(cd.hy[j]) : T(0);
     const bool inner = hm && hp && vm && vp;                 // every neighbour present: no wall branches
     const int kc = (tj + 1) * PX + ti + 1;
@@ -219,90 +234,110 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
     const T* __restrict__ tv = cd.tv;
     const T* __restrict__ tw = SEP ? cd.twv : cd.tw;       // SEP: the v-factor w_v of each weight
 
-    // general: the 23 + 23 + 13 sums per lane; SEP: v-moments per lane (x-face h: 4, b: 2, tangential h: 3,
-    // b: 1, normal-flux h: 3, b: 1; the y-face alike; cell h: 4, b: 2), folded into the 23 + 23 + 13 at a
-    // class change.  A sum of h and the sum of b with the same weight are kept as one pair (one packed FMA):
-    //   SEP      xp: (0, 4) (1, 5) (6, 9) (10, 13) of the 14 v-moments, xs: 2 3 7 8 11 12;  cp: (0, 4) (1, 5),
-    //            csm: 2 3 of the 6 cell v-moments
-    //   general  xp: (0, 10) (1, 11) (2, 12) (13, 17) (18, 22) of the 23 sums, xs: 3..9, 14..16, 19..21;
-    //            cp: (0, 10) (1, 11) (2, 12), csm: 3..9 of the 13 cell sums
-    constexpr int NXP = SEP ? 4 : 5, NXS = SEP ? 6 : 13, NCP2 = SEP ? 2 : 3, NCS = SEP ? 2 : 7;
-    V xp[NXP], yp[NXP], cp2[NCP2];
-    T xs[NXS], ys[NXS], csm[NCS], ac[NCM];
-    auto zero_faces = [&]() {
+    // A sum of h and the sum of b with the same weight are kept as one pair (one packed FMA), the others of h alone:
+    //   SEP      f: pairs v^0 v^1, h v^2 v^3;  x: the same;  y: pairs v^0 v^1 v^2, h v^3 v^4
+    //   general  f: pairs 1 u v, h uu uv vv uuu uuv uvv vvv;  x: pairs 1 u v uu uv, h vv uuu uuv uvv vvv uu|u|^2 uv|u|^2;
+    //            y: pairs 1 u v uv vv, h uu uuu uuv uvv vvv vv|u|^2 uv|u|^2;  and in wall cells the part of f0 +- h s
+    //            of nodes parallel to the wall, which the wall face leaves out: zx pairs 1 v, h vv vvv; zy pairs 1 u,
+    //            h uu uuu
+    constexpr int NFP = SEP ? 2 : 3, NFS = SEP ? 2 : 7, NXP = SEP ? 2 : 5, NXS = SEP ? 2 : 7, NYP = SEP ? 3 : 5,
+                  NYS = SEP ? 2 : 7, NZ = SEP ? 0 : 1;
+    V fp_[NFP], xp[NXP], yp[NYP], zxp[2 * NZ + 1], zyp[2 * NZ + 1];
+    T fs_[NFS], xs[NXS], ys[NYS], zxs[2 * NZ + 1], zys[2 * NZ + 1], ac[NCM];
+    auto zero_sums = [&]() {
 #pragma unroll
-        for (int q = 0; q < NXP; ++q) { xp[q] = bc(T(0)); yp[q] = bc(T(0)); }
+        for (int q = 0; q < NFP; ++q) fp_[q] = bc(T(0));
 #pragma unroll
-        for (int q = 0; q < NXS; ++q) { xs[q] = T(0); ys[q] = T(0); }
+        for (int q = 0; q < NFS; ++q) fs_[q] = T(0);
+#pragma unroll
+        for (int q = 0; q < NXP; ++q) xp[q] = bc(T(0));
+#pragma unroll
+        for (int q = 0; q < NXS; ++q) xs[q] = T(0);
+#pragma unroll
+        for (int q = 0; q < NYP; ++q) yp[q] = bc(T(0));
+#pragma unroll
+        for (int q = 0; q < NYS; ++q) ys[q] = T(0);
+#pragma unroll
+        for (int q = 0; q < 2 * NZ; ++q) { zxp[q] = bc(T(0)); zyp[q] = bc(T(0)); zxs[q] = T(0); zys[q] = T(0); }
     };
-    auto zero_cell = [&]() {
-#pragma unroll
-        for (int q = 0; q < NCP2; ++q) cp2[q] = bc(T(0));
-#pragma unroll
-        for (int q = 0; q < NCS; ++q) csm[q] = T(0);
-    };
-    zero_faces();
-    zero_cell();
+    zero_sums();
 #pragma unroll
     for (int q = 0; q < NCM; ++q) ac[q] = T(0);
     int cur = -1, cend = 0;                                  // current sign class, the first block past it
     T ul = T(0), wul = T(0);                                 // SEP: the lane's u and w_u in the current class
-    // the 14 v-moments of a face (SEP) or its 23 sums (general) in slot order
-    auto face_sums = [&](const V (&P)[NXP], const T (&S_)[NXS], T (&m)[SEP ? 14 : NM]) {
-        if constexpr (SEP) {
-            m[0] = P[0].x; m[1] = P[1].x; m[2] = S_[0]; m[3] = S_[1]; m[4] = P[0].y; m[5] = P[1].y;
-            m[6] = P[2].x; m[7] = S_[2]; m[8] = S_[3]; m[9] = P[2].y; m[10] = P[3].x; m[11] = S_[4];
-            m[12] = S_[5]; m[13] = P[3].y;
-        } else {
-            m[0] = P[0].x; m[1] = P[1].x; m[2] = P[2].x;
-#pragma unroll
-            for (int q = 0; q < 7; ++q) m[3 + q] = S_[q];
-            m[10] = P[0].y; m[11] = P[1].y; m[12] = P[2].y; m[13] = P[3].x;
-            m[14] = S_[7]; m[15] = S_[8]; m[16] = S_[9]; m[17] = P[3].y; m[18] = P[4].x;
-            m[19] = S_[10]; m[20] = S_[11]; m[21] = S_[12]; m[22] = P[4].y;
-        }
-    };
-    // the 23 face sums of one face from its v-moments m (SEP)
-    auto unfold = [&](const T (&m)[14], T (&o)[NM]) {
+    // the 23 face sums of one face from its v-moments (SEP): D, DB of d0 and e0, S, SB tangential slopes, N, NB normal
+    auto unfold = [&](const T (&D)[4], const T (&DB)[2], const T (&S_)[3], T SB, const T (&N)[3], T NB, T (&o)[NM]) {
         const T w1 = wul, w2 = w1 * ul, w3 = w2 * ul, w4 = w3 * ul;     // w_u u^a
-        o[0] = w1 * m[0]; o[1] = w2 * m[0]; o[2] = w1 * m[1]; o[3] = w3 * m[0]; o[4] = w2 * m[1];
-        o[5] = w1 * m[2]; o[6] = w4 * m[0]; o[7] = w3 * m[1]; o[8] = w2 * m[2]; o[9] = w1 * m[3];
-        o[10] = w1 * m[4]; o[11] = w2 * m[4]; o[12] = w1 * m[5];
-        o[13] = w1 * m[6]; o[14] = w2 * m[6]; o[15] = w1 * m[7]; o[16] = w3 * m[6] + w1 * m[8];
-        o[17] = w1 * m[9];
-        o[18] = w1 * m[10]; o[19] = w2 * m[10]; o[20] = w1 * m[11]; o[21] = w3 * m[10] + w1 * m[12];
-        o[22] = w1 * m[13];
+        o[0] = w1 * D[0]; o[1] = w2 * D[0]; o[2] = w1 * D[1]; o[3] = w3 * D[0]; o[4] = w2 * D[1];
+        o[5] = w1 * D[2]; o[6] = w4 * D[0]; o[7] = w3 * D[1]; o[8] = w2 * D[2]; o[9] = w1 * D[3];
+        o[10] = w1 * DB[0]; o[11] = w2 * DB[0]; o[12] = w1 * DB[1];
+        o[13] = w1 * S_[0]; o[14] = w2 * S_[0]; o[15] = w1 * S_[1]; o[16] = w3 * S_[0] + w1 * S_[2];
+        o[17] = w1 * SB;
+        o[18] = w1 * N[0]; o[19] = w2 * N[0]; o[20] = w1 * N[1]; o[21] = w3 * N[0] + w1 * N[2];
+        o[22] = w1 * NB;
     };
-    // add the sums of the current sign class to its two half-face slots
+    // add the sums of the current sign class to its two half-face slots and to the cell's moments
     auto flush = [&]() {
-        T tx_, ty_;
+        const T sx_ = (cur & 1) ? -hxh : hxh, sy_ = (cur & 2) ? -hyh : hyh;
+        T ox[NM], oy[NM];
         if constexpr (SEP) {
-            T mx[14], my[14], ox[NM], oy[NM];
-            face_sums(xp, xs, mx);
-            face_sums(yp, ys, my);
-            unfold(mx, ox);
-            unfold(my, oy);
-            const T c0 = cp2[0].x, c1 = cp2[1].x, c2 = csm[0], c3 = csm[1], c4 = cp2[0].y, c5 = cp2[1].y;
+            const T F[4] = {fp_[0].x, fp_[1].x, fs_[0], fs_[1]}, FB[2] = {fp_[0].y, fp_[1].y};
+            const T X[4] = {xp[0].x, xp[1].x, xs[0], xs[1]}, XB[2] = {xp[0].y, xp[1].y};
+            const T Y[5] = {yp[0].x, yp[1].x, yp[2].x, ys[0], ys[1]}, YB[3] = {yp[0].y, yp[1].y, yp[2].y};
+            T D[4], DB[2], S_[3], N[3];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) D[q] = F[q] + sx_ * X[q];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) DB[q] = FB[q] + sx_ * XB[q];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) { S_[q] = Y[q]; N[q] = ul * (ul * X[q] + Y[q + 1]); }
+            unfold(D, DB, S_, YB[0], N, ul * (ul * XB[0] + YB[1]), ox);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) D[q] = F[q] + sy_ * Y[q];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) DB[q] = FB[q] + sy_ * YB[q];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) { S_[q] = X[q]; N[q] = ul * X[q + 1] + Y[q + 2]; }
+            unfold(D, DB, S_, XB[0], N, ul * XB[1] + YB[2], oy);
             const T w1 = wul, w2 = w1 * ul, w3 = w2 * ul, w4 = w3 * ul;
-            ac[0] += w1 * c0; ac[1] += w2 * c0; ac[2] += w1 * c1; ac[3] += w3 * c0;
-            ac[4] += w2 * c1; ac[5] += w1 * c2; ac[6] += w4 * c0; ac[7] += w3 * c1;
-            ac[8] += w2 * c2; ac[9] += w1 * c3;
-            ac[10] += w1 * c4; ac[11] += w2 * c4; ac[12] += w1 * c5;
-            zero_cell();
-            tx_ = lane_totals<NM>(ox, lane);
-            ty_ = lane_totals<NM>(oy, lane);
+            ac[0] += w1 * F[0]; ac[1] += w2 * F[0]; ac[2] += w1 * F[1]; ac[3] += w3 * F[0];
+            ac[4] += w2 * F[1]; ac[5] += w1 * F[2]; ac[6] += w4 * F[0]; ac[7] += w3 * F[1];
+            ac[8] += w2 * F[2]; ac[9] += w1 * F[3];
+            ac[10] += w1 * FB[0]; ac[11] += w2 * FB[0]; ac[12] += w1 * FB[1];
         } else {
-            T ox[NM], oy[NM];
-            face_sums(xp, xs, ox);
-            face_sums(yp, ys, oy);
-            tx_ = lane_totals<NM>(ox, lane);
-            ty_ = lane_totals<NM>(oy, lane);
+            // monomials 1, u, v, uu, uv, vv, uuu, uuv, uvv, vvv
+            const T F[10] = {fp_[0].x, fp_[1].x, fp_[2].x, fs_[0], fs_[1], fs_[2], fs_[3], fs_[4], fs_[5], fs_[6]};
+            const T X[10] = {xp[0].x, xp[1].x, xp[2].x, xp[3].x, xp[4].x, xs[0], xs[1], xs[2], xs[3], xs[4]};
+            const T Y[10] = {yp[0].x, yp[1].x, yp[2].x, ys[0], yp[3].x, yp[4].x, ys[1], ys[2], ys[3], ys[4]};
+#pragma unroll
+            for (int q = 0; q < 10; ++q) {
+                ox[q] = F[q] + sx_ * X[q];
+                oy[q] = F[q] + sy_ * Y[q];
+                ac[q] += F[q];
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                ox[10 + q] = fp_[q].y + sx_ * xp[q].y;
+                oy[10 + q] = fp_[q].y + sy_ * yp[q].y;
+                ac[10 + q] += fp_[q].y;
+                ox[13 + q] = Y[q];
+                oy[13 + q] = X[q];
+            }
+            ox[16] = Y[3] + Y[5]; ox[17] = yp[0].y;
+            oy[16] = X[3] + X[5]; oy[17] = xp[0].y;
+            ox[18] = X[3] + Y[4]; ox[19] = X[6] + Y[7]; ox[20] = X[7] + Y[8]; ox[21] = xs[5] + ys[6];
+            ox[22] = xp[3].y + yp[3].y;
+            oy[18] = X[4] + Y[5]; oy[19] = X[7] + Y[8]; oy[20] = X[8] + Y[9]; oy[21] = xs[6] + ys[5];
+            oy[22] = xp[4].y + yp[4].y;
+            ox[0] -= zxp[0].x; ox[2] -= zxp[1].x; ox[5] -= zxs[0]; ox[9] -= zxs[1]; ox[10] -= zxp[0].y; ox[12] -= zxp[1].y;
+            oy[0] -= zyp[0].x; oy[1] -= zyp[1].x; oy[3] -= zys[0]; oy[6] -= zys[1]; oy[10] -= zyp[0].y; oy[11] -= zyp[1].y;
         }
+        const T tx_ = lane_totals<NM>(ox, lane), ty_ = lane_totals<NM>(oy, lane);
         if (lane < NM) {
             sacc[warp][(cur & 1) ? 1 : 0][lane] += tx_;
             sacc[warp][(cur & 2) ? 3 : 2][lane] += ty_;
         }
-        zero_faces();
+        zero_sums();
     };
 
     // Ring of S slots: chunk k lands in slot k % S (mbarrier bars); each warp arrives on empty once it has
@@ -328,12 +363,16 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
         auto run_blocks = [&](auto inner_tag) {
             constexpr bool INNER = decltype(inner_tag)::value;
             // the velocities of block g + 1 are loaded while block g is summed
-            T nu_ = __ldg(tu + vb0 * VB + lane), nv_ = __ldg(tv + vb0 * VB + lane), nw_ = __ldg(tw + vb0 * VB + lane);
+            // (SEP reads u only where the class changes)
+            T nu_ = SEP ? T(0) : __ldg(tu + vb0 * VB + lane), nv_ = __ldg(tv + vb0 * VB + lane),
+              nw_ = __ldg(tw + vb0 * VB + lane);
             for (int g = 0; g < gk; ++g) {
-                const T u = nu_, v = nv_, w = nw_;
+                [[maybe_unused]] const T u = nu_;
+                const T v = nv_, w = nw_;
                 if (g + 1 < gk) {
                     const int a1 = (vb0 + g + 1) * VB + lane;
-                    nu_ = __ldg(tu + a1); nv_ = __ldg(tv + a1); nw_ = __ldg(tw + a1);
+                    if (!SEP) nu_ = __ldg(tu + a1);
+                    nv_ = __ldg(tv + a1); nw_ = __ldg(tw + a1);
                 }
                 // the classes occupy consecutive blocks: a new one starts where the current one ends
                 if (vb0 + g >= cend) {
@@ -343,11 +382,10 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
                         cend = cd.cls_end[cur];
                     } while (vb0 + g >= cend);
                     if (SEP) {
-                        ul = u;
+                        ul = __ldg(tu + (vb0 + g) * VB + lane);
                         wul = __ldg(cd.twu + (vb0 + g) * VB + lane);
                     }
                 }
-                const int cls = cur;
                 const V* ph = cb + (size_t)g * blk + (size_t)kc * VB + lane;
                 const V f0 = ph[0];
                 V sxv, syv;
@@ -358,55 +396,45 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
                     sxv = slope2(ph[-VB], f0, ph[VB], wxm, wxp, hm, hp, sx);
                     syv = slope2(ph[-PX * VB], f0, ph[PX * VB], wym, wyp, vm, vp, sy);
                 }
-                const bool xn = (cls & 1) != 0, yn = (cls & 2) != 0;
-                V dx = pfma(sxv, bc(xn ? -hxh : hxh), f0);       // reconstruction at the downwind x-face
-                V dy = pfma(syv, bc(yn ? -hyh : hyh), f0);
-                if constexpr (!INNER) {
-                    // a velocity parallel to a wall carries nothing into it
-                    if ((xn ? !hm : !hp) && u == T(0)) dx = bc(T(0));
-                    if ((yn ? !vm : !vp) && v == T(0)) dy = bc(T(0));
-                }
-                const T sxh = sxv.x, syh = syv.x;
+                const T c1 = w * v, c2 = c1 * v, c3 = c2 * v;
                 if constexpr (SEP) {
                     // w is w_v here; v-moments of every summand
-                    const T c1 = w * v, c2 = c1 * v, c3 = c2 * v;
                     const V bw = bc(w), bc1 = bc(c1);
-                    const V tx = pmul(bc(ul), pfma(bc(ul), sxv, pmul(bc(v), syv)));   // u_n (u_n s_n + u_t s_t)
-                    const V ty = pmul(bc(v), pfma(bc(v), syv, pmul(bc(ul), sxv)));
-                    xp[0] = pfma(dx, bw, xp[0]); xp[1] = pfma(dx, bc1, xp[1]);
-                    xs[0] += dx.x * c2; xs[1] += dx.x * c3;
-                    yp[0] = pfma(dy, bw, yp[0]); yp[1] = pfma(dy, bc1, yp[1]);
-                    ys[0] += dy.x * c2; ys[1] += dy.x * c3;
-                    xp[2] = pfma(syv, bw, xp[2]); xs[2] += syh * c1; xs[3] += syh * c2;
-                    yp[2] = pfma(sxv, bw, yp[2]); ys[2] += sxh * c1; ys[3] += sxh * c2;
-                    xp[3] = pfma(tx, bw, xp[3]); xs[4] += tx.x * c1; xs[5] += tx.x * c2;
-                    yp[3] = pfma(ty, bw, yp[3]); ys[4] += ty.x * c1; ys[5] += ty.x * c2;
-                    cp2[0] = pfma(f0, bw, cp2[0]); cp2[1] = pfma(f0, bc1, cp2[1]);
-                    csm[0] += f0.x * c2; csm[1] += f0.x * c3;
-                    continue;
-                }
-                if constexpr (!SEP) {
-                    const T wu = w * u, wv = w * v, wuu = wu * u, wuv = wu * v, wvv = wv * v;
-                    const T m[10] = {w, wu, wv, wuu, wuv, wvv, wuu * u, wuu * v, wvv * u, wvv * v};
-                    const T wq = wuu + wvv;
-                    const V tx = pmul(bc(u), pfma(bc(u), sxv, pmul(bc(v), syv)));
-                    const V ty = pmul(bc(v), pfma(bc(v), syv, pmul(bc(u), sxv)));
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        xp[q] = pfma(dx, bc(m[q]), xp[q]);
-                        yp[q] = pfma(dy, bc(m[q]), yp[q]);
-                        cp2[q] = pfma(f0, bc(m[q]), cp2[q]);
+                    fp_[0] = pfma(f0, bw, fp_[0]); fp_[1] = pfma(f0, bc1, fp_[1]);
+                    xp[0] = pfma(sxv, bw, xp[0]); xp[1] = pfma(sxv, bc1, xp[1]);
+                    yp[0] = pfma(syv, bw, yp[0]); yp[1] = pfma(syv, bc1, yp[1]); yp[2] = pfma(syv, bc(c2), yp[2]);
+                    fs_[0] += f0.x * c2; fs_[1] += f0.x * c3;
+                    xs[0] += sxv.x * c2; xs[1] += sxv.x * c3;
+                    ys[0] += syv.x * c3; ys[1] += syv.x * (c3 * v);
+                } else {
+                    const T wu = w * u, wuu = wu * u, wuv = wu * v, wuuu = wuu * u, wuuv = wuu * v, wuvv = wuv * v;
+                    const T r2 = u * u + v * v;
+                    const V bw = bc(w), bu = bc(wu), bv = bc(c1), buv = bc(wuv);
+                    fp_[0] = pfma(f0, bw, fp_[0]); fp_[1] = pfma(f0, bu, fp_[1]); fp_[2] = pfma(f0, bv, fp_[2]);
+                    xp[0] = pfma(sxv, bw, xp[0]); xp[1] = pfma(sxv, bu, xp[1]); xp[2] = pfma(sxv, bv, xp[2]);
+                    xp[3] = pfma(sxv, bc(wuu), xp[3]); xp[4] = pfma(sxv, buv, xp[4]);
+                    yp[0] = pfma(syv, bw, yp[0]); yp[1] = pfma(syv, bu, yp[1]); yp[2] = pfma(syv, bv, yp[2]);
+                    yp[3] = pfma(syv, buv, yp[3]); yp[4] = pfma(syv, bc(c2), yp[4]);
+                    fs_[0] += f0.x * wuu; fs_[1] += f0.x * wuv; fs_[2] += f0.x * c2; fs_[3] += f0.x * wuuu;
+                    fs_[4] += f0.x * wuuv; fs_[5] += f0.x * wuvv; fs_[6] += f0.x * c3;
+                    xs[0] += sxv.x * c2; xs[1] += sxv.x * wuuu; xs[2] += sxv.x * wuuv; xs[3] += sxv.x * wuvv;
+                    xs[4] += sxv.x * c3; xs[5] += sxv.x * (wuu * r2); xs[6] += sxv.x * (wuv * r2);
+                    ys[0] += syv.x * wuu; ys[1] += syv.x * wuuu; ys[2] += syv.x * wuuv; ys[3] += syv.x * wuvv;
+                    ys[4] += syv.x * c3; ys[5] += syv.x * (c2 * r2); ys[6] += syv.x * (wuv * r2);
+                    if constexpr (!INNER) {
+                        // a velocity parallel to a wall carries nothing into it
+                        const bool xn = (cur & 1) != 0, yn = (cur & 2) != 0;
+                        if ((xn ? !hm : !hp) && u == T(0)) {
+                            const V d = pfma(sxv, bc(xn ? -hxh : hxh), f0);
+                            zxp[0] = pfma(d, bw, zxp[0]); zxp[1] = pfma(d, bv, zxp[1]);
+                            zxs[0] += d.x * c2; zxs[1] += d.x * c3;
+                        }
+                        if ((yn ? !vm : !vp) && v == T(0)) {
+                            const V d = pfma(syv, bc(yn ? -hyh : hyh), f0);
+                            zyp[0] = pfma(d, bw, zyp[0]); zyp[1] = pfma(d, bu, zyp[1]);
+                            zys[0] += d.x * wuu; zys[1] += d.x * wuuu;
+                        }
                     }
-#pragma unroll
-                    for (int q = 3; q < 10; ++q) {
-                        xs[q - 3] += dx.x * m[q];
-                        ys[q - 3] += dy.x * m[q];
-                        csm[q - 3] += f0.x * m[q];
-                    }
-                    xp[3] = pfma(syv, bc(w), xp[3]); xs[7] += syh * wu; xs[8] += syh * wv; xs[9] += syh * wq;
-                    yp[3] = pfma(sxv, bc(w), yp[3]); ys[7] += sxh * wu; ys[8] += sxh * wv; ys[9] += sxh * wq;
-                    xp[4] = pfma(tx, bc(w), xp[4]); xs[10] += tx.x * wu; xs[11] += tx.x * wv; xs[12] += tx.x * wq;
-                    yp[4] = pfma(ty, bc(w), yp[4]); ys[10] += ty.x * wu; ys[11] += ty.x * wv; ys[12] += ty.x * wq;
                 }
             }
         };
@@ -419,12 +447,6 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
     }
     if (!valid) return;
     if (cur >= 0) flush();
-    if constexpr (!SEP) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q) { ac[q] = cp2[q].x; ac[10 + q] = cp2[q].y; }
-#pragma unroll
-        for (int q = 0; q < 7; ++q) ac[3 + q] = csm[q];
-    }
     const T cm = lane_totals<NCM>(ac, lane);
     __syncwarp();
     const int c = j * nx + i;
@@ -706,12 +728,12 @@ __global__ void __launch_bounds__(NW * 32) k4_cells(Batch<T> B)
     };
     for (int k = threadIdx.x; k < PX; k += blockDim.x) {
         const int ii = i0 + xlo + k;
-        gxr[k] = (ii >= 0 && ii < nx - 1) ? T(cd.rdx[ii]) : T(0);
+        gxr[k] = (ii >= 0 && ii < nx - 1) ? T(2) * T(cd.rdx[ii]) : T(0);
         gxh[k] = (ii >= 0 && ii < nx) ? T(cd.hx[ii]) : T(0);
     }
     for (int k = threadIdx.x; k < PY; k += blockDim.x) {
         const int jj = j0 + ylo + k;
-        gyr[k] = (jj >= 0 && jj < ny - 1) ? T(cd.rdy[jj]) : T(0);
+        gyr[k] = (jj >= 0 && jj < ny - 1) ? T(2) * T(cd.rdy[jj]) : T(0);
         gyh[k] = (jj >= 0 && jj < ny) ? T(cd.hy[jj]) : T(0);
     }
     // the lane's velocity in each of the CTA's blocks
