@@ -17,6 +17,7 @@
 #include "hbugks.h"
 #include "hb_kernels.cuh"
 #include "hb_cells.cuh"
+#include "hb_micro.cuh"
 
 using namespace hb;
 
@@ -95,10 +96,11 @@ struct HostCase {
     // node's weight (1/2 or 1/4 for a node with u = 0 or v = 0, stored in two or four classes)
     std::vector<int> vcan, vcls;
     std::vector<double> vfac;
-    int k1b, k2b, k3b, k4b, ksb;
+    int k1b, k2b, k3b, ksb;
     int k4shape;
     int k1sep;                      // face sums by v-moments: no zero node, every sign class 1..32 u-nodes wide
     int pairs;                      // every sign class holds an even number of velocity blocks
+    int ng[2];                      // groups of one or two velocity blocks of one sign class
 };
 
 // K1 tile (TX x TY cells, one warp each) and velocity blocks staged per pass, per storage precision
@@ -118,46 +120,64 @@ constexpr auto k1_kernel()
     return k1_cells<T, K1_TX<T>, K1_TY<T>, K1_G<T>, K1_S<T>, SEP>;
 }
 
-// K4 tile shapes (TX, TY, warps per CTA)
-// K4 variants: tile (TX, TY), warps per CTA, velocity blocks per CTA (2: single precision only, and only for
-// cases whose sign classes each hold an even number of blocks)
+// K4 variants as the ABI names them: tx x ty cells and vpl velocity blocks.  A CTA of k4_march takes a strip of
+// `cols` columns and marches over `rows` of them (hb_micro.cuh); single precision always carries two velocity blocks
+// per lane, FP64 one.
 struct Shape {
-    int tx, ty, nw, vpl;
+    int tx, ty, vpl, cols, rows;
 };
-constexpr Shape K4_SHAPES[] = {{4, 4, 8, 1}, {4, 2, 8, 1}, {2, 2, 4, 1}, {8, 4, 16, 1}, {4, 2, 8, 2}};
+constexpr Shape K4_SHAPES[] = {{4, 4, 1, 4, 16}, {4, 2, 1, 2, 16}, {2, 2, 1, 2, 2}, {8, 4, 1, 4, 32}, {4, 2, 2, 4, 8}};
 constexpr int N_K4_SHAPES = 5;
-
-template <typename T>
-size_t k4_smem_of(int shape, int nt)
-{
-    switch (shape) {
-        case 0: return k4_cells_smem<T, 4, 4, 1>(nt);
-        case 1: return k4_cells_smem<T, 4, 2, 1>(nt);
-        case 2: return k4_cells_smem<T, 2, 2, 1>(nt);
-        case 3: return k4_cells_smem<T, 8, 4, 1>(nt);
-        default: return k4_cells_smem<T, 4, 2, 2>(nt);
-    }
-}
+template <typename T> constexpr int K4_VPL = std::is_same<T, float>::value ? 2 : 1;
 
 constexpr size_t SMEM_MAX = 219 * 1024;   // dynamic shared memory per CTA, leaving room for the static arrays
 
-// largest tile whose shared memory lets two CTAs share an SM, else the largest that fits at all
+// Strip and segment of the micro update's CTAs
+struct March {
+    int cols, rows;
+};
+template <typename T>
+size_t k4_smem_of(int cols, int nt, bool imp)
+{
+    return cols == 4 ? K4Layout<T, 4, K4_VPL<T>>::bytes(nt, imp) : K4Layout<T, 2, K4_VPL<T>>::bytes(nt, imp);
+}
+// of a variant: two columns where four need more shared memory than a CTA may have, and in a mesh of fewer columns,
+// since only strips of two may be partial.  Every strip and segment gives the same bits.
+template <typename T>
+March k4_march_of(int shape, int nx, int nt, bool imp)
+{
+    const Shape s = K4_SHAPES[shape];
+    return {s.cols == 4 && nx >= 4 && nt <= K4_NT4L && k4_smem_of<T>(4, nt, imp) <= SMEM_MAX ? 4 : 2, s.rows};
+}
+
+// Bytes a tile of a variant holds: its cells on all levels, twice its halo rectangle, face and cell parameters and
+// fluxes.  A variant is offered for a case while that fits a CTA's shared memory.
+template <typename T>
+size_t k4_tile_bytes(int shape, int nt)
+{
+    const Shape s = K4_SHAPES[shape];
+    const size_t cells = s.tx * s.ty, faces = s.ty * (s.tx + 1) + (s.ty + 1) * s.tx, halo = (s.tx + 3) * (s.ty + 3);
+    const size_t pair = VB * sizeof(P2<T>) * s.vpl;
+    return nt * cells * pair + 2 * halo * pair + 2 * (faces * NP + cells * NCP) * sizeof(T) + 2 * faces * pair;
+}
+
+// largest tile two of which fit an SM's shared memory, else the largest that fits at all
 template <typename T>
 int pick_k4_shape(int nt)
 {
     for (int s = 0; s < N_K4_SHAPES; ++s)
-        if (K4_SHAPES[s].vpl == 1 && k4_smem_of<T>(s, nt) <= 113 * 1024) return s;
+        if (K4_SHAPES[s].vpl == 1 && k4_tile_bytes<T>(s, nt) <= 113 * 1024) return s;
     for (int s = 0; s < N_K4_SHAPES; ++s)
-        if (K4_SHAPES[s].vpl == 1 && k4_smem_of<T>(s, nt) <= SMEM_MAX) return s;
+        if (K4_SHAPES[s].vpl == 1 && k4_tile_bytes<T>(s, nt) <= SMEM_MAX) return s;
     return -1;
 }
 
-// a K4 variant a case of this precision can run: its shared memory fits a CTA, and two velocity blocks per
-// CTA need single precision and sign classes of an even number of blocks (the CTA's blocks share one class)
+// a K4 variant a case of this precision is offered: its tile fits a CTA, and two velocity blocks per CTA need single
+// precision and sign classes of an even number of blocks
 template <typename T>
 bool k4_shape_ok(int shape, int nt, bool pairs)
 {
-    if (shape < 0 || shape >= N_K4_SHAPES || k4_smem_of<T>(shape, nt) > SMEM_MAX) return false;
+    if (shape < 0 || shape >= N_K4_SHAPES || k4_tile_bytes<T>(shape, nt) > SMEM_MAX) return false;
     return K4_SHAPES[shape].vpl == 1 || (sizeof(T) == 4 && pairs);
 }
 
@@ -227,6 +247,8 @@ void fill_host(HostCase& h, const hbugks_case& c)
     {
         int cnt[4] = {0, 0, 0, 0};
         for (int c : h.vcls) ++cnt[c];
+        h.ng[0] = h.nvb;
+        h.ng[1] = (cnt[0] + 1) / 2 + (cnt[1] + 1) / 2 + (cnt[2] + 1) / 2 + (cnt[3] + 1) / 2;
         h.pairs = cnt[0] % 2 == 0 && cnt[1] % 2 == 0 && cnt[2] % 2 == 0 && cnt[3] % 2 == 0;
     }
     {
@@ -356,6 +378,8 @@ struct LaunchSpec {
     int table;     // block offset table index
     int total;     // total blocks
     size_t smem;   // dynamic shared memory bytes
+    int nt;        // K4: levels, strip and segment
+    March march;
 };
 
 template <typename T>
@@ -398,11 +422,11 @@ namespace {
 template <typename T>
 void fill_offsets(Impl<T>& im, int ncases);
 
-void set_k4_blocks(HostCase& h)
+// CTAs of the micro update of a case
+template <typename T>
+int k4_blocks(const HostCase& h, March m)
 {
-    if (h.k4shape < 0) { h.k4b = 0; return; }
-    const Shape s4 = K4_SHAPES[h.k4shape];
-    h.k4b = ((h.nx + s4.tx - 1) / s4.tx) * ((h.ny + s4.ty - 1) / s4.ty) * (h.nvb / s4.vpl);
+    return ((h.nx + m.cols - 1) / m.cols) * ((h.ny + m.rows - 1) / m.rows) * h.ng[K4_VPL<T> - 1];
 }
 
 template <typename T>
@@ -417,7 +441,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
         h.k4shape = pick_k4_shape<T>(h.nt);
         im.max_nt = std::max(im.max_nt, h.nt);
         h.k1b = ((h.nx + K1_TX<T> - 1) / K1_TX<T>) * ((h.ny + K1_TY<T> - 1) / K1_TY<T>) * h.nt;
-        set_k4_blocks(h);
+        if (cases[k].phys.spectral_implicit) im.any_implicit = true;
     }
     im.d_cases = cv.take<CaseDev<T>>(ncases);
     im.d_status = cv.take<CaseStatus>(ncases);
@@ -427,13 +451,24 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
     im.d_tune_off = cv.take<int>(2);
     // launch specs: K1 per shape, K2, K3, K4 per shape; plus the step kernel (state setting only)
     im.specs.clear();
-    auto add = [&](int kind, int shape) { im.specs.push_back(LaunchSpec{kind, shape, (int)im.specs.size(), 0, 0}); };
+    auto add = [&](int kind, int shape) { im.specs.push_back(LaunchSpec{kind, shape, (int)im.specs.size(), 0, 0, 0, {}}); };
     add(0, 0);
     add(0, 1);
     add(1, 0);
     add(2, 0);
     im.k3_table = (int)im.specs.size() - 1;
-    for (int sh = 0; sh < N_K4_SHAPES; ++sh) add(4, sh);
+    // the micro update: one launch per strip, segment and level count (a warp per level)
+    std::vector<int> nts;
+    for (int k = 0; k < ncases; ++k)
+        if (std::find(nts.begin(), nts.end(), im.hc[k].nt) == nts.end()) nts.push_back(im.hc[k].nt);
+    std::sort(nts.begin(), nts.end());
+    for (int nt : nts)
+        for (int cols : {2, 4})
+            for (int rows : {2, 8, 16, 32}) {
+                add(4, 0);
+                im.specs.back().nt = nt;
+                im.specs.back().march = March{cols, rows};
+            }
     add(5, 0);
     im.steps_table = (int)im.specs.size() - 1;
     const int ntab = (int)im.specs.size();
@@ -466,7 +501,14 @@ void fill_offsets(Impl<T>& im, int ncases)
                 case 0: nb = h.k1sep == sp.shape ? h.k1b : 0; smem = k1_smem_of<T>(); break;
                 case 1: nb = h.k2b; break;
                 case 2: nb = h.k3b; break;
-                case 4: if (h.k4shape == sp.shape) { nb = h.k4b; smem = std::max(smem, k4_smem_of<T>(sp.shape, h.nt)); } break;
+                case 4:
+                    if (h.k4shape >= 0 && h.nt == sp.nt) {
+                        const March m = k4_march_of<T>(h.k4shape, h.nx, h.nt, im.any_implicit);
+                        if (m.cols != sp.march.cols || m.rows != sp.march.rows) break;
+                        nb = k4_blocks<T>(h, m);
+                        smem = k4_smem_of<T>(m.cols, h.nt, im.any_implicit);
+                    }
+                    break;
                 case 5: nb = h.ksb; break;
             }
             acc += nb;
@@ -691,26 +733,18 @@ void launch_k1(int shape, int total, size_t smem, Batch<T> b, cudaStream_t s)
     else k1_kernel<T, false>()<<<total, K1_TX<T> * K1_TY<T> * 32, smem, s>>>(b);
 }
 
-template <typename T, bool IMP>
-void launch_k4_(int shape, int total, size_t smem, Batch<T> b, cudaStream_t s)
-{
-    switch (shape) {
-        case 0: k4_cells<T, 4, 4, 8, IMP, 1><<<total, 8 * 32, smem, s>>>(b); break;
-        case 1: k4_cells<T, 4, 2, 8, IMP, 1><<<total, 8 * 32, smem, s>>>(b); break;
-        case 2: k4_cells<T, 2, 2, 4, IMP, 1><<<total, 4 * 32, smem, s>>>(b); break;
-        case 3: k4_cells<T, 8, 4, 16, IMP, 1><<<total, 16 * 32, smem, s>>>(b); break;
-        default:
-            if constexpr (sizeof(T) == 4) k4_cells<T, 4, 2, 8, IMP, 2><<<total, 8 * 32, smem, s>>>(b);
-            break;
-    }
-}
-
 // the explicit-only kernels unless a case of the handle takes the spectral source at the new iterate
 template <typename T>
-void launch_k4(bool imp, int shape, int total, size_t smem, Batch<T> b, cudaStream_t s)
+void launch_k4(bool imp, March m, int nt, int total, size_t smem, Batch<T> b, cudaStream_t s)
 {
-    if (imp) launch_k4_<T, true>(shape, total, smem, b, s);
-    else launch_k4_<T, false>(shape, total, smem, b, s);
+    constexpr int P = K4_VPL<T>;
+    auto go = [&](auto plain, auto implicit) {
+        if (imp) implicit<<<total, nt * 32, smem, s>>>(b, m.rows);
+        else plain<<<total, nt * 32, smem, s>>>(b, m.rows);
+    };
+    if (m.cols == 2) go(k4_march<T, 2, P, false, K4_T2>, k4_march<T, 2, P, true, K4_T2>);
+    else if (nt <= K4_NT4) go(k4_march<T, 4, P, false, K4_T4>, k4_march<T, 4, P, true, K4_T4>);
+    else go(k4_march<T, 4, P, false, K4_T4L>, k4_march<T, 4, P, true, K4_T4L>);
 }
 
 // every K4 shape may be chosen later (autotuning), so each gets the largest dynamic shared memory it can use
@@ -726,14 +760,10 @@ cudaError_t set_smem_attributes()
     auto set = [&](auto k) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
     };
-    set(k4_cells<T, 4, 4, 8, false, 1>); set(k4_cells<T, 4, 2, 8, false, 1>);
-    set(k4_cells<T, 2, 2, 4, false, 1>); set(k4_cells<T, 8, 4, 16, false, 1>);
-    set(k4_cells<T, 4, 4, 8, true, 1>); set(k4_cells<T, 4, 2, 8, true, 1>);
-    set(k4_cells<T, 2, 2, 4, true, 1>); set(k4_cells<T, 8, 4, 16, true, 1>);
-    if constexpr (sizeof(T) == 4) {
-        set(k4_cells<T, 4, 2, 8, false, 2>);
-        set(k4_cells<T, 4, 2, 8, true, 2>);
-    }
+    constexpr int P = K4_VPL<T>;
+    set(k4_march<T, 2, P, false, K4_T2>); set(k4_march<T, 2, P, true, K4_T2>);
+    set(k4_march<T, 4, P, false, K4_T4>); set(k4_march<T, 4, P, true, K4_T4>);
+    set(k4_march<T, 4, P, false, K4_T4L>); set(k4_march<T, 4, P, true, K4_T4L>);
     return e;
 }
 
@@ -766,7 +796,7 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
                 k3_macro<T><<<sp.total, k3_threads(im.max_nt), 0, s>>>(b);
                 break;
             }
-            case 4: launch_k4<T>(im.any_implicit, sp.shape, sp.total, sp.smem, b, s); break;
+            case 4: launch_k4<T>(im.any_implicit, sp.march, sp.nt, sp.total, sp.smem, b, s); break;
         }
     }
     if (ev) {
@@ -871,8 +901,8 @@ hbugks_status upload_offsets(hbugks_t h, Impl<T>& im)
 }
 
 // ------------------------------------------------------------------------------ autotuner of the K4 variant
-// The micro update's variant (cells per CTA, velocity blocks per CTA) trades halo re-reads, pass-1 work and the
-// indices and parameters shared by a CTA's blocks against shared memory per CTA and so against CTAs per SM;
+// The micro update's variant (columns and rows a CTA marches over) trades the upwind column and row that are computed
+// twice against shared memory and registers per CTA, and on small meshes against the number of CTAs;
 // which wins depends on the level count, the velocity grid, the mesh and the GPU.  Each variant the case can
 // run is timed on the case itself (one warm-up launch, then three), after one iteration from rest has filled
 // the parameters the kernel reads.  Choices are cached per process by everything that sets the launch: mesh
@@ -900,7 +930,7 @@ hbugks_status autotune(hbugks_t h, Impl<T>& im, int ncases)
         std::lock_guard<std::mutex> lk(tune_cache().mu);
         for (int k = 0; k < ncases; ++k) {
             const HostCase& hc = im.hc[k];
-            keys[k] = {hc.nx, hc.ny, hc.nu, hc.nv, hc.nvb, hc.nt, (int)sizeof(T), sms, hc.src.phys.spectral_implicit};
+            keys[k] = {hc.nx, hc.ny, hc.nu, hc.nv, hc.nvb, hc.nt, (int)sizeof(T), sms, im.any_implicit ? 1 : 0};
             auto it = tune_cache().best.find(keys[k]);
             if (it != tune_cache().best.end()) im.hc[k].k4shape = it->second;
             else need = true;
@@ -924,15 +954,15 @@ hbugks_status autotune(hbugks_t h, Impl<T>& im, int ncases)
             float best_ms = 0.f;
             for (int sh = 0; sh < N_K4_SHAPES; ++sh) {
                 if (!k4_shape_ok<T>(sh, hc.nt, hc.pairs != 0)) continue;
-                const size_t smem = k4_smem_of<T>(sh, hc.nt);
-                const Shape S = K4_SHAPES[sh];
-                const int off[2] = {0, ((hc.nx + S.tx - 1) / S.tx) * ((hc.ny + S.ty - 1) / S.ty) * (hc.nvb / S.vpl)};
+                const bool imp = im.any_implicit;
+                const March m = k4_march_of<T>(sh, hc.nx, hc.nt, imp);
+                const size_t smem = k4_smem_of<T>(m.cols, hc.nt, imp);
+                const int off[2] = {0, k4_blocks<T>(hc, m)};
                 HB_CK(cudaMemcpyAsync(im.d_tune_off, off, sizeof off, cudaMemcpyHostToDevice, h->s));
                 const Batch<T> b{im.d_cases + k, 1, im.d_tune_off};
-                const bool imp = hc.src.phys.spectral_implicit != 0;
-                launch_k4<T>(imp, sh, off[1], smem, b, h->s);
+                launch_k4<T>(imp, m, hc.nt, off[1], smem, b, h->s);
                 HB_CK(cudaEventRecord(e0, h->s));
-                for (int r = 0; r < 3; ++r) launch_k4<T>(imp, sh, off[1], smem, b, h->s);
+                for (int r = 0; r < 3; ++r) launch_k4<T>(imp, m, hc.nt, off[1], smem, b, h->s);
                 HB_CK(cudaEventRecord(e1, h->s));
                 HB_CK(cudaEventSynchronize(e1));
                 float ms = 0.f;
@@ -945,7 +975,6 @@ hbugks_status autotune(hbugks_t h, Impl<T>& im, int ncases)
         }
         HB_CK(cudaGetLastError());
     }
-    for (auto& hc : im.hc) set_k4_blocks(hc);
     return upload_offsets(h, im);
 }
 
@@ -955,7 +984,6 @@ hbugks_status do_create(hbugks_t h, Impl<T>& im, int ncases, const hbugks_case* 
     plan(im, ncases, cases, h->ws);
     for (auto& hc : im.hc) {
         if (hc.k4shape < 0) return HBUGKS_EINVAL;
-        if (hc.src.phys.spectral_implicit) im.any_implicit = true;
     }
     HB_CK(set_smem_attributes<T>());
     std::vector<std::vector<char>> keep;
@@ -1573,7 +1601,6 @@ hbugks_status hbugks_set_micro_variant(hbugks_t h, int case_index, int tx, int t
         hbugks_status rc = begin(h);
         if (rc) return rc;
         hc.k4shape = sh;
-        set_k4_blocks(hc);
         if ((rc = upload_offsets(h, im)) != HBUGKS_OK) return rc;
         HB_CK(cudaStreamSynchronize(h->s));
         if (h->g1) { cudaGraphExecDestroy(h->g1); h->g1 = nullptr; }

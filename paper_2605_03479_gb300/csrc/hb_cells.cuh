@@ -7,11 +7,10 @@
 // lying downwind of it (Sec 2.2, upwind interface reconstruction):
 //   k1_cells : per (cell, level): velocity sums of the reconstruction of h^k at the cell's downwind faces,
 //              kept per sign class (half-face sums), and the raw moments of h^k;
-//   k4_cells : per (cell, level, 32 velocities): interface micro fluxes (Eq. micro_flux), spectral source and
-//              the semi-implicit collision update (Eq. fv_h).
-// A CTA of k1_cells owns a tile of cells and one level and runs over all velocity blocks; a CTA of k4_cells
-// owns a tile of cells and one or two velocity blocks of one sign class and runs over all levels.  Both stage
-// the tile and its halo in shared memory with bulk copies (TMA) completing on an mbarrier.  The distributions
+//   k4_march : per (cell, level, velocity): interface micro fluxes, spectral source and update (hb_micro.cuh).
+// A CTA of k1_cells owns a tile of cells and one level and runs over all velocity blocks; a CTA of k4_march
+// owns a strip of cells and one or two velocity blocks of one sign class on all levels.  Both stage
+// their cells with a halo in shared memory with bulk copies (TMA) completing on an mbarrier.  The distributions
 // h and b of a velocity are stored side by side and carried as one pair (hb_common.cuh): one 8-byte access
 // and, in single precision, one packed FP32x2 instruction for both wherever they see the same arithmetic
 // (differences, limited slopes, reconstruction, the flux combination, velocity sums with a common weight,
@@ -43,7 +42,7 @@ __device__ __forceinline__ bool pos64(double x) { return (unsigned)(__double2hii
 __device__ __forceinline__ double2 vleer2(double2 s1, double2 s2)
 {
     const double px = s1.x * s2.x, py = s1.y * s2.y;
-    const double qx = px * rcp64(s1.x + s2.x), qy = py * rcp64(s1.y + s2.y);
+    const double qx = px * rcp64(__dadd_rn(s1.x, s2.x)), qy = py * rcp64(__dadd_rn(s1.y, s2.y));
     return make_double2(pos64(px) ? qx : 0.0, pos64(py) ? qy : 0.0);
 }
 
@@ -63,41 +62,6 @@ template <typename V, typename T>
 __device__ __forceinline__ V slope2i(V fm, V f0, V fp, T wm, T wp)
 {
     return vleer2(pmul(psub(f0, fm), bc(wm)), pmul(psub(fp, f0), bc(wp)));
-}
-
-// spectral source of one cell and lane: sum_d e_d (f_{n-d} - f_{n+d}) for (h, b) (Eq. D_explicit in paired
-// form), levels lv pairs apart in shared memory, e_d as broadcast pairs (etb[0] = 0)
-template <int NH, typename V>
-__device__ __forceinline__ V spectral2(const V* fc, int n, int nt, int lv, const V* etb)
-{
-    V e = etb[0];
-#pragma unroll
-    for (int d = 1; d <= NH; ++d) {
-        int nm = n - d; nm += nm < 0 ? nt : 0;
-        int np = n + d; np -= np >= nt ? nt : 0;
-        e = pfma(etb[d], psub(fc[nm * lv], fc[np * lv]), e);
-    }
-    return e;
-}
-
-// spectral source of every level of one cell and lane, in place: the pair of level n (levels lv pairs apart)
-// becomes sum_d e_d (f_{n-d} - f_{n+d}), with the operations of spectral2 in the same order
-template <int NH, typename V, typename T>
-__device__ __forceinline__ void spectral_all(V* fc, int lv, const T* et)
-{
-    constexpr int NT = 2 * NH + 1;
-    V f[NT], eb[NH + 1];
-#pragma unroll
-    for (int m = 0; m < NT; ++m) f[m] = fc[m * lv];
-#pragma unroll
-    for (int d = 0; d <= NH; ++d) eb[d] = bc(et[d]);
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-        V e = eb[0];
-#pragma unroll
-        for (int d = 1; d <= NH; ++d) e = pfma(eb[d], psub(f[(n - d + NT) % NT], f[(n + d) % NT]), e);
-        fc[n * lv] = e;
-    }
 }
 
 __device__ __forceinline__ void mbar_setup(uint64_t* bars, int n)
@@ -459,583 +423,6 @@ template <typename T, int TX, int TY, int G, int S>
 constexpr size_t k1_cells_smem()
 {
     return (size_t)S * G * (TX + 2) * (TY + 2) * VB * sizeof(P2<T>);
-}
-
-// ------------------------------------------------------------------------------ K4: micro update
-
-// Micro flux pair (delta form, divided by dG_f) through the downwind face of the reconstructing cell, for one
-// lane: u_n [C1' dH + H Q + C4' d0 + C5' (u_n s_n + u_t s_t)] for h and u_n [C1' dB + B (Q + lin) + C4' e0 +
-// C5' (...)] for b, from the face's parameters fp (shared memory; the cubic at qo and linear term at lo belong to
-// the upwind side), the expm1 factors (ex, ey) of the interface Maxwellian at the lane's velocity, the
-// reconstructed pair d0 and the normal and tangential slope pairs; unb, utb are (u_n, u_n) and (u_t, u_t).
-template <typename T, typename V>
-__device__ __forceinline__ V flux2(const T* fp, int qo, int lo, T ex, T ey, T href, T u, T v, V unb, V utb, V d0,
-                                   V sn, V st)
-{
-    const T* sc = fp + F_RM1;      // r - 1, r, 1/(2 lam), 1/(2 lam) - 1/(2 lam0), C1', C4', C5', nin
-    const T E = ex + ey + ex * ey;
-    const T dH = href * (sc[0] + sc[1] * E);
-    const T H = href + dH;
-    const T i2l = sc[2];
-    const T dB = dH * i2l + href * sc[3];
-    const T* l = fp + lo;
-    const T Q = cubic(fp + qo, u, v);
-    const T Qb = Q + l[0] + l[1] * u + l[2] * v;
-    V m = pk(sc[4] * dH + H * Q, sc[4] * dB + (H * i2l) * Qb);
-    m = pfma(bc(sc[5]), d0, m);
-    m = pfma(bc(sc[6]), pfma(unb, sn, pmul(utb, st)), m);
-    return pmul(unb, m);
-}
-
-// Flux pair (delta form, divided by dG_f) of the distribution a diffuse wall re-emits, rho_w H_w u_n: velocities
-// of the block leave the wall.
-template <typename T, typename V>
-__device__ __forceinline__ V flux_wall2(const T* fp, const T* __restrict__ tb, int iu, int ivn, T href, V unb)
-{
-    const T* wp = fp + F_WRM1;
-    const T ex = __ldg(tb + iu), ey = __ldg(tb + ivn);
-    const T E = ex + ey + ex * ey;
-    const T dHw = href * (wp[0] + wp[1] * E);
-    return pmul(unb, pk(dHw, dHw * wp[2] + href * wp[3]));
-}
-
-// Equilibrium pair (H+ - H_ref, B+ - B_ref) of one cell-parameter slot q at the lane's velocity: the Maxwellian
-// from the cell table factors (ex, ey), and with the Shakhov model the correction (L Q) H for h and (L Q + 2 L) B
-// for b (L, Q the linear and quadratic factors of s (c.q)(2 lam |c|^2 - 4); r2 = u^2 + v^2).
-template <typename T>
-__device__ __forceinline__ P2<T> eq2(const T* q, T ex, T ey, T href, T u, T v, T r2, bool shakhov)
-{
-    const T E = ex + ey + ex * ey;
-    const T dH = href * (q[E_RM1] + q[E_R] * E);
-    const T dB = dH * q[E_I2L] + href * q[E_DI2L];
-    if (!shakhov) return pk(dH, dB);
-    const T H = href + dH;
-    const T L = q[E_L] + q[E_L + 1] * u + q[E_L + 2] * v;
-    const T Qs = q[E_Q] + q[E_Q + 1] * u + q[E_Q + 2] * v + q[E_Q + 3] * r2;
-    const T sk = L * Qs;
-    return pfma(pk(H, H * q[E_I2L]), pk(sk, sk + T(2) * L), pk(dH, dB));
-}
-
-// One bulk copy of the per-level batches of k4_cells, formed once per CTA: level l's copy reads src + l sstride
-// and lands in ring slot l & 1 (dst + (l & 1) dslot).  kind 0: a row of the halo rectangle, 1: a row of face
-// parameters (both of level k in batch k), 2: a row of cell coefficients (level k - 1 in batch k); bytes 0: the
-// row lies outside the domain.
-struct alignas(16) K4Copy {
-    const char* src;
-    long long sstride;
-    uint32_t dst, dslot, bytes;
-    int kind;
-};
-
-// Shared-memory layout of k4_cells (byte offsets, pairs for distributions, each block 16-byte aligned).  A CTA
-// owns VPL velocity blocks of one sign class (h = 0..VPL-1 below), and each lane one velocity of every block:
-//   own   [nt][VPL][NCT][32] pairs   the tile's own cells on every level: h^k as loaded; in the explicit form
-//                                    replaced once by the spectral source of every level
-//   rect  [2][VPL][NR][32] pairs     per level: the tile with its halo, (TX+3) x (TY+3) cells, two cells on
-//                                    the upwind side of each axis and one on the downwind side (ring of 2)
-//   fp    [2][NFT][NP] T             per level: parameters of the tile's faces (ring of 2 levels)
-//   cp    [2][NCT][NCP] T            per level: update coefficients of the tile's cells (ring of 2 levels)
-//   flux  [2][VPL][NFT][32] pairs    per level: micro fluxes of the tile's faces (double buffered)
-template <typename T, int TX, int TY, int VPL>
-struct K4Layout {
-    using V = P2<T>;
-    static constexpr int PX = TX + 3, PY = TY + 3, NR = PX * PY, NCT = TX * TY;
-    static constexpr int NFX = TY * (TX + 1), NFY = (TY + 1) * TX, NFT = NFX + NFY;
-    static constexpr size_t RECT = (size_t)VPL * NR * VB;               // pairs per ring slot
-    static constexpr size_t FP = (size_t)NFT * NP, CP = (size_t)NCT * NCP, FLUX = (size_t)VPL * NFT * VB;
-    __host__ __device__ static constexpr size_t own_bytes(int nt) { return (size_t)nt * VPL * NCT * VB * sizeof(V); }
-    __host__ __device__ static constexpr size_t rect_off(int nt) { return own_bytes(nt); }
-    __host__ __device__ static constexpr size_t fp_off(int nt) { return rect_off(nt) + 2 * RECT * sizeof(V); }
-    __host__ __device__ static constexpr size_t cp_off(int nt) { return fp_off(nt) + 2 * FP * sizeof(T); }
-    __host__ __device__ static constexpr size_t flux_off(int nt) { return cp_off(nt) + 2 * CP * sizeof(T); }
-    __host__ __device__ static constexpr size_t bytes(int nt) { return flux_off(nt) + 2 * FLUX * sizeof(V); }
-};
-
-// A CTA: a TX x TY tile of cells, VPL velocity blocks of one sign class, all levels.  Per level, the first pass
-// reconstructs every tile cell and the upwind halo cells and evaluates the flux through each one's downwind
-// face (every face of the tile exactly once); the second pass applies Eq. fv_h to the tile cells.  Each item
-// (a cell of a pass) forms its indices, addresses and face or cell parameters once and serves the lane's
-// velocity in each of the VPL blocks.  The second pass of level n runs in the same barrier interval as the
-// first pass of level n + 1 (fluxes double buffered), so one barrier separates the levels.  In the explicit
-// form the spectral source of every level is formed once per CTA, in place in the own-cell store, and each
-// warp keeps h^k of its pass-2 cells from pass 1.  With IMP and a case that asks for it, the spectral source is
-// taken at the new iterate instead: pass 2 leaves each level's right-hand side in the own-cell store and a last
-// pass applies the per-cell inverse across levels.  Batch k of bulk copies (the halo rectangle and face
-// parameters of level k, the cell coefficients of level k - 1; batch 0 also every level of the tile's own
-// cells) completes on mbarrier k & 1 and is issued one level ahead of its use.
-template <typename T, int TX, int TY, int NW, bool IMP, int VPL>
-__global__ void __launch_bounds__(NW * 32) k4_cells(Batch<T> B)
-{
-    using L = K4Layout<T, TX, TY, VPL>;
-    using V = P2<T>;
-    constexpr int PX = L::PX, PY = L::PY, NR = L::NR, NCT = L::NCT, NFX = L::NFX, NFT = L::NFT;
-    constexpr int NIT = NCT + TY + TX, NPASS = (NIT + NW - 1) / NW;
-    constexpr int NP2 = (NCT + NW - 1) / NW;                  // tile cells per warp in pass 2
-    constexpr int SROWS = 4;                                  // tile rows per strip of the CTA order
-    constexpr int LVO = VPL * NCT * VB;                       // level stride of the own-cell store (pairs)
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t bars[2];
-    __shared__ T gxr[PX], gxh[PX], gyr[PY], gyh[PY];
-    const int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
-    if (!cd.st->active) return;
-    // another CTA may set the error word while this one starts: decide for the whole CTA at once
-    if (__syncthreads_or(*(volatile int*)cd.err != 0)) return;
-    const bool expire = *(volatile const int*)cd.expire != 0;
-    const int nvg = cd.nvb / VPL, nx = cd.nx, ny = cd.ny;
-    // CTA order: velocity group fastest (the CTAs of one tile share its parameters in L2), then tiles in
-    // strips of SROWS tile rows, column by column (neighbour tiles, whose halos overlap, run close in time)
-    const int lb = blockIdx.x - B.off[cs];
-    const int vb = (lb % nvg) * VPL, tile = lb / nvg;         // vb: the CTA's first velocity block
-    const int ntx = (nx + TX - 1) / TX, nty = (ny + TY - 1) / TY;
-    const int strip = tile / (ntx * SROWS), rows = min(SROWS, nty - strip * SROWS);
-    const int rem = tile - strip * ntx * SROWS;
-    const int i0 = (rem / rows) * TX, j0 = (strip * SROWS + rem % rows) * TY;
-    const int nt = cd.nt, nc = cd.nc, nh = cd.nh, nfx = cd.nfx, nf = cd.nf;
-    const int nuv = cd.nu + cd.nv;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int cls = __ldg(cd.vcls + vb);
-    const bool xneg = (cls & 1) != 0, yneg = (cls & 2) != 0;
-    const int xlo = xneg ? -1 : -2, ylo = yneg ? -1 : -2;
-    const int iend = min(i0 + TX, nx), jend = min(j0 + TY, ny);
-    V* const own = reinterpret_cast<V*>(smem_raw);
-    V* const rect = reinterpret_cast<V*>(smem_raw + L::rect_off(nt));
-    T* const fps = reinterpret_cast<T*>(smem_raw + L::fp_off(nt));
-    T* const cps = reinterpret_cast<T*>(smem_raw + L::cp_off(nt));
-    V* const fbuf = reinterpret_cast<V*>(smem_raw + L::flux_off(nt));
-    mbar_setup(bars, 2);
-    const int p = cd.st->parity;
-    const V* gf = cd.f[p];
-    const size_t bstride = (size_t)nt * nc * VB;              // pairs between consecutive velocity blocks
-    // bulk copies of the rectangle rows (clipped to the domain)
-    const int c0 = max(i0 + xlo, 0), c1 = min(i0 + xlo + PX, nx);
-    const int nfr = iend - i0;                                // valid cells per tile row
-    const uint32_t row_b = (uint32_t)((c1 - c0) * VB * sizeof(V));
-    int rrows = 0;
-    for (int r = 0; r < PY; ++r) {
-        const int jj = j0 + ylo + r;
-        rrows += (jj >= 0 && jj < ny) ? 1 : 0;
-    }
-    const uint32_t rect_b = (uint32_t)(VPL * rrows) * row_b;
-    const uint32_t fp_b = (uint32_t)(((jend - j0) * (nfr + 1) + (jend - j0 + 1) * nfr) * NP * sizeof(T));
-    const uint32_t cp_b = (uint32_t)((jend - j0) * nfr * NCP * sizeof(T));
-    // batch 0 (warp 0): rectangle and face parameters of level 0, every level of the own cells
-    {
-        constexpr int NRECT = VPL * PY, NFPR = 2 * TY + 1;
-        const int nown = nt * VPL * TY;
-        if (warp == 0) {
-            if (lane == 0)
-                mbar_arrive_expect(&bars[0], rect_b + fp_b + (uint32_t)(nt * VPL * (jend - j0) * nfr * VB * sizeof(V)));
-            __syncwarp();
-            for (int q = lane; q < NRECT + NFPR + nown; q += 32) {
-                if (q < NRECT) {
-                    const int h = q / PY, r = q % PY, jj = j0 + ylo + r;
-                    if (jj < 0 || jj >= ny) continue;
-                    bulk_g2s(rect + (size_t)(h * NR + r * PX + c0 - (i0 + xlo)) * VB,
-                             gf + (vb + h) * bstride + ((size_t)jj * nx + c0) * VB, row_b, &bars[0]);
-                } else if (q < NRECT + NFPR) {
-                    const int r = q - NRECT;
-                    if (r < TY) {                             // x-faces of tile row r
-                        const int jj = j0 + r;
-                        if (jj >= ny) continue;
-                        bulk_g2s(fps + (size_t)r * (TX + 1) * NP, cd.fpar + ((size_t)jj * (nx + 1) + i0) * NP,
-                                 (uint32_t)((nfr + 1) * NP * sizeof(T)), &bars[0]);
-                    } else {                                  // y-faces of face row r - TY
-                        const int fr = r - TY, jj = j0 + fr;
-                        if (jj > jend) continue;
-                        bulk_g2s(fps + (size_t)(NFX + fr * TX) * NP, cd.fpar + ((size_t)nfx + (size_t)jj * nx + i0) * NP,
-                                 (uint32_t)(nfr * NP * sizeof(T)), &bars[0]);
-                    }
-                } else {
-                    const int o = q - NRECT - NFPR;           // own cells: row, block, level
-                    const int r = o % TY, h = (o / TY) % VPL, n = o / (TY * VPL), jj = j0 + r;
-                    if (jj >= ny) continue;
-                    bulk_g2s(own + ((size_t)(n * VPL + h) * NCT + r * TX) * VB,
-                             gf + (vb + h) * bstride + (size_t)n * nc * VB + ((size_t)jj * nx + i0) * VB,
-                             (uint32_t)(nfr * VB * sizeof(V)), &bars[0]);
-                }
-            }
-        }
-    }
-    // the copies of batches 1..nt, formed once: at each level warp 0 then only offsets them
-    constexpr int NQ = VPL * PY + 2 * TY + 1 + TY;
-    static_assert(NQ <= 32, "one lane of warp 0 per copy of a batch");
-    __shared__ K4Copy cpy[32];
-    if (warp == 0 && lane < NQ) {
-        K4Copy c;
-        c.bytes = 0;
-        c.src = nullptr;
-        c.sstride = 0;
-        c.dst = 0;
-        c.dslot = 0;
-        c.kind = 0;
-        if (lane < VPL * PY) {
-            const int h = lane / PY, r = lane % PY, jj = j0 + ylo + r;
-            if (jj >= 0 && jj < ny) {
-                c.src = reinterpret_cast<const char*>(gf + (vb + h) * bstride + ((size_t)jj * nx + c0) * VB);
-                c.sstride = (long long)nc * VB * sizeof(V);
-                c.dst = smem_u32(rect + (size_t)(h * NR + r * PX + c0 - (i0 + xlo)) * VB);
-                c.dslot = (uint32_t)(L::RECT * sizeof(V));
-                c.bytes = row_b;
-            }
-        } else if (lane < VPL * PY + 2 * TY + 1) {
-            const int r = lane - VPL * PY;
-            c.kind = 1;
-            c.sstride = (long long)nf * NP * sizeof(T);
-            c.dslot = (uint32_t)(L::FP * sizeof(T));
-            if (r < TY) {                                     // x-faces of tile row r
-                const int jj = j0 + r;
-                if (jj < ny) {
-                    c.src = reinterpret_cast<const char*>(cd.fpar + ((size_t)jj * (nx + 1) + i0) * NP);
-                    c.dst = smem_u32(fps + (size_t)r * (TX + 1) * NP);
-                    c.bytes = (uint32_t)((nfr + 1) * NP * sizeof(T));
-                }
-            } else {                                          // y-faces of face row r - TY
-                const int fr = r - TY, jj = j0 + fr;
-                if (jj <= jend) {
-                    c.src = reinterpret_cast<const char*>(cd.fpar + ((size_t)nfx + (size_t)jj * nx + i0) * NP);
-                    c.dst = smem_u32(fps + (size_t)(NFX + fr * TX) * NP);
-                    c.bytes = (uint32_t)(nfr * NP * sizeof(T));
-                }
-            }
-        } else {
-            const int r = lane - VPL * PY - 2 * TY - 1, jj = j0 + r;   // cells of tile row r
-            c.kind = 2;
-            if (jj < ny) {
-                c.src = reinterpret_cast<const char*>(cd.cpar + ((size_t)jj * nx + i0) * NCP);
-                c.sstride = (long long)nc * NCP * sizeof(T);
-                c.dst = smem_u32(cps + (size_t)r * TX * NCP);
-                c.dslot = (uint32_t)(L::CP * sizeof(T));
-                c.bytes = (uint32_t)(nfr * NCP * sizeof(T));
-            }
-        }
-        cpy[lane] = c;
-    }
-    __syncwarp();
-    // batch k >= 1 (warp 0): rectangle and face parameters of level k (k < nt), cell coefficients of level k - 1
-    auto issue_next = [&](int k) {
-        const bool lvl = k < nt;
-        uint64_t* bar = &bars[k & 1];
-        if (lane == 0) mbar_arrive_expect(bar, (lvl ? rect_b + fp_b : 0u) + cp_b);
-        __syncwarp();
-        if (lane < NQ) {
-            const K4Copy c = cpy[lane];
-            if (c.bytes != 0 && (lvl || c.kind == 2)) {
-                const int l = c.kind == 2 ? k - 1 : k;
-                bulk_g2s_at(c.dst + (uint32_t)(l & 1) * c.dslot, c.src + (long long)l * c.sstride, c.bytes, bar);
-            }
-        }
-    };
-    for (int k = threadIdx.x; k < PX; k += blockDim.x) {
-        const int ii = i0 + xlo + k;
-        gxr[k] = (ii >= 0 && ii < nx - 1) ? T(2) * T(cd.rdx[ii]) : T(0);
-        gxh[k] = (ii >= 0 && ii < nx) ? T(cd.hx[ii]) : T(0);
-    }
-    for (int k = threadIdx.x; k < PY; k += blockDim.x) {
-        const int jj = j0 + ylo + k;
-        gyr[k] = (jj >= 0 && jj < ny - 1) ? T(2) * T(cd.rdy[jj]) : T(0);
-        gyh[k] = (jj >= 0 && jj < ny) ? T(cd.hy[jj]) : T(0);
-    }
-    // the lane's velocity in each of the CTA's blocks
-    T u[VPL], v[VPL], href[VPL], r2[VPL];
-    int iu[VPL], ivn[VPL];
-#pragma unroll
-    for (int h = 0; h < VPL; ++h) {
-        const int av = (vb + h) * VB + lane;
-        u[h] = __ldg(cd.tu + av);
-        v[h] = __ldg(cd.tv + av);
-        href[h] = __ldg(cd.thref + av);
-        r2[h] = u[h] * u[h] + v[h] * v[h];
-        iu[h] = __ldg(cd.viu + av);
-        ivn[h] = cd.nu + __ldg(cd.viv + av);
-    }
-    V etb[IMP ? 8 : 1];                                       // implicit-capable kernels: e_d as pairs
-#pragma unroll
-    for (int d = 0; d < (IMP ? 8 : 1); ++d) etb[d] = bc(cd.et[d]);
-    const T* __restrict__ ftab = cd.ftab;
-    const T* __restrict__ wtab = cd.wtab;
-    const T* __restrict__ ctab = cd.ctab;
-    const bool shakhov = cd.shakhov != 0;
-    const int NTf = nt * nuv;                                 // per-face stride of the expm1 tables
-    const int qoff = xneg ? F_QR : F_QL, loff = xneg ? F_LBR : F_LBL;
-    const int qoffy = yneg ? F_QR : F_QL, loffy = yneg ? F_LBR : F_LBL;
-    int* err = cd.err;
-
-    const bool implicit = IMP && cd.spectral_implicit != 0;   // IMP = false compiles the explicit form alone
-    // a tile none of whose first-pass cells (tile cells and upwind halo) touches a wall: every stencil neighbour
-    // of each exists
-    const bool interior = i0 >= 2 && j0 >= 2 && i0 + TX <= nx - 2 && j0 + TY <= ny - 2;
-    constexpr bool PAIRED = NCT == 2 * NW;                    // each warp owns two tile cells in pass 1
-    V f0k[NP2][VPL];                                          // h^k of the warp's pass-2 cells (explicit form)
-#pragma unroll
-    for (int r = 0; r < NP2; ++r)
-#pragma unroll
-        for (int h = 0; h < VPL; ++h) f0k[r][h] = bc(T(0));
-
-    __syncthreads();                                          // the spacing tables above, for every warp
-    for (int s = 0; s <= nt; ++s) {
-        if (warp == 0 && s < nt) issue_next(s + 1);
-        // the test hook reports the first wait as expired only after it has completed
-        const int fail = !mbar_wait(&bars[s & 1], (uint32_t)((s >> 1) & 1), err) || expire;
-        if (!fail) {
-            if (!IMP && s == 0) {
-                // the spectral source of every level of the warp's own cells, once, in place of h^k
-#pragma unroll
-                for (int r = 0; r < NP2; ++r) {
-                    const int ct = warp + r * NW;
-                    if (ct >= NCT) break;
-                    if (i0 + ct % TX >= nx || j0 + ct / TX >= ny) continue;
-#pragma unroll
-                    for (int h = 0; h < VPL; ++h) {
-                        V* fc = own + (size_t)(h * NCT + ct) * VB + lane;
-                        switch (nh) {
-                            case 0: spectral_all<0>(fc, LVO, cd.et); break;
-                            case 1: spectral_all<1>(fc, LVO, cd.et); break;
-                            case 2: spectral_all<2>(fc, LVO, cd.et); break;
-                            case 3: spectral_all<3>(fc, LVO, cd.et); break;
-                            case 4: spectral_all<4>(fc, LVO, cd.et); break;
-                            case 5: spectral_all<5>(fc, LVO, cd.et); break;
-                            case 6: spectral_all<6>(fc, LVO, cd.et); break;
-                            default: spectral_all<7>(fc, LVO, cd.et); break;
-                        }
-                    }
-                }
-                __syncwarp();
-            }
-            if (s > 0) {
-                // ---- pass 2, level s - 1 (ahead of pass 1 of level s, which refills f0k): Eq. fv_h with the
-                // spectral source (delta form)
-                const int n = s - 1;
-                const V* F = fbuf + (size_t)(n & 1) * L::FLUX + lane;
-                V* on = cd.f[p ^ 1] + vb * bstride + (size_t)n * nc * VB + lane;
-                const T* cpn = cps + (size_t)(n & 1) * L::CP;
-                const T* ctn = ctab + n * 2 * nuv;
-#pragma unroll
-                for (int r = 0; r < NP2; ++r) {
-                    const int ct = warp + r * NW;
-                    if (ct >= NCT) break;
-                    const int ti = ct % TX, tj = ct / TX;
-                    const int i = i0 + ti, j = j0 + tj;
-                    if (i >= nx || j >= ny) continue;
-                    const int c = j * nx + i;
-                    const T* tb = ctn + c * nt * 2 * nuv;
-                    const int fL = tj * (TX + 1) + ti, fB = NFX + tj * TX + ti;
-                    const T* cp = cpn + ct * NCP;
-                    const V* k = reinterpret_cast<const V*>(cp + C_K);   // kself, -kE, kp1, kp0, -kdx, -kdy
-#pragma unroll
-                    for (int h = 0; h < VPL; ++h) {
-                        const T ex0 = __ldg(tb + iu[h]), ey0 = __ldg(tb + ivn[h]);
-                        const T ex1 = __ldg(tb + nuv + iu[h]), ey1 = __ldg(tb + nuv + ivn[h]);
-                        const V* Fh = F + (size_t)h * NFT * VB;
-                        const V dX = psub(Fh[(fL + 1) * VB], Fh[fL * VB]);
-                        const V dY = psub(Fh[(fB + TX) * VB], Fh[fB * VB]);
-                        V* fc = own + (size_t)(h * NCT + ct) * VB + lane;   // level m at fc[m * LVO]
-                        V e, f0;
-                        if constexpr (!IMP) {
-                            e = fc[n * LVO];                  // precomputed
-                            f0 = f0k[r][h];
-                        } else {
-                            switch (implicit ? 0 : nh) {
-                                case 0: e = etb[0]; break;
-                                case 1: e = spectral2<1>(fc, n, nt, LVO, etb); break;
-                                case 2: e = spectral2<2>(fc, n, nt, LVO, etb); break;
-                                case 3: e = spectral2<3>(fc, n, nt, LVO, etb); break;
-                                case 4: e = spectral2<4>(fc, n, nt, LVO, etb); break;
-                                case 5: e = spectral2<5>(fc, n, nt, LVO, etb); break;
-                                case 6: e = spectral2<6>(fc, n, nt, LVO, etb); break;
-                                default: e = spectral2<7>(fc, n, nt, LVO, etb); break;
-                            }
-                            f0 = fc[n * LVO];
-                        }
-                        // equilibria of W^{k+1} (slot 1) and W^k (slot 0), delta form
-                        const V q1 = eq2(cp + C_EQ1, ex1, ey1, href[h], u[h], v[h], r2[h], shakhov);
-                        const V q0 = eq2(cp + C_EQ0, ex0, ey0, href[h], u[h], v[h], r2[h], shakhov);
-                        V x = pmul(k[0], f0);
-                        x = pfma(k[4], dX, x);
-                        x = pfma(k[5], dY, x);
-                        x = pfma(k[1], e, x);
-                        x = pfma(k[2], q1, x);
-                        x = pfma(k[3], q0, x);
-                        if (implicit) fc[n * LVO] = x;       // right-hand side of level n; h^k no longer needed
-                        else on[h * bstride + (size_t)c * VB] = x;
-                    }
-                }
-            }
-            if (s < nt) {
-                // ---- pass 1, level s: reconstruction and downwind-face fluxes
-                const int n = s;
-                V* F = fbuf + (size_t)(n & 1) * L::FLUX + lane;
-                const V* rh = rect + (size_t)(n & 1) * L::RECT + lane;
-                const T* fpn = fps + (size_t)(n & 1) * L::FP;
-                const T* ftn = ftab + n * nuv;
-                int rfirst = 0;
-                if (PAIRED && interior) {
-                    // both tile cells of the warp, every block, as one straight-line block, stores last, so that
-                    // the independent chains interleave
-                    V fl[2][VPL][2];
-                    int sl[2][2];
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const int it = warp + q * NW, ti = it % TX, tj = it / TX;
-                        const int i = i0 + ti, j = j0 + tj;
-                        const int kx = ti - xlo, ky = tj - ylo;
-                        const int fix = xneg ? i : i + 1, fjy = yneg ? j : j + 1;
-                        sl[q][0] = tj * (TX + 1) + fix - i0;
-                        sl[q][1] = NFX + (fjy - j0) * TX + ti;
-                        const T* tbx = ftn + (j * (nx + 1) + fix) * NTf;
-                        const T* tby = ftn + (nfx + fjy * nx + i) * NTf;
-                        const T wxm = gxr[kx - 1], wxp = gxr[kx], wym = gyr[ky - 1], wyp = gyr[ky];
-                        const V hx = bc(xneg ? -gxh[kx] : gxh[kx]), hy = bc(yneg ? -gyh[ky] : gyh[ky]);
-#pragma unroll
-                        for (int h = 0; h < VPL; ++h) {
-                            const T exx = __ldg(tbx + iu[h]), eyx = __ldg(tbx + ivn[h]);
-                            const T exy = __ldg(tby + iu[h]), eyy = __ldg(tby + ivn[h]);
-                            const V* ph = rh + (size_t)(h * NR + ky * PX + kx) * VB;
-                            const V f0 = ph[0];
-                            f0k[q][h] = f0;
-                            const V sxv = slope2i(ph[-VB], f0, ph[VB], wxm, wxp);
-                            const V syv = slope2i(ph[-PX * VB], f0, ph[PX * VB], wym, wyp);
-                            const V dx0 = pfma(sxv, hx, f0);
-                            const V dy0 = pfma(syv, hy, f0);
-                            const V ub = bc(u[h]), vbb = bc(v[h]);
-                            fl[q][h][0] = flux2(fpn + sl[q][0] * NP, qoff, loff, exx, eyx, href[h], u[h], v[h], ub, vbb,
-                                                dx0, sxv, syv);
-                            fl[q][h][1] = flux2(fpn + sl[q][1] * NP, qoffy, loffy, exy, eyy, href[h], u[h], v[h], vbb,
-                                                ub, dy0, syv, sxv);
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < 2; ++q)
-#pragma unroll
-                        for (int h = 0; h < VPL; ++h) {
-                            F[(h * NFT + sl[q][0]) * VB] = fl[q][h][0];
-                            F[(h * NFT + sl[q][1]) * VB] = fl[q][h][1];
-                        }
-                    rfirst = 2;
-                }
-#pragma unroll
-                for (int r = 0; r < NPASS; ++r) {
-                    if (r < rfirst) continue;
-                    const int it = warp + r * NW;
-                    if (it >= NIT) break;
-                    int ti, tj;
-                    bool dox = true, doy = true;
-                    if ((r + 1) * NW <= NCT || it < NCT) {
-                        ti = it % TX; tj = it / TX;
-                        if (i0 + ti >= nx || j0 + tj >= ny) continue;
-                    } else if (it < NCT + TY) {
-                        tj = it - NCT; ti = xneg ? iend - i0 : -1; doy = false;
-                        if (j0 + tj >= ny) continue;
-                    } else {
-                        ti = it - NCT - TY; tj = yneg ? jend - j0 : -1; dox = false;
-                        if (i0 + ti >= nx) continue;
-                    }
-                    const int i = i0 + ti, j = j0 + tj;
-                    if (!interior && (i < 0 || i >= nx || j < 0 || j >= ny)) {
-                        // upwind face of the tile on a wall: the re-emitted distribution
-                        int slot;
-                        const T* wt;
-                        if (dox) {
-                            const int fi = i < 0 ? 0 : nx;
-                            slot = tj * (TX + 1) + fi - i0;
-                            wt = wtab + ((i < 0 ? 3 : 1) * cd.nslot + wall_slot(cd, n)) * nuv;
-                        } else {
-                            const int fj = j < 0 ? 0 : ny;
-                            slot = NFX + (fj - j0) * TX + ti;
-                            wt = wtab + ((j < 0 ? 0 : 2) * cd.nslot + wall_slot(cd, n)) * nuv;
-                        }
-#pragma unroll
-                        for (int h = 0; h < VPL; ++h)
-                            F[(h * NFT + slot) * VB] = flux_wall2(fpn + slot * NP, wt, iu[h], ivn[h], href[h],
-                                                                  bc(dox ? u[h] : v[h]));
-                        continue;
-                    }
-                    const int kx = ti - xlo, ky = tj - ylo;
-                    const int fix = xneg ? i : i + 1, fjy = yneg ? j : j + 1;
-                    const int slx = tj * (TX + 1) + fix - i0, sly = NFX + (fjy - j0) * TX + ti;
-                    const T* tbx = ftn + (j * (nx + 1) + fix) * NTf;
-                    const T* tby = ftn + (nfx + fjy * nx + i) * NTf;
-                    const T wxm = gxr[kx - 1], wxp = gxr[kx], wym = gyr[ky - 1], wyp = gyr[ky];
-#pragma unroll
-                    for (int h = 0; h < VPL; ++h) {
-                        // expm1 factors of the interface Maxwellians first: their latency overlaps the
-                        // reconstruction
-                        T exx = T(0), eyx = T(0), exy = T(0), eyy = T(0);
-                        if (dox) { exx = __ldg(tbx + iu[h]); eyx = __ldg(tbx + ivn[h]); }
-                        if (doy) { exy = __ldg(tby + iu[h]); eyy = __ldg(tby + ivn[h]); }
-                        const V* ph = rh + (size_t)(h * NR + ky * PX + kx) * VB;
-                        const V f0 = ph[0];
-                        if (r < NP2 && it < NCT) f0k[r][h] = f0;
-                        V sxv, syv;
-                        if (interior) {
-                            sxv = slope2i(ph[-VB], f0, ph[VB], wxm, wxp);
-                            syv = slope2i(ph[-PX * VB], f0, ph[PX * VB], wym, wyp);
-                        } else {
-                            sxv = slope2(ph[-VB], f0, ph[VB], wxm, wxp, i > 0, i < nx - 1, nx > 1);
-                            syv = slope2(ph[-PX * VB], f0, ph[PX * VB], wym, wyp, j > 0, j < ny - 1, ny > 1);
-                        }
-                        const V ub = bc(u[h]), vbb = bc(v[h]);
-                        if (dox) {
-                            const V d0 = pfma(sxv, bc(xneg ? -gxh[kx] : gxh[kx]), f0);
-                            F[(h * NFT + slx) * VB] = flux2(fpn + slx * NP, qoff, loff, exx, eyx, href[h], u[h], v[h],
-                                                            ub, vbb, d0, sxv, syv);
-                        }
-                        if (doy) {
-                            const V d0 = pfma(syv, bc(yneg ? -gyh[ky] : gyh[ky]), f0);
-                            F[(h * NFT + sly) * VB] = flux2(fpn + sly * NP, qoffy, loffy, exy, eyy, href[h], u[h],
-                                                            v[h], vbb, ub, d0, syv, sxv);
-                        }
-                    }
-                }
-            }
-        }
-        // one barrier per level: it publishes this level's fluxes, frees the ring slots read here, and makes
-        // the CTA agree on a failed wait
-        if (__syncthreads_or(fail)) {
-            // warp 0, which issued them, waits (bounded) for batches s and s + 1, so that no bulk copy still
-            // lands in shared memory after the CTA exits
-            if (threadIdx.x == 0 && expire) atomicExch(err, 1);
-            if (warp == 0) {
-                mbar_drain(&bars[s & 1], (uint32_t)((s >> 1) & 1));
-                if (s < nt) mbar_drain(&bars[(s + 1) & 1], (uint32_t)(((s + 1) >> 1) & 1));
-            }
-            return;
-        }
-    }
-    if (implicit) {
-        // spectral source at the new iterate: f^{k+1} = minv (right-hand sides over the levels), per cell, block
-        // and lane
-        for (int ct = warp; ct < NCT; ct += NW) {
-            const int ti = ct % TX, tj = ct / TX;
-            const int i = i0 + ti, j = j0 + tj;
-            if (i >= nx || j >= ny) continue;
-            const int c = j * nx + i;
-            const T* Mi = cd.minv + (size_t)c * nt * nt;
-#pragma unroll
-            for (int h = 0; h < VPL; ++h) {
-                const V* fc = own + (size_t)(h * NCT + ct) * VB + lane;
-                V rr[MAXNT];
-#pragma unroll
-                for (int m = 0; m < MAXNT; ++m) rr[m] = m < nt ? fc[m * LVO] : bc(T(0));
-                V* o = cd.f[p ^ 1] + (vb + h) * bstride + (size_t)c * VB + lane;
-#pragma unroll
-                for (int n = 0; n < MAXNT; ++n) {
-                    if (n >= nt) break;
-                    V acc = bc(T(0));
-#pragma unroll
-                    for (int m = 0; m < MAXNT; ++m)
-                        if (m < nt) acc = pfma(bc(__ldg(Mi + n * nt + m)), rr[m], acc);
-                    o[(size_t)n * nc * VB] = acc;
-                }
-            }
-        }
-    }
-}
-
-template <typename T, int TX, int TY, int VPL>
-constexpr size_t k4_cells_smem(int nt)
-{
-    return K4Layout<T, TX, TY, VPL>::bytes(nt);
 }
 
 }  // namespace hb

@@ -124,7 +124,7 @@ struct CaseDev {
     T* fpar;                           // [nt][nf][NP]
     T* ftab;                           // [nf][nt][nu + nv]   expm1 factors of the interface Maxwellian
     T* wtab;                           // [4][nslot][nu + nv]  expm1 factors of each wall's Maxwellian
-    T* ctab;                           // [nc][nt][2][nu + nv] expm1 factors of the cell equilibria (W^k, W^{k+1})
+    T* ctab;                           // [nc][nt][nu + nv][2] expm1 factors of the cell equilibria (W^k, W^{k+1})
     const int* viu;                    // per stored velocity: u index (0 for padding)
     const int* viv;                    // per stored velocity: v index
     const int* vcan;                   // per stored velocity: canonical index jv * nu + iu, -1 for padding

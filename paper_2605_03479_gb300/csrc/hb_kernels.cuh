@@ -650,15 +650,18 @@ __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
     }
     __syncthreads();
     // tables of expm1(lam0 x^2 - lam (x - U)^2) over the 1-D velocity nodes, so that for a Maxwellian of density rho:
-    // H - H_ref = H_ref [(r - 1) + r (ex + ey + ex ey)], r = rho lam / lam0.  The CTA's rows are consecutive in memory.
-    const int nuv = cd.nu + cd.nv, rows = min(K3_CELLS, nc - lb * K3_CELLS) * nt * 2;
-    T* dst = cd.ctab + (size_t)lb * K3_CELLS * nt * 2 * nuv;
+    // H - H_ref = H_ref [(r - 1) + r (ex + ey + ex ey)], r = rho lam / lam0.  The entries of W^k and W^{k+1} lie side by
+    // side (one load gives both); the CTA's rows are consecutive in memory.
+    const int nuv = cd.nu + cd.nv, rows = min(K3_CELLS, nc - lb * K3_CELLS) * nt;
+    P2<T>* dst = reinterpret_cast<P2<T>*>(cd.ctab) + (size_t)lb * K3_CELLS * nt * nuv;
     int row = (int)threadIdx.x / nuv, k = (int)threadIdx.x - row * nuv;
     for (int q = threadIdx.x; row < rows; q += blockDim.x) {
-        const T* e = coef[row];
+        const T* e = coef[2 * row];
+        const T* e1 = coef[2 * row + 1];
         const bool isu = k < cd.nu;
         const T x = isu ? cd.tu1[k] : cd.tv1[k - cd.nu];
-        dst[q] = t_expm1<T>(e[0] * x * x + (isu ? e[1] : e[3]) * x - (isu ? e[2] : e[4]));
+        dst[q] = pk(t_expm1<T>(e[0] * x * x + (isu ? e[1] : e[3]) * x - (isu ? e[2] : e[4])),
+                    t_expm1<T>(e1[0] * x * x + (isu ? e1[1] : e1[3]) * x - (isu ? e1[2] : e1[4])));
         k += blockDim.x;
         while (k >= nuv) { k -= nuv; ++row; }
     }
