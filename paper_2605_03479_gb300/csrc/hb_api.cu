@@ -293,9 +293,19 @@ void fill_host(HostCase& h, const hbugks_case& c)
             o[1] = W.v_mean + W.v_re * cs - W.v_im * sn;
             o[2] = W.T_mean + W.T_re * cs - W.T_im * sn;   // Eq. bc_temp
         }
-    h.k2b = (h.nf * h.nt + 127) / 128;
+    h.k2b = (h.nf * h.nt + K2_ITEMS - 1) / K2_ITEMS;
     h.k3b = (h.nc + K3_CELLS - 1) / K3_CELLS;
     h.ksb = (h.nc + 127) / 128;
+}
+
+// indices of 1-D nodes ordered by class: positive, negative, zero
+std::vector<int> class_order(const std::vector<double>& x)
+{
+    std::vector<int> o;
+    for (int c = 0; c < 3; ++c)
+        for (int k = 0; k < (int)x.size(); ++k)
+            if ((c == 0 && x[k] > 0) || (c == 1 && x[k] < 0) || (c == 2 && x[k] == 0)) o.push_back(k);
+    return o;
 }
 
 template <typename T>
@@ -333,6 +343,13 @@ void layout_case(Carver& cv, const HostCase& h, CaseDev<T>& d)
     d.u1 = cv.take<double>(h.nu); d.wu1 = cv.take<double>(h.nu);
     d.v1 = cv.take<double>(h.nv); d.wv1 = cv.take<double>(h.nv);
     d.tu1 = cv.take<T>(h.nu); d.tv1 = cv.take<T>(h.nv);
+    d.su1 = cv.take<T>(h.nu); d.sv1 = cv.take<T>(h.nv);
+    d.ou1 = cv.take<int>(h.nu); d.ov1 = cv.take<int>(h.nv);
+    for (int a = 0; a < 2; ++a) {
+        const std::vector<double>& x = a == 0 ? h.u : h.v;
+        d.ncls[a][0] = (int)std::count_if(x.begin(), x.end(), [](double z) { return z > 0; });
+        d.ncls[a][1] = d.ncls[a][0] + (int)std::count_if(x.begin(), x.end(), [](double z) { return z < 0; });
+    }
     d.refmom = cv.take<double>(5 * 13);
     const size_t ns = (size_t)h.nvb * h.nc * h.nt * VB;
     for (int k = 0; k < 2; ++k) {
@@ -359,6 +376,7 @@ void layout_case(Carver& cv, const HostCase& h, CaseDev<T>& d)
     d.vcan = cv.take<int>(h.nvp);
     d.vcls = cv.take<int>(h.nvb);
     d.shakhov = h.src.phys.pr != 1.0;
+    d.zeros = std::find(h.u.begin(), h.u.end(), 0.0) != h.u.end() || std::find(h.v.begin(), h.v.end(), 0.0) != h.v.end();
     d.fflux = cv.take<double>((size_t)h.nf * h.nt * 4);
     d.cpar = cv.take<T>((size_t)h.nc * h.nt * NCP);
     d.rpart = cv.take<double>((size_t)h.k3b * 4);
@@ -641,18 +659,25 @@ cudaError_t upload_case(const HostCase& h, const CaseDev<T>& d, cudaStream_t s, 
     std::vector<T> wxr((size_t)9 * h.nu), wyr((size_t)9 * h.nv);
     std::vector<double> xr0(36, 0.0), yr0(36, 0.0);
     std::vector<T> xr0t(36), yr0t(36);
-    for (int k = 0; k < h.nu; ++k) {
-        const double x = h.u[k], g = h.wu[k] * exp(-x * x);
-        const int row = x > 0 ? 1 : (x < 0 ? 2 : 3);
-        double pw = g;
-        for (int q = 0; q < 9; ++q) { wxr[(size_t)q * h.nu + k] = T(pw); xr0[row * 9 + q] += pw; xr0[q] += pw; pw *= x; }
-    }
-    for (int k = 0; k < h.nv; ++k) {
-        const double y = h.v[k], g = h.wv[k] * exp(-y * y);
-        const int row = y > 0 ? 1 : (y < 0 ? 2 : 3);
-        double pw = g;
-        for (int q = 0; q < 9; ++q) { wyr[(size_t)q * h.nv + k] = T(pw); yr0[row * 9 + q] += pw; yr0[q] += pw; pw *= y; }
-    }
+    auto ref_sums = [](const std::vector<double>& x, const std::vector<double>& w, const std::vector<int>& ord,
+                       std::vector<T>& wr, std::vector<double>& r0) {
+        for (size_t k = 0; k < x.size(); ++k) {
+            const double z = x[ord[k]];
+            const int row = z > 0 ? 1 : (z < 0 ? 2 : 3);
+            double pw = w[ord[k]] * exp(-z * z);
+            for (int q = 0; q < 9; ++q) { wr[q * x.size() + k] = T(pw); r0[row * 9 + q] += pw; r0[q] += pw; pw *= z; }
+        }
+    };
+    const std::vector<int> ou = class_order(h.u), ov = class_order(h.v);
+    ref_sums(h.u, h.wu, ou, wxr, xr0);
+    ref_sums(h.v, h.wv, ov, wyr, yr0);
+    std::vector<T> su1(h.nu), sv1(h.nv);
+    for (int k = 0; k < h.nu; ++k) su1[k] = T(h.u[ou[k]]);
+    for (int k = 0; k < h.nv; ++k) sv1[k] = T(h.v[ov[k]]);
+    if ((e = put(d.su1, su1.data(), sizeof(T) * h.nu))) return e;
+    if ((e = put(d.sv1, sv1.data(), sizeof(T) * h.nv))) return e;
+    if ((e = put(d.ou1, ou.data(), sizeof(int) * h.nu))) return e;
+    if ((e = put(d.ov1, ov.data(), sizeof(int) * h.nv))) return e;
     for (int k = 0; k < 36; ++k) { xr0t[k] = T(xr0[k]); yr0t[k] = T(yr0[k]); }
     if ((e = put(d.wxr, wxr.data(), sizeof(T) * wxr.size()))) return e;
     if ((e = put(d.wyr, wyr.data(), sizeof(T) * wyr.size()))) return e;
@@ -790,7 +815,7 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
         Range r(names[sp.kind]);
         switch (sp.kind) {
             case 0: launch_k1<T>(sp.shape, sp.total, sp.smem, b, s); break;
-            case 1: k2_face_params<T><<<sp.total, 128, 0, s>>>(b); break;
+            case 1: k2_face_params<T><<<sp.total, K2_ITEMS * K2_WARPS, 0, s>>>(b); break;
             case 2: {
                 Range rt("k_tables");          // the same launch writes the equilibrium tables
                 k3_macro<T><<<sp.total, k3_threads(im.max_nt), 0, s>>>(b);

@@ -111,7 +111,10 @@ struct CaseDev {
     const double *u1, *wu1, *v1, *wv1; // 1-D grids
     const T *tu1, *tv1;                // 1-D nodes in the storage precision
     const double* refmom;              // [5][13]: full, u>0, u<0, v>0, v<0 moments of (H_ref, B_ref)
-    const T *wxr, *wyr;                // [9][nu], [9][nv]: w x^p exp(-lam0 x^2) per 1-D node
+    const T *su1, *sv1;                // the same ordered by class: positive, negative, zero nodes
+    const int *ou1, *ov1;              // their places in tu1, tv1
+    int ncls[2][2];                    // per axis: one past the last positive and the last negative node in that order
+    const T *wxr, *wyr;                // [9][nu], [9][nv]: w x^p exp(-lam0 x^2) per 1-D node, in that order
     const double *xr0, *yr0;           // [4][9]: sums of the above over all / positive / negative / zero nodes
     const T *xr0t, *yr0t;              // the same in the storage precision
     const double* wconst;              // [4][nslot][WCN] reflected-half constants of each wall Maxwellian
@@ -131,6 +134,7 @@ struct CaseDev {
     const int* vcls;                   // per velocity block: sign class (bit 0: u < 0, bit 1: v < 0)
     int cls_end[4];                    // one past the last block of sign classes 0..c (classes are consecutive)
     int shakhov;                       // Pr != 1
+    int zeros;                         // the velocity grid has a zero node
     double* fflux;                     // [nf][nt][4]
     T* cpar;                           // [nt][nc][NCP]
     double* rpart;                     // [k3 blocks][4]
@@ -337,12 +341,12 @@ __device__ __noinline__ void ugks_coeffs(P dG, P tau, P C[5])
     }
 }
 
-// Coefficients a of (a.psi) g whose moments per unit density are w (continuous Maxwellian, K = 1).
-__device__ __forceinline__ void micro_slope(const double w[4], double U, double V, double lam, double a[4])
+// Coefficients a of (a.psi) g whose moments per unit density are w (continuous Maxwellian, K = 1); i2l = 1/(2 lam).
+__device__ __forceinline__ void micro_slope(const double w[4], double U, double V, double lam, double i2l, double a[4])
 {
     double R2 = w[1] - U * w[0];
     double R3 = w[2] - V * w[0];
-    double e = U * U + V * V + 1.5 / lam;
+    double e = U * U + V * V + 3.0 * i2l;
     double R4 = 2.0 * w[3] - e * w[0];
     a[3] = (4.0 / 3.0) * lam * lam * (R4 - 2.0 * U * R2 - 2.0 * V * R3);
     a[2] = 2.0 * lam * R3 - V * a[3];
@@ -409,93 +413,5 @@ __device__ __forceinline__ T cubic(const T* c, T u, T v)
 // Discrete sums of polynomial x Maxwellian over the tensor velocity grid factor into 1-D sums
 //   X[p] = sum_i wu_i u_i^p exp(-lam (u_i - U)^2)  (over u_i > 0, u_i < 0, u_i = 0 or all),
 //   Y[q] likewise in v,  so  sum_a w_a u^p v^q rho (lam/pi) e^{-lam |u - U|^2} = rho lam/pi X[p] Y[q].
-
-template <typename P>
-struct SumsT {
-    P s[4][9];   // [0] all, [1] positive nodes, [2] negative nodes, [3] zero nodes; powers 0..8
-};
-
-// polynomial in (u, v) of total degree <= 4
-template <typename P>
-struct PolyT {
-    P c[5][5];
-    __device__ void zero()
-    {
-#pragma unroll
-        for (int p = 0; p < 5; ++p)
-#pragma unroll
-            for (int q = 0; q < 5; ++q) c[p][q] = P(0);
-    }
-};
-
-// C = u A (dir 0) or v A (dir 1), truncated at total degree 4: every product in the face parameters has a
-// monomial u_n or u_t as one factor, so it shifts the coefficients by one power
-template <typename P>
-__device__ __forceinline__ void poly_shift(int dir, const PolyT<P>& A, PolyT<P>& C)
-{
-    C.zero();
-    if (dir == 0) {
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-            for (int q = 0; q < 4 - p; ++q)
-                if (A.c[p][q] != P(0)) C.c[p + 1][q] = A.c[p][q];
-    } else {
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-            for (int q = 0; q < 4 - p; ++q)
-                if (A.c[p][q] != P(0)) C.c[p][q + 1] = A.c[p][q];
-    }
-}
-
-// P_h(a) = a0 + a1 u + a2 v + a3/2 (u^2 + v^2 + 1/(2 lam)),  P_b(a) = P_h(a) + a3/(2 lam)
-template <typename P>
-__device__ inline void poly_P(const double* a, double i2l, bool for_b, PolyT<P>& out)
-{
-    out.zero();
-    out.c[0][0] = P(a[0] + 0.5 * a[3] * i2l + (for_b ? a[3] * i2l : 0.0));
-    out.c[1][0] = P(a[1]);
-    out.c[0][1] = P(a[2]);
-    out.c[2][0] = P(0.5 * a[3]);
-    out.c[0][2] = P(0.5 * a[3]);
-}
-
-// moments sum w psi [Q H ; R B] over the grid part selected by (rx, ry), H = pref e^{..}, B = H i2l:
-//   (sum Q H, sum u Q H, sum v Q H, 1/2 sum (|u|^2 Q H + R B)).  The selected rows of the 1-D sums are copied
-// through constant indices first, so that everything stays in registers.
-template <typename P>
-__device__ __forceinline__ void sum_row(const SumsT<P>& X, int r, P (&o)[9])
-{
-#pragma unroll
-    for (int q = 0; q < 9; ++q) o[q] = r == 0 ? X.s[0][q] : r == 1 ? X.s[1][q] : r == 2 ? X.s[2][q] : X.s[3][q];
-}
-
-template <typename P>
-__device__ __forceinline__ void mom4(const PolyT<P>& Q, const PolyT<P>& R, const SumsT<P>& X, int rx, const SumsT<P>& Y,
-                                     int ry, P pref, P i2l, P out[4])
-{
-    P xr[9], yr[9];
-    sum_row(X, rx, xr);
-    sum_row(Y, ry, yr);
-    P o0 = 0, o1 = 0, o2 = 0, o3 = 0, ob = 0;
-#pragma unroll
-    for (int p = 0; p < 5; ++p)
-#pragma unroll
-        for (int q = 0; q < 5 - p; ++q) {
-            const P a = Q.c[p][q], r = R.c[p][q];
-            if (a != P(0)) {
-                o0 += a * xr[p] * yr[q];
-                o1 += a * xr[p + 1] * yr[q];
-                o2 += a * xr[p] * yr[q + 1];
-                o3 += a * (xr[p + 2] * yr[q] + xr[p] * yr[q + 2]);
-            }
-            if (r != P(0)) ob += r * xr[p] * yr[q];
-        }
-    out[0] = pref * o0;
-    out[1] = pref * o1;
-    out[2] = pref * o2;
-    out[3] = P(0.5) * pref * (o3 + i2l * ob);
-}
 
 }  // namespace hb

@@ -70,348 +70,422 @@ __device__ __forceinline__ void heat_flux_raw(const double* A, double U, double 
 
 // ------------------------------------------------------------------------------ K2 face parameters
 
-// delta-form velocity sum sum_a w_a u^p v^q (H0 - H_ref) over the subset given by the rows (rx, ry), from the
-// reference 1-D sums X0, Y0 (FP64) and the table sums dX, dY = sum w x^p e^{-lam0 x^2} expm1(..):
-//   (lam0/pi) [(r - 1) X0 Y0 + r (dX Y0 + X0 dY + dX dY)]
-template <typename T>
-__device__ __forceinline__ double dsum(const double* X0, const double* Y0, const SumsT<T>& dX, const SumsT<T>& dY,
-                                       int rx, int ry, int p, int q, double r, double lam0)
+// A CTA takes K2_ITEMS (face, level) items with one lane each in every one of its four warps, which divide the work:
+//   A  interface state from the velocity sums (each warp for itself), then warp 0 the heat flux and Shakhov factor,
+//      1 and 2 the slopes a^L and a^R, 3 the slope a_t, the relaxation time and the weights C1..C5;
+//   B  all warps: the expm1 table of the interface Maxwellian (lanes over the nodes, one item after another) and its
+//      27 sums per axis (lanes over the items, a warp per power);
+//   C  warp 0 the compatibility condition (A), 1 the Shakhov moments, 2 and 3 the moments of the left and right slopes;
+//   D  warp 0 the macro flux and the wall density, 1 and 2 the micro-flux parameters of the two upwind sides, 3 the rest.
+// On small meshes the time is the chain of one thread, in large ones FP64 instructions and latency at few warps.
+// Against one thread per item doing all of it (219 registers, nine FP64 instructions per division, polynomials in (u, v)
+// whose axis was known at run time only): 57 -> 29 us (8x8, N_T 3), 0.210 -> 0.139 ms (64x64, 48x48, N_T 7),
+// 5.49 -> 3.94 ms (48 uneven cavities), 1.12 -> 0.70 ms (128x128, 64x64, N_T 11); FP64 0.190 -> 0.078 ms (32x32, 24x24)
+// and 2.97 -> 2.03 ms (twelve 64x64, 32x32).  32 items fill a warp; 4 warps balance the parts of A and C.
+constexpr int K2_ITEMS = 32, K2_WARPS = 4, K2_NODES = 32;
+
+// All polynomials are kept in the face's own velocity components, n along its normal and t along the other axis, in
+// the order 1, n, t, n^2, nt, t^2, n^3, n^2 t, n t^2, t^3, so that a product by u_n is a shift of the 1-D sums by one
+// power and every pattern of zero coefficients is known when compiling.
+
+// place of coefficient k (0..9 a cubic, 10..12 a linear form) after exchanging the two components
+__device__ __forceinline__ constexpr int nt_order(int k)
 {
-    const double x0 = X0[rx * 9 + p], y0 = Y0[ry * 9 + q];
-    const double dx = (double)dX.s[rx][p], dy = (double)dY.s[ry][q];
-    return lam0 / M_PI * ((r - 1.0) * x0 * y0 + r * (dx * y0 + x0 * dy + dx * dy));
+    constexpr int o[13] = {0, 2, 1, 5, 4, 3, 9, 8, 7, 6, 10, 12, 11};
+    return o[k];
 }
 
-// Velocity sums of the upwinded reconstruction at face g, level n, from the half-face sums of its cells: at an
-// interior face the low-side cell's u_n > 0 class plus the high-side cell's u_n < 0 class; at a wall the
-// interior cell's class moving into the wall, with the tangential-slope sums (13..17) over both classes.
+// P_h(a) = a0 + a1 u + a2 v + a3/2 (u^2 + v^2 + 1/(2 lam)) of a slope and P_b(a) = P_h(a) + a3/(2 lam): constant term,
+// the addition for b, then the coefficients of n, t and n^2 (= that of t^2)
 template <typename T>
-__device__ __forceinline__ void face_sums(const CaseDev<T>& cd, const FaceGeo& g, int n, double* m)
+__device__ __forceinline__ void slope_poly(const double w[4], double U, double V, double lam, double i2l, int ax,
+                                           T (*o)[K2_ITEMS], int lane)
 {
-    const int sp = g.axis == 0 ? 0 : 2;                  // half-face slot of the u_n > 0 class, sp + 1: u_n < 0
-    const size_t stride = (size_t)cd.nt * 4 * NM;
-    const double* L = g.hasL ? cd.hmom + (size_t)(g.jL * cd.nx + g.iL) * stride + (size_t)n * 4 * NM : nullptr;
-    const double* R = g.hasR ? cd.hmom + (size_t)(g.jR * cd.nx + g.iR) * stride + (size_t)n * 4 * NM : nullptr;
-    if (g.hasL && g.hasR) {
-        for (int k = 0; k < NM; ++k) m[k] = L[sp * NM + k] + R[(sp + 1) * NM + k];
-    } else if (g.hasR) {
-        for (int k = 0; k < NM; ++k) m[k] = R[(sp + 1) * NM + k];
-        for (int k = 13; k < 18; ++k) m[k] += R[sp * NM + k];
-    } else {
-        for (int k = 0; k < NM; ++k) m[k] = L[sp * NM + k];
-        for (int k = 13; k < 18; ++k) m[k] += L[(sp + 1) * NM + k];
+    double a[4];
+    micro_slope(w, U, V, lam, i2l, a);
+    o[0][lane] = T(a[0] + 0.5 * a[3] * i2l);
+    o[1][lane] = T(a[3] * i2l);
+    o[2][lane] = T(ax == 0 ? a[1] : a[2]);
+    o[3][lane] = T(ax == 0 ? a[2] : a[1]);
+    o[4][lane] = T(0.5 * a[3]);
+}
+
+// cubic Q = u_n P_h(a_side) + u_t P_h(a_t); dn, dt: the additions to its coefficients of n and t for b
+template <typename T>
+__device__ __forceinline__ void side_poly(const T (*ps)[K2_ITEMS], const T (*pt)[K2_ITEMS], int lane, T (&c)[10], T& dn, T& dt)
+{
+    c[0] = T(0);
+    c[1] = ps[0][lane];
+    c[2] = pt[0][lane];
+    c[3] = ps[2][lane];
+    c[4] = ps[3][lane] + pt[2][lane];
+    c[5] = pt[3][lane];
+    c[6] = c[8] = ps[4][lane];
+    c[7] = c[9] = pt[4][lane];
+    dn = ps[1][lane];
+    dt = pt[1][lane];
+}
+
+// moments sum w psi [Q H ; R B] of the cubic c (CUB false: without nt and the cubic terms) times u_n^S, R = c + d0 +
+// dn n + dt t, with the 1-D sums x along the normal and y along t of the selected grid part, H = pref e^{..}, B = H i2l:
+// (sum Q H, sum u_n Q H, sum u_t Q H, 1/2 sum (|u|^2 Q H + R B)).  The inner sums over powers of n serve every moment.
+template <int S, bool CUB, typename P>
+__device__ __forceinline__ void mom4(const P (&c)[10], P d0, P dn, P dt, const P (&x)[9], const P (&y)[9], P pref, P i2l,
+                                     P (&out)[4])
+{
+    P m[3][3];                                               // [power added to n][power added to t]
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        const P *v = x + S + z;
+        P t[4];
+        t[0] = c[0] * v[0] + c[1] * v[1] + c[3] * v[2];
+        t[1] = c[2] * v[0];
+        t[2] = c[5] * v[0];
+        t[3] = P(0);
+        if (CUB) {
+            t[0] += c[6] * v[3];
+            t[1] += c[4] * v[1] + c[7] * v[2];
+            t[2] += c[8] * v[1];
+            t[3] = c[9] * v[0];
+        }
+#pragma unroll
+        for (int k = 0; k + z < 3; ++k) {
+            m[z][k] = t[0] * y[k] + t[1] * y[k + 1] + t[2] * y[k + 2];
+            if (CUB) m[z][k] += t[3] * y[k + 3];
+        }
     }
+    const P ob = m[0][0] + (d0 * x[S] + dn * x[S + 1]) * y[0] + dt * x[S] * y[1];
+    out[0] = pref * m[0][0];
+    out[1] = pref * m[1][0];
+    out[2] = pref * m[0][1];
+    out[3] = P(0.5) * pref * (m[2][0] + m[0][2] + i2l * ob);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(128) k2_face_params(Batch<T> B)
+__global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B)
 {
-    int cs = find_case(B.off, B.ncases, blockIdx.x);
+    const int cs = find_case(B.off, B.ncases, blockIdx.x);
     const CaseDev<T>& cd = B.cases[cs];
+    // uniform over the CTA: neither word changes while this kernel runs
     if (!cd.st->active || *(volatile int*)cd.err) return;
-    const int item = (blockIdx.x - B.off[cs]) * blockDim.x + threadIdx.x;
-    const int nt = cd.nt;
-    if (item >= cd.nf * nt) return;
+    __shared__ T pL[5][K2_ITEMS], pR[5][K2_ITEMS], pt[5][K2_ITEMS], pA[5][K2_ITEMS], shk_[13][K2_ITEMS], Cw[5][K2_ITEMS];
+    __shared__ T tco[5][K2_ITEMS];                           // exponent coefficients of the table
+    __shared__ T S[2][3][9][K2_ITEMS];                       // table sums per axis, node class (> 0, < 0, 0) and power
+    __shared__ T se[K2_NODES][K2_ITEMS + 1];
+    __shared__ T F1s[4][K2_ITEMS], F2L[4][K2_ITEMS], F2R[4][K2_ITEMS];
+    __shared__ double dF1[4][K2_ITEMS], sdG[K2_ITEMS], st[10][K2_ITEMS];
+    const int nt = cd.nt, nu = cd.nu, nv = cd.nv, nuv = nu + nv, nitems = cd.nf * nt;
+    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+    const int base = (blockIdx.x - B.off[cs]) * K2_ITEMS;
+    const bool valid = base + lane < nitems;
+    const int item = valid ? base + lane : nitems - 1;       // lanes past the end repeat the last item and store nothing
     const int f = item / nt, n = item - f * nt;
     const FaceGeo g = face_geo(cd, f);
-    const int p = cd.st->parity;
-    const double* W = cd.W[p];
-    double m[NM];                                        // velocity sums of the reconstructed deviations
-    face_sums(cd, g, n, m);
+    const int ax = g.axis;
+    const double* W = cd.W[cd.st->parity];
     const bool wall = !(g.hasL && g.hasR);
     const double nin = wall ? (g.hasL ? -1.0 : 1.0) : 0.0;
-    const int ax = g.axis;
-    const int inc_row = nin > 0 ? 2 : 1;      // incident: u_n nin < 0
-    int refset = 0;
-    if (wall) refset = ax == 0 ? (nin > 0 ? 2 : 1) : (nin > 0 ? 4 : 3);
-    double A[13];
-#pragma unroll
-    for (int k = 0; k < 13; ++k) A[k] = m[k] + cd.refmom[refset * 13 + k];
-
-    // ---- diffuse wall: free-transport density estimate (Eq. rho_wall) and the mixed kinetic average
+    const int inc_row = nin > 0 ? 2 : 1;                     // incident: u_n nin < 0
+    const int refset = !wall ? 0 : ax == 0 ? (nin > 0 ? 2 : 1) : (nin > 0 ? 4 : 3);
     const int wsl = wall_slot(cd, n);
     const double* wc = wall ? cd.wconst + ((size_t)g.wall * cd.nslot + wsl) * WCN : nullptr;
-    double Amix[13], Dw = 1.0, rhow0 = 0.0;
-#pragma unroll
-    for (int k = 0; k < 13; ++k) Amix[k] = A[k];
-    if (wall) {
-        Dw = wc[13];                                        // sum over reflected velocities of w |u_n| H_w
-        rhow0 = -nin * (ax == 0 ? A[1] : A[2]) / Dw;
-#pragma unroll
-        for (int k = 0; k < 13; ++k) Amix[k] = A[k] + rhow0 * wc[k];
-    }
-
-    // ---- interface Maxwellian from the kinetic average, heat flux, relaxation time
-    double W0[4] = {Amix[0], Amix[1], Amix[2], 0.5 * (Amix[3] + Amix[5] + Amix[10])};
-    double rho0, U0, V0, lamf;
-    prim(W0, rho0, U0, V0, lamf);
-    double q0x, q0y;
-    heat_flux_raw(Amix, U0, V0, q0x, q0y);
-    const double tau = relax_time(cd.mu0, cd.w_vss, rcp64(cd.lam0), rcp64(rho0), lamf);
-
-    // ---- face step (Eq. dt_face) and time-integration weights (Eq. C_coeffs)
     const int cL = g.jL * cd.nx + g.iL, cR = g.jR * cd.nx + g.iR;
-    double dGf;
-    if (!g.hasL) dGf = cd.dG[cR];
-    else if (!g.hasR) dGf = cd.dG[cL];
-    else if (cd.face_step == 1) dGf = 2.0 * cd.dG[cL] * cd.dG[cR] / (cd.dG[cL] + cd.dG[cR]);
-    else dGf = fmin(cd.dG[cL], cd.dG[cR]);
-    T Ct[5];
-    ugks_coeffs<T>(T(dGf), T(tau), Ct);
-    double C[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) C[k] = (double)Ct[k];
+    // Velocity sums of the upwinded reconstruction from the half-face sums of the face's cells: at an interior face the
+    // low-side cell's u_n > 0 class plus the high-side cell's u_n < 0 class; at a wall the interior cell's class moving
+    // into the wall, with the tangential-slope sums (13..17) over both classes.
+    const int sp = ax == 0 ? 0 : 2;                          // half-face slot of the u_n > 0 class, sp + 1: u_n < 0
+    const double* hL = g.hasL ? cd.hmom + ((size_t)cL * nt + n) * 4 * NM + sp * NM : nullptr;
+    const double* hR = g.hasR ? cd.hmom + ((size_t)cR * nt + n) * 4 * NM + (sp + 1) * NM : nullptr;
+    const double* ha = g.hasL ? hL : hR;
+    const double* hb = wall ? (g.hasL ? hL + NM : hR - NM) : hR;   // at a wall: the other class
+    auto msum = [&](int k) { return ha[k] + (!wall || (k >= 13 && k < 18) ? hb[k] : 0.0); };
 
-    // ---- equilibrium slopes a^L, a^R (normal), a_t (tangential)
-    double aL[4], aR[4], at[4], Aa[4], w[4];
-    if (g.hasL) {
-        const double* WL = W + ((size_t)n * cd.nc + cL) * 4;
-        const double d = ax == 0 ? cd.hx[g.iL] : cd.hy[g.jL];
+    // ---- A: interface Maxwellian from the kinetic average; diffuse wall: its mixed with the free-transport estimate
+    // of the re-emitted distribution (Eq. rho_wall)
+    auto amix = [&](int k, double rhow0) {
+        const double a = msum(k) + cd.refmom[refset * 13 + k];
+        return wall ? fma(rhow0, wc[k], a) : a;
+    };
+    if (role == 0) {
+        double rhow0 = 0.0;
+        if (wall) rhow0 = -nin * (msum(ax == 0 ? 1 : 2) + cd.refmom[refset * 13 + (ax == 0 ? 1 : 2)]) * rcp64(wc[13]);
+        const double w[4] = {amix(0, rhow0), amix(1, rhow0), amix(2, rhow0),
+                             0.5 * (amix(3, rhow0) + amix(5, rhow0) + amix(10, rhow0))};
+        double r, a, b, l;
+        prim(w, r, a, b, l);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) w[k] = (W0[k] - WL[k]) / d / rho0;
-        micro_slope(w, U0, V0, lamf, aL);
+        for (int k = 0; k < 4; ++k) st[k][lane] = w[k];
+        st[4][lane] = a;
+        st[5][lane] = b;
+        st[6][lane] = l;
+        st[7][lane] = rcp64(r);
+        st[8][lane] = 0.5 * rcp64(l);
+        st[9][lane] = rhow0;
     }
-    if (g.hasR) {
-        const double* WR = W + ((size_t)n * cd.nc + cR) * 4;
-        const double d = ax == 0 ? cd.hx[g.iR] : cd.hy[g.jR];
+    __syncthreads();
+    const double rho0 = st[0][lane], U0 = st[4][lane], V0 = st[5][lane], lamf = st[6][lane], ir = st[7][lane],
+                 i2ld = st[8][lane], il0 = rcp64(cd.lam0);
+    if (role == 0) {
+        double Am[13], q0x, q0y, sh[13];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) w[k] = (WR[k] - W0[k]) / d / rho0;
-        micro_slope(w, U0, V0, lamf, aR);
-    }
-    if (!g.hasL) {
+        for (int k = 0; k < 13; ++k) Am[k] = amix(k, st[9][lane]);
+        heat_flux_raw(Am, U0, V0, q0x, q0y);
+        // Shakhov factor s (c.q)(2 lam |c|^2 - 4) and the b-part addition 2 s (c.q)
+        shakhov_poly((1.0 - cd.pr) * 0.8 * lamf * lamf * ir, q0x, q0y, U0, V0, lamf, sh);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) aL[k] = aR[k];
-    }
-    if (!g.hasR) {
+        for (int k = 0; k < 13; ++k) shk_[ax == 0 ? k : nt_order(k)][lane] = T(sh[k]);
+    } else if (role < 3) {
+        // equilibrium slopes a^L, a^R (normal); a wall face has the interior side's in both
+        const bool low = role == 1 ? g.hasL : !g.hasR;
+        const double* Wc = W + ((size_t)n * cd.nc + (low ? cL : cR)) * 4;
+        const double d = ax == 0 ? cd.hx[low ? g.iL : g.iR] : cd.hy[low ? g.jL : g.jR];
+        const double s = (low ? ir : -ir) * rcp64(d);
+        double w[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) aR[k] = aL[k];
+        for (int k = 0; k < 4; ++k) w[k] = (st[k][lane] - Wc[k]) * s;
+        slope_poly<T>(w, U0, V0, lamf, i2ld, ax, role == 1 ? pL : pR, lane);
+    } else {
+        const double w[4] = {msum(13) * ir, msum(14) * ir, msum(15) * ir, 0.5 * (msum(16) + msum(17)) * ir};
+        slope_poly<T>(w, U0, V0, lamf, i2ld, ax, pt, lane);
+        tco[0][lane] = T(cd.lam0 - lamf);
+        tco[1][lane] = T(2.0 * lamf * U0);
+        tco[2][lane] = T(lamf * U0 * U0);
+        tco[3][lane] = T(2.0 * lamf * V0);
+        tco[4][lane] = T(lamf * V0 * V0);
+        // face step (Eq. dt_face) and time-integration weights (Eq. C_coeffs)
+        double dGf;
+        if (!g.hasL) dGf = cd.dG[cR];
+        else if (!g.hasR) dGf = cd.dG[cL];
+        else if (cd.face_step == 1) dGf = 2.0 * cd.dG[cL] * cd.dG[cR] * rcp64(cd.dG[cL] + cd.dG[cR]);
+        else dGf = fmin(cd.dG[cL], cd.dG[cR]);
+        sdG[lane] = dGf;
+        T Ct[5];
+        ugks_coeffs<T>(T(dGf), T(relax_time(cd.mu0, cd.w_vss, il0, ir, lamf)), Ct);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) Cw[k][lane] = Ct[k];
     }
-    w[0] = m[13] / rho0; w[1] = m[14] / rho0; w[2] = m[15] / rho0; w[3] = 0.5 * (m[16] + m[17]) / rho0;
-    micro_slope(w, U0, V0, lamf, at);
+    __syncthreads();
 
-    // ---- separable table of the interface Maxwellian and its 1-D sums
-    const int nu = cd.nu, nv = cd.nv, nuv = nu + nv;
-    T* tb = cd.ftab + (size_t)item * nuv;
-    SumsT<T> dX, dY;
+    // ---- B: separable table of the interface Maxwellian and its 1-D sums.  The nodes are taken in the order of their
+    // class (positive, negative, zero), so that a node adds to one sum only.
+    for (int axis = 0; axis < 2; ++axis) {
+        const int nn = axis == 0 ? nu : nv, e0 = cd.ncls[axis][0], e1 = cd.ncls[axis][1];
+        const T* __restrict__ xn = axis == 0 ? cd.su1 : cd.sv1;
+        const T* __restrict__ wq = axis == 0 ? cd.wxr : cd.wyr;
+        const int* __restrict__ ord = axis == 0 ? cd.ou1 : cd.ov1;
+        T* const tab = cd.ftab + (axis == 0 ? 0 : nu);
+        T acc[3][3];                                         // powers role, role + 4, role + 8; node classes
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int q = 0; q < 9; ++q) { dX.s[r][q] = T(0); dY.s[r][q] = T(0); }
-    {
-        const T dl = T(cd.lam0 - lamf);
-        T tl = T(2.0 * lamf * U0), l2 = T(lamf * U0 * U0);
-        // the sums of the three node classes (positive, negative, zero) in registers: a node adds its term to
-        // its own class and zero to the other two
-        T sp_[9], sn_[9], sz_[9];
+            for (int b = 0; b < 3; ++b) acc[a][b] = T(0);
+        for (int k0 = 0; k0 < nn; k0 += K2_NODES) {
+            const int kn = min(K2_NODES, nn - k0);
+            if (lane < kn) {
+                const T x = __ldg(xn + k0 + lane);
+                const int o = __ldg(ord + k0 + lane);
+#pragma unroll 4
+                for (int i = role; i < K2_ITEMS; i += K2_WARPS) {
+                    const T e = t_expm1<T>(tco[0][i] * x * x + tco[1 + 2 * axis][i] * x - tco[2 + 2 * axis][i]);
+                    se[lane][i] = e;
+                    if (base + i < nitems) tab[(size_t)(base + i) * nuv + o] = e;
+                }
+            }
+            __syncthreads();
+            const int b0 = min(max(e0 - k0, 0), kn), b1 = min(max(e1 - k0, 0), kn);
 #pragma unroll
-        for (int q = 0; q < 9; ++q) { sp_[q] = T(0); sn_[q] = T(0); sz_[q] = T(0); }
-        for (int k = 0; k < nu; ++k) {
-            const T x = cd.tu1[k];
-            const T e = t_expm1<T>(dl * x * x + tl * x - l2);
-            tb[k] = e;
-            const T ep = x > T(0) ? e : T(0), en = x < T(0) ? e : T(0), ez = x == T(0) ? e : T(0);
+            for (int a = 0; a < 3; ++a) {
+                const int q = role + K2_WARPS * a;
+                if (q >= 9) break;
+                const T* __restrict__ wk = wq + (size_t)q * nn + k0;
+#pragma unroll 4
+                for (int k = 0; k < b0; ++k) acc[a][0] += __ldg(wk + k) * se[k][lane];
+#pragma unroll 4
+                for (int k = b0; k < b1; ++k) acc[a][1] += __ldg(wk + k) * se[k][lane];
+                for (int k = b1; k < kn; ++k) acc[a][2] += __ldg(wk + k) * se[k][lane];
+            }
+            __syncthreads();
+        }
 #pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                const T wq = cd.wxr[q * nu + k];
-                sp_[q] += wq * ep; sn_[q] += wq * en; sz_[q] += wq * ez;
+        for (int a = 0; a < 3; ++a) {
+            const int q = role + K2_WARPS * a;
+            if (q >= 9) break;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) S[axis][b][q][lane] = acc[a][b];
+        }
+    }
+    __syncthreads();
+
+    // ---- C: velocity moments of the Maxwellian's polynomials
+    const T pref = T(rho0 * lamf / M_PI), i2l = T(i2ld);
+    // full 1-D sums of the interface Maxwellian over node subset r (0 all, 1 positive, 2 negative, 3 zero); dif: the
+    // table part alone
+    auto row = [&](int axis, int r, T (&o)[9]) {
+        const T* ref = (axis == 0 ? cd.xr0t : cd.yr0t) + r * 9;
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+            o[q] = ref[q] + (r == 0 ? S[axis][0][q][lane] + S[axis][1][q][lane] + S[axis][2][q][lane]
+                                    : S[axis][r - 1][q][lane]);
+    };
+    auto rows = [&](int r, T (&x)[9], T (&y)[9]) { row(ax, r, x); row(1 - ax, 0, y); };   // subset r along the normal
+    // moments back from (n, t) to (u, v) order
+    auto put = [&](T (*o)[K2_ITEMS], const T (&m)[4]) {
+        o[0][lane] = m[0];
+        o[1][lane] = ax == 0 ? m[1] : m[2];
+        o[2][lane] = ax == 0 ? m[2] : m[1];
+        o[3][lane] = m[3];
+    };
+    const int half = wall ? inc_row : 0;                     // velocities carried by the integral solution
+    T x[9], y[9];
+    if (role == 0) {
+        // compatibility: moments of (A.psi) g0 = - moments of (u_n a_n + u_t a_t) g0
+        T c[10], d[10], dn, dt, en, M[4], tmp[4];
+        side_poly(pL, pt, lane, c, dn, dt);
+        rows(wall ? 0 : 1, x, y);
+        mom4<0, true>(c, T(0), dn, dt, x, y, pref, i2l, M);
+        if (!wall) {
+            side_poly(pR, pt, lane, d, en, dt);
+            rows(2, x, y);
+            mom4<0, true>(d, T(0), en, dt, x, y, pref, i2l, tmp);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) M[k] += tmp[k];
+            if (cd.zeros) {
+                // nodes with u_n = 0 take the average of both sides
+#pragma unroll
+                for (int k = 0; k < 10; ++k) c[k] = T(0.5) * (c[k] + d[k]);
+                rows(3, x, y);
+                mom4<0, true>(c, T(0), T(0.5) * (dn + en), dt, x, y, pref, i2l, tmp);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) M[k] += tmp[k];
             }
         }
+        const double w[4] = {-(double)M[0] * ir, -(double)(ax == 0 ? M[1] : M[2]) * ir, -(double)(ax == 0 ? M[2] : M[1]) * ir,
+                             -(double)M[3] * ir};
+        slope_poly<T>(w, U0, V0, lamf, i2ld, ax, pA, lane);
+    } else if (role == 1) {
+        // C1 term: moments of u_n s (c.q)(2 lam |c|^2 - 4)
+        T c[10], o[4];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) { dX.s[1][q] = sp_[q]; dX.s[2][q] = sn_[q]; dX.s[3][q] = sz_[q]; }
-#pragma unroll
-        for (int q = 0; q < 9; ++q) { sp_[q] = T(0); sn_[q] = T(0); sz_[q] = T(0); }
-        tl = T(2.0 * lamf * V0);
-        l2 = T(lamf * V0 * V0);
-        for (int k = 0; k < nv; ++k) {
-            const T y = cd.tv1[k];
-            const T e = t_expm1<T>(dl * y * y + tl * y - l2);
-            tb[nu + k] = e;
-            const T ep = y > T(0) ? e : T(0), en = y < T(0) ? e : T(0), ez = y == T(0) ? e : T(0);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                const T wq = cd.wyr[q * nv + k];
-                sp_[q] += wq * ep; sn_[q] += wq * en; sz_[q] += wq * ez;
+        for (int k = 0; k < 10; ++k) c[k] = shk_[k][lane];
+        rows(half, x, y);
+        mom4<1, true>(c, shk_[10][lane], shk_[11][lane], shk_[12][lane], x, y, pref, i2l, o);
+        put(F1s, o);
+    } else {
+        // C2 term: u_n (u_n P(a_bar) + u_t P(a_t)), a_bar = a^L for u_n > 0 (warp 2), a^R for u_n < 0 (warp 3; at a wall
+        // the incident velocities' one side is warp 2's)
+        T o[4] = {T(0), T(0), T(0), T(0)};
+        if (role == 2 || !wall) {
+            T c[10], dn, dt;
+            side_poly(role == 2 ? pL : pR, pt, lane, c, dn, dt);
+            rows(wall ? inc_row : role - 1, x, y);
+            mom4<1, true>(c, T(0), dn, dt, x, y, pref, i2l, o);
+        }
+        put(role == 2 ? F2L : F2R, o);
+        if (role == 3) {
+            // C1 term, Maxwellian part: moments of u_n psi (H0 - H_ref, B0 - B_ref), in FP64 from the reference sums
+            const double rr = rho0 * lamf * il0, di2l = i2ld - 0.5 * il0, fac = cd.lam0 / M_PI;
+            const int rx = ax == 0 ? half : 0, ry = ax == 0 ? 0 : half;
+            const double* X0 = cd.xr0 + rx * 9;
+            const double* Y0 = cd.yr0 + ry * 9;
+            auto dif = [&](int axis, int r, int q) -> double {
+                return r == 0 ? (double)(S[axis][0][q][lane] + S[axis][1][q][lane] + S[axis][2][q][lane])
+                              : (double)S[axis][r - 1][q][lane];
+            };
+            // (lam0/pi) [(r - 1) X0 Y0 + r (dX Y0 + X0 dY + dX dY)] and (lam0/pi) X0 Y0
+            auto Sd = [&](int p, int q) {
+                const double x0 = X0[p], y0 = Y0[q], dx = dif(0, rx, p), dy = dif(1, ry, q);
+                return fac * ((rr - 1.0) * x0 * y0 + rr * (dx * y0 + x0 * dy + dx * dy));
+            };
+            double o4[4];
+            if (ax == 0) {
+                const double s10 = Sd(1, 0);
+                o4[0] = s10; o4[1] = Sd(2, 0); o4[2] = Sd(1, 1);
+                o4[3] = 0.5 * (Sd(3, 0) + Sd(1, 2)) + 0.5 * (i2ld * s10 + di2l * fac * X0[1] * Y0[0]);
+            } else {
+                const double s01 = Sd(0, 1);
+                o4[0] = s01; o4[1] = Sd(1, 1); o4[2] = Sd(0, 2);
+                o4[3] = 0.5 * (Sd(2, 1) + Sd(0, 3)) + 0.5 * (i2ld * s01 + di2l * fac * X0[0] * Y0[1]);
             }
-        }
 #pragma unroll
-        for (int q = 0; q < 9; ++q) { dY.s[1][q] = sp_[q]; dY.s[2][q] = sn_[q]; dY.s[3][q] = sz_[q]; }
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            dX.s[0][q] = dX.s[1][q] + dX.s[2][q] + dX.s[3][q];
-            dY.s[0][q] = dY.s[1][q] + dY.s[2][q] + dY.s[3][q];
+            for (int k = 0; k < 4; ++k) dF1[k][lane] = o4[k];
         }
     }
-    // full 1-D sums of the interface Maxwellian (reference + table part)
-    SumsT<T> X, Y;
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            X.s[r][q] = cd.xr0t[r * 9 + q] + dX.s[r][q];
-            Y.s[r][q] = cd.yr0t[r * 9 + q] + dY.s[r][q];
-        }
-    const T pref = T(rho0 * lamf / M_PI), i2l = T(0.5 / lamf);
-    auto rows = [&](int r, int& rx, int& ry) { rx = ax == 0 ? r : 0; ry = ax == 0 ? 0 : r; };
-    // u_n and u_t as the axis a product by them shifts a polynomial along (0: u, 1: v)
-    const int axn = ax, axt = 1 - ax;
-    PolyT<T> PhL, PbL, PhR, PbR, Pht, Pbt, t1, t2;
-    poly_P<T>(aL, 0.5 / lamf, false, PhL); poly_P<T>(aL, 0.5 / lamf, true, PbL);
-    poly_P<T>(aR, 0.5 / lamf, false, PhR); poly_P<T>(aR, 0.5 / lamf, true, PbR);
-    poly_P<T>(at, 0.5 / lamf, false, Pht); poly_P<T>(at, 0.5 / lamf, true, Pbt);
-    // Q_side = u_n P_h(a_side) + u_t P_h(a_t),  R_side likewise with P_b
-    PolyT<T> QL, RL, QR, RR, Q0, R0;
-    poly_shift(axn, PhL, QL); poly_shift(axt, Pht, t1);
-    poly_shift(axn, PbL, RL); poly_shift(axt, Pbt, t2);
-    poly_shift(axn, PhR, QR);
-    poly_shift(axn, PbR, RR);
-#pragma unroll
-    for (int a = 0; a < 5; ++a)
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-            QL.c[a][b] += t1.c[a][b];
-            RL.c[a][b] += t2.c[a][b];
-            QR.c[a][b] += t1.c[a][b];
-            RR.c[a][b] += t2.c[a][b];
-            Q0.c[a][b] = T(0.5) * (QL.c[a][b] + QR.c[a][b]);
-            R0.c[a][b] = T(0.5) * (RL.c[a][b] + RR.c[a][b]);
-        }
-    // compatibility: moments of (A.psi) g0 = - moments of (u_n a_n + u_t a_t) g0
-    T M[4], tmp[4];
-    int rx, ry;
-    if (!wall) {
-        rows(1, rx, ry); mom4(QL, RL, X, rx, Y, ry, pref, i2l, M);
-        rows(2, rx, ry); mom4(QR, RR, X, rx, Y, ry, pref, i2l, tmp);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) M[k] += tmp[k];
-        rows(3, rx, ry); mom4(Q0, R0, X, rx, Y, ry, pref, i2l, tmp);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) M[k] += tmp[k];
-    } else {
-        mom4(QL, RL, X, 0, Y, 0, pref, i2l, M);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) w[k] = -(double)M[k] / rho0;
-    micro_slope(w, U0, V0, lamf, Aa);
+    __syncthreads();
 
-    // ---- macro flux deviation (Eq. macro_flux minus the flux of H_ref, which cancels in every cell balance)
-    // Shakhov factor s (c.q)(2 lam |c|^2 - 4) and the b-part addition 2 s (c.q)
-    double sp[13];
-    shakhov_poly((1.0 - cd.pr) * 4.0 * lamf * lamf / (5.0 * rho0), q0x, q0y, U0, V0, lamf, sp);
-    PolyT<T> shk, cq2, sb;
-    shk.zero(); cq2.zero();
-    shk.c[0][0] = T(sp[0]); shk.c[1][0] = T(sp[1]); shk.c[0][1] = T(sp[2]); shk.c[2][0] = T(sp[3]);
-    shk.c[1][1] = T(sp[4]); shk.c[0][2] = T(sp[5]); shk.c[3][0] = T(sp[6]); shk.c[2][1] = T(sp[7]);
-    shk.c[1][2] = T(sp[8]); shk.c[0][3] = T(sp[9]);
-    cq2.c[0][0] = T(sp[10]); cq2.c[1][0] = T(sp[11]); cq2.c[0][1] = T(sp[12]);
-    sb = shk;
-    sb.c[0][0] += cq2.c[0][0]; sb.c[1][0] += cq2.c[1][0]; sb.c[0][1] += cq2.c[0][1];
-    const int half = wall ? inc_row : 0;  // velocities carried by the integral solution
-    PolyT<T> q1, r1;
-    poly_shift(axn, shk, q1); poly_shift(axn, sb, r1);
-    T F1s[4], F2[4], F3[4];
-    rows(half, rx, ry);
-    mom4(q1, r1, X, rx, Y, ry, pref, i2l, F1s);
-    // C2 term: u_n (u_n P(a_bar) + u_t P(a_t)) with a_bar = a^L for u_n > 0, a^R for u_n < 0
-    PolyT<T> uQ, uR;
-    if (!wall) {
-        poly_shift(axn, QL, uQ); poly_shift(axn, RL, uR);
-        rows(1, rx, ry); mom4(uQ, uR, X, rx, Y, ry, pref, i2l, F2);
-        poly_shift(axn, QR, uQ); poly_shift(axn, RR, uR);
-        rows(2, rx, ry); mom4(uQ, uR, X, rx, Y, ry, pref, i2l, tmp);
+    // ---- D: macro flux deviation (Eq. macro_flux minus the flux of H_ref, which cancels in every cell balance) and the
+    // parameters of the micro flux (delta form, divided by dG_f; level-major: a tile's faces of one level are rows)
+    if (!valid) return;
+    T* pp = cd.fpar + ((size_t)n * cd.nf + f) * NP;
+    const double dGf = sdG[lane], idG = rcp64(dGf);
+    const double rr = rho0 * lamf * il0;
+    if (role == 0) {
+        // C3 term: u_n P(A)
+        const T c[10] = {pA[0][lane], pA[2][lane], pA[3][lane], pA[4][lane], T(0), pA[4][lane], T(0), T(0), T(0), T(0)};
+        T o[4];
+        rows(half, x, y);
+        mom4<1, false>(c, pA[1][lane], T(0), T(0), x, y, pref, i2l, o);
+        const T F3[4] = {o[0], ax == 0 ? o[1] : o[2], ax == 0 ? o[2] : o[1], o[3]};
+        // C4 term: u_n psi (h_0 - H_ref) (reconstruction; incident velocities only at a wall); C5 term
+        double F4[4], F5[4], I[4], F[4];
+        if (ax == 0) { F4[0] = msum(1); F4[1] = msum(3); F4[2] = msum(4); F4[3] = 0.5 * (msum(6) + msum(8) + msum(11)); }
+        else { F4[0] = msum(2); F4[1] = msum(4); F4[2] = msum(5); F4[3] = 0.5 * (msum(7) + msum(9) + msum(12)); }
+        F5[0] = msum(18); F5[1] = msum(19); F5[2] = msum(20); F5[3] = 0.5 * (msum(21) + msum(22));
+        double C[5];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) F2[k] += tmp[k];
-    } else {
-        poly_shift(axn, QL, uQ); poly_shift(axn, RL, uR);
-        rows(inc_row, rx, ry); mom4(uQ, uR, X, rx, Y, ry, pref, i2l, F2);
-    }
-    // C3 term: u_n P(A)
-    PolyT<T> PhA, PbA;
-    poly_P<T>(Aa, 0.5 / lamf, false, PhA); poly_P<T>(Aa, 0.5 / lamf, true, PbA);
-    poly_shift(axn, PhA, uQ); poly_shift(axn, PbA, uR);
-    rows(half, rx, ry);
-    mom4(uQ, uR, X, rx, Y, ry, pref, i2l, F3);
-    // C1 term, Maxwellian part: moments of u_n psi (H0 - H_ref, B0 - B_ref), in FP64 from the reference sums
-    const double rr = rho0 * lamf / cd.lam0, i2ld = 0.5 / lamf, di2l = 0.5 / lamf - 0.5 / cd.lam0;
-    double dF1[4];
-    {
-        rows(half, rx, ry);
-        auto S = [&](int pp, int qq) { return dsum(cd.xr0, cd.yr0, dX, dY, rx, ry, pp, qq, rr, cd.lam0); };
-        auto Sr = [&](int pp, int qq) { return cd.lam0 / M_PI * cd.xr0[rx * 9 + pp] * cd.yr0[ry * 9 + qq]; };
-        if (ax == 0) {
-            const double s10 = S(1, 0);
-            dF1[0] = s10; dF1[1] = S(2, 0); dF1[2] = S(1, 1);
-            dF1[3] = 0.5 * (S(3, 0) + S(1, 2)) + 0.5 * (i2ld * s10 + di2l * Sr(1, 0));
+        for (int k = 0; k < 5; ++k) C[k] = (double)Cw[k][lane];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            I[k] = C[0] * (dF1[k][lane] + (double)F1s[k][lane]) + C[1] * (double)(F2L[k][lane] + F2R[k][lane]) +
+                   C[2] * (double)F3[k] + C[3] * F4[k] + C[4] * F5[k];
+        double rhow = 0.0;
+        if (!wall) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) F[k] = I[k] * idG;
         } else {
-            const double s01 = S(0, 1);
-            dF1[0] = s01; dF1[1] = S(1, 1); dF1[2] = S(0, 2);
-            dF1[3] = 0.5 * (S(2, 1) + S(0, 3)) + 0.5 * (i2ld * s01 + di2l * Sr(0, 1));
+            // impermeability (Eq. rho_wall) with the time-integrated incident mass flux; reflected part rho_w H_w
+            const double* oc = cd.oconst + g.wall * 8;       // [0..3] incident flux of H_ref, [4..7] reflected
+            rhow = -nin * (oc[0] + I[0] * idG) * rcp64(wc[13]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) F[k] = I[k] * idG + rhow * wc[14 + k] - oc[4 + k];
         }
-    }
-    // C4 term: u_n psi (h_0 - H_ref) (reconstruction; incident velocities only at a wall); C5 term
-    double F4[4], F5[4];
-    if (ax == 0) { F4[0] = m[1]; F4[1] = m[3]; F4[2] = m[4]; F4[3] = 0.5 * (m[6] + m[8] + m[11]); }
-    else { F4[0] = m[2]; F4[1] = m[4]; F4[2] = m[5]; F4[3] = 0.5 * (m[7] + m[9] + m[12]); }
-    F5[0] = m[18]; F5[1] = m[19]; F5[2] = m[20]; F5[3] = 0.5 * (m[21] + m[22]);
-    double I[4], F[4];
+        double* fo = cd.fflux + (size_t)item * 4;
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        I[k] = C[0] * (dF1[k] + (double)F1s[k]) + C[1] * (double)F2[k] + C[2] * (double)F3[k] + C[3] * F4[k] + C[4] * F5[k];
-    double rhow = 0.0;
-    if (!wall) {
+        for (int k = 0; k < 4; ++k) fo[k] = F[k];
+        if (wall) {
+            const double* ws = cd.wall + ((size_t)g.wall * cd.nslot + wsl) * 3;
+            const double lamw = cd.lam0 * rcp64(ws[2]), iw = 0.5 * rcp64(lamw);
+            const double rw = rhow * lamw * il0;
+            pp[F_WRM1] = T(rw - 1.0);
+            pp[F_WR] = T(rw);
+            pp[F_WI2L] = T(iw);
+            pp[F_WDI2L] = T(iw - 0.5 * il0);
+        } else {
+            pp[F_WRM1] = pp[F_WR] = pp[F_WI2L] = pp[F_WDI2L] = T(0);
+        }
+    } else if (role < 3) {
+        // for the upwind side: the cubic Q = C1' s(c.q)(2 lam |c|^2 - 4) + C2' (u_n P_h(a_side) + u_t P_h(a_t)) +
+        // C3' P_h(A) and the linear b-part difference C1' 2 s (c.q) + C2' (u_n a_side,3 + u_t a_t,3)/(2 lam) +
+        // C3' A_3/(2 lam)
+        T c[10], dn, dt;
+        side_poly(role == 1 ? pL : pR, pt, lane, c, dn, dt);
+        const T C1p = T((double)Cw[0][lane] * idG), C2p = T((double)Cw[1][lane] * idG), C3p = T((double)Cw[2][lane] * idG);
+        const T pa[10] = {pA[0][lane], pA[2][lane], pA[3][lane], pA[4][lane], T(0), pA[4][lane], T(0), T(0), T(0), T(0)};
+        T* q = pp + (role == 1 ? F_QL : F_QR);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) F[k] = I[k] / dGf;
+        for (int k = 0; k < 10; ++k) q[ax == 0 ? k : nt_order(k)] = C1p * shk_[k][lane] + C2p * c[k] + C3p * pa[k];
+        T* l = pp + (role == 1 ? F_LBL : F_LBR);
+        l[0] = C1p * shk_[10][lane] + C3p * pA[1][lane];
+        l[ax == 0 ? 1 : 2] = C1p * shk_[11][lane] + C2p * dn;
+        l[ax == 0 ? 2 : 1] = C1p * shk_[12][lane] + C2p * dt;
     } else {
-        // impermeability (Eq. rho_wall) with the time-integrated incident mass flux; reflected part rho_w H_w
-        const double* oc = cd.oconst + g.wall * 8;           // [0..3] incident flux of H_ref, [4..7] reflected
-        const double Iinc0 = dGf * oc[0] + I[0];
-        rhow = -nin * Iinc0 / (dGf * Dw);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) F[k] = I[k] / dGf + rhow * wc[14 + k] - oc[4 + k];
-    }
-    double* fo = cd.fflux + (size_t)item * 4;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) fo[k] = F[k];
-
-    // ---- parameters of the micro flux (delta form, divided by dG_f): for each upwind side the cubic
-    // Q = C1' s(c.q)(2 lam |c|^2 - 4) + C2' (u_n P_h(a_side) + u_t P_h(a_t)) + C3' P_h(A) and the linear b-part
-    // difference C1' 2 s (c.q) + C2' (u_n a_side,3 + u_t a_t,3)/(2 lam) + C3' A_3/(2 lam)
-    T* pp = cd.fpar + ((size_t)n * cd.nf + f) * NP;      // level-major: a tile's faces of one level are rows
-    const T C1p = T(C[0] / dGf), C2p = T(C[1] / dGf), C3p = T(C[2] / dGf);
-    for (int side = 0; side < 2; ++side) {
-        const PolyT<T>& Qs = side == 0 ? QL : QR;
-        const PolyT<T>& Rs = side == 0 ? RL : RR;
-        PolyT<T> qf, lb;
-#pragma unroll
-        for (int a = 0; a < 5; ++a)
-#pragma unroll
-            for (int b = 0; b < 5; ++b) {
-                qf.c[a][b] = C1p * shk.c[a][b] + C2p * Qs.c[a][b] + C3p * PhA.c[a][b];
-                lb.c[a][b] = C1p * cq2.c[a][b] + C2p * (Rs.c[a][b] - Qs.c[a][b]) + C3p * (PbA.c[a][b] - PhA.c[a][b]);
-            }
-        T* q = pp + (side == 0 ? F_QL : F_QR);
-        q[0] = qf.c[0][0]; q[1] = qf.c[1][0]; q[2] = qf.c[0][1]; q[3] = qf.c[2][0]; q[4] = qf.c[1][1];
-        q[5] = qf.c[0][2]; q[6] = qf.c[3][0]; q[7] = qf.c[2][1]; q[8] = qf.c[1][2]; q[9] = qf.c[0][3];
-        T* l = pp + (side == 0 ? F_LBL : F_LBR);
-        l[0] = lb.c[0][0]; l[1] = lb.c[1][0]; l[2] = lb.c[0][1];
-    }
-    pp[F_RM1] = T(rr - 1.0);
-    pp[F_R] = T(rr);
-    pp[F_I2L] = T(i2ld);
-    pp[F_DI2L] = T(di2l);
-    pp[F_C1] = C1p;
-    pp[F_C4] = T(C[3] / dGf);
-    pp[F_C5] = T(C[4] / dGf);
-    pp[F_NIN] = T(nin);
-    if (wall) {
-        const double* ws = cd.wall + ((size_t)g.wall * cd.nslot + wsl) * 3;
-        const double lamw = cd.lam0 / ws[2];
-        const double rw = rhow * lamw / cd.lam0;
-        pp[F_WRM1] = T(rw - 1.0);
-        pp[F_WR] = T(rw);
-        pp[F_WI2L] = T(0.5 / lamw);
-        pp[F_WDI2L] = T(0.5 / lamw - 0.5 / cd.lam0);
-    } else {
-        pp[F_WRM1] = pp[F_WR] = pp[F_WI2L] = pp[F_WDI2L] = T(0);
+        pp[F_RM1] = T(rr - 1.0);
+        pp[F_R] = T(rr);
+        pp[F_I2L] = T(i2ld);
+        pp[F_DI2L] = T(i2ld - 0.5 * il0);
+        pp[F_C1] = T((double)Cw[0][lane] * idG);
+        pp[F_C4] = T((double)Cw[3][lane] * idG);
+        pp[F_C5] = T((double)Cw[4][lane] * idG);
+        pp[F_NIN] = T(nin);
     }
 }
 
