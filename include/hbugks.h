@@ -214,8 +214,8 @@ HBUGKS_API hbugks_status hbugks_harmonic_noalloc(int nx, int ny, int nu, int nv,
 /* Variant of the micro-update kernel of a case, named by a tile (tx x ty cells) and vpl, blocks of 32 velocities.
  * The variants are 4x4, 4x2, 2x2 and 8x4 with vpl 1, and 4x2 with vpl 2, which needs single precision and sign
  * classes that each hold an even number of velocity blocks.  The kernel marches over a strip of columns on all
- * levels; a variant sets the strip and the rows a CTA marches over: 4x4 four columns and 16 rows, 4x2 two and 16
- * (with vpl 2 four and 8), 2x2 two and 2, 8x4 four and 32 (two columns instead of four where four do not fit, or in a
+ * levels; a variant sets the strip and the rows it marches over: 4x4 four columns and 16 rows, 4x2 two and 16
+ * (with vpl 2 two and 32), 2x2 two and 2, 8x4 four and 32 (two columns instead of four where four do not fit, or in a
  * mesh of fewer than four columns).  hbugks_create() picks one per case by timing every variant the
  * case can run on the case itself (autotuning, cached per process by mesh size, velocity grid, level count,
  * precision and SM count).  get: the variant of case `case_index`.  set: pin one, for example to reproduce a
@@ -251,7 +251,7 @@ HBUGKS_API hbugks_status hbugks_test_expire_wait(hbugks_t h);
 HBUGKS_API int hbugks_launches_per_iteration(hbugks_t h);
 
 /* How hbugks_iterate and hbugks_enqueue_iterations run their iterations.  mode 0 (default): one launch of a
- * CUDA graph whose conditional while node repeats one iteration and a one-thread loop test until the count is
+ * CUDA graph whose conditional while node repeats one iteration (its last kernel holds the loop test) until the count is
  * spent, every case has converged or diverged, or a device wait has failed; the host reads the statuses once, at
  * the end.  mode 1: graphs of 16 iterations launched from the host, which reads the statuses after each (the
  * earlier design, kept for comparison).  Both run the same kernels and give bitwise the same state.  The paper

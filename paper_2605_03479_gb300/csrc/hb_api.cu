@@ -39,6 +39,7 @@ cudaError_t& last_cuda_error()
 }
 
 constexpr int CHUNK = 16;   // iterations per captured graph
+constexpr int GPU_SMS = 152; // of the GB300 this library is built for (launch shapes only)
 
 // NVTX range (header-only NVTX 3): a tracing tool attached to the process (Nsight Systems, or any library named
 // by NVTX_INJECTION64_PATH) sees every call of the C ABI, and every kernel stage that an iteration enqueues, as
@@ -103,21 +104,28 @@ struct HostCase {
     int ng[2];                      // groups of one or two velocity blocks of one sign class
 };
 
-// K1 tile (TX x TY cells, one warp each) and velocity blocks staged per pass, per storage precision
-template <typename T> constexpr int K1_TX = 4;
-template <typename T> constexpr int K1_TY = 2;
-template <typename T> constexpr int K1_G = std::is_same<T, float>::value ? 6 : 4;
-template <typename T> constexpr int K1_S = 3;   // pipeline stages of the staged velocity blocks
+// K1: tile (TX x TY cells, one warp each), velocity blocks per staged chunk, stages of the ring, CTAs per SM
+template <typename T, bool SEP> struct K1Cfg { static constexpr int TX = 4, TY = 2, G = 4, S = 3, CTAS = 1; };
+template <> struct K1Cfg<float, true> { static constexpr int TX = 4, TY = 2, G = 3, S = 3, CTAS = 3; };
+template <> struct K1Cfg<float, false> { static constexpr int TX = 4, TY = 2, G = 4, S = 3, CTAS = 2; };
 
-template <typename T>
+template <typename T, bool SEP>
 constexpr size_t k1_smem_of()
 {
-    return k1_cells_smem<T, K1_TX<T>, K1_TY<T>, K1_G<T>, K1_S<T>>();
+    using C = K1Cfg<T, SEP>;
+    return k1_cells_smem<T, C::TX, C::TY, C::G, C::S, SEP>();
 }
-template <typename T, bool SEP>
+template <class P, bool SEP>
 constexpr auto k1_kernel()
 {
-    return k1_cells<T, K1_TX<T>, K1_TY<T>, K1_G<T>, K1_S<T>, SEP>;
+    using C = K1Cfg<typename P::value_type, SEP>;
+    return k1_cells<P, C::TX, C::TY, C::G, C::S, SEP, C::CTAS>;
+}
+template <typename T, bool SEP>
+int k1_blocks(int nx, int ny, int nt)
+{
+    using C = K1Cfg<T, SEP>;
+    return ((nx + C::TX - 1) / C::TX) * ((ny + C::TY - 1) / C::TY) * nt;
 }
 
 // K4 variants as the ABI names them: tx x ty cells and vpl velocity blocks.  A CTA of k4_march takes a strip of
@@ -126,7 +134,7 @@ constexpr auto k1_kernel()
 struct Shape {
     int tx, ty, vpl, cols, rows;
 };
-constexpr Shape K4_SHAPES[] = {{4, 4, 1, 4, 16}, {4, 2, 1, 2, 16}, {2, 2, 1, 2, 2}, {8, 4, 1, 4, 32}, {4, 2, 2, 4, 8}};
+constexpr Shape K4_SHAPES[] = {{4, 4, 1, 4, 16}, {4, 2, 1, 2, 16}, {2, 2, 1, 2, 2}, {8, 4, 1, 4, 32}, {4, 2, 2, 2, 32}};
 constexpr int N_K4_SHAPES = 5;
 template <typename T> constexpr int K4_VPL = std::is_same<T, float>::value ? 2 : 1;
 
@@ -144,10 +152,11 @@ size_t k4_smem_of(int cols, int nt, bool imp)
 // of a variant: two columns where four need more shared memory than a CTA may have, and in a mesh of fewer columns,
 // since only strips of two may be partial.  Every strip and segment gives the same bits.
 template <typename T>
-March k4_march_of(int shape, int nx, int nt, bool imp)
+March k4_march_of(int shape, int nx, int nt, int nuv, bool imp)
 {
     const Shape s = K4_SHAPES[shape];
-    return {s.cols == 4 && nx >= 4 && nt <= K4_NT4L && k4_smem_of<T>(4, nt, imp) <= SMEM_MAX ? 4 : 2, s.rows};
+    const bool levels = nt <= K4_NT4 || (nt <= K4_NT4L && 8LL * nt * nuv * (int)sizeof(T) <= INT_MAX);   // 32-bit offsets
+    return {s.cols == 4 && nx >= 4 && levels && k4_smem_of<T>(4, nt, imp) <= SMEM_MAX ? 4 : 2, s.rows};
 }
 
 // Bytes a tile of a variant holds: its cells on all levels, twice its halo rectangle, face and cell parameters and
@@ -338,8 +347,9 @@ void layout_case(Carver& cv, const HostCase& h, CaseDev<T>& d)
     d.hx = cv.take<double>(h.nx); d.hy = cv.take<double>(h.ny);
     d.rdx = cv.take<double>(h.nx); d.rdy = cv.take<double>(h.ny);
     d.vu = cv.take<double>(h.nvp); d.vv = cv.take<double>(h.nvp); d.vw = cv.take<double>(h.nvp);
-    d.tu = cv.take<T>(h.nvp); d.tv = cv.take<T>(h.nvp); d.tw = cv.take<T>(h.nvp); d.thref = cv.take<T>(h.nvp);
-    d.twu = cv.take<T>(h.nvp); d.twv = cv.take<T>(h.nvp);
+    d.tu = cv.take<T>(h.nvp); d.tv = cv.take<T>(h.nvp); d.thref = cv.take<T>(h.nvp);
+    d.twu = cv.take<T>(h.nvp);
+    d.wrow = cv.take<T>((size_t)h.nvb * (h.k1sep ? K1_WT<true> : K1_WT<false>));
     d.u1 = cv.take<double>(h.nu); d.wu1 = cv.take<double>(h.nu);
     d.v1 = cv.take<double>(h.nv); d.wv1 = cv.take<double>(h.nv);
     d.tu1 = cv.take<T>(h.nu); d.tv1 = cv.take<T>(h.nv);
@@ -396,8 +406,9 @@ struct LaunchSpec {
     int table;     // block offset table index
     int total;     // total blocks
     size_t smem;   // dynamic shared memory bytes
-    int nt;        // K4: levels, strip and segment
+    int nt;        // K4: levels, strip and segment, groups per CTA
     March march;
+    int groups;
 };
 
 template <typename T>
@@ -440,11 +451,31 @@ namespace {
 template <typename T>
 void fill_offsets(Impl<T>& im, int ncases);
 
-// CTAs of the micro update of a case
+// groups of the micro update of a case (one per strip, segment and velocity group)
 template <typename T>
-int k4_blocks(const HostCase& h, March m)
+int k4_groups(const HostCase& h, March m)
 {
     return ((h.nx + m.cols - 1) / m.cols) * ((h.ny + m.rows - 1) / m.rows) * h.ng[K4_VPL<T> - 1];
+}
+
+// Groups per CTA when a launch has `total` of them: as many as 15 warps and shared memory take
+// (registers are handed out for four warps of a CTA at a time; with five groups of three warps instead of CTAs of three
+// 0.416 -> 0.347 ms, 90x90, 28x28, N_T 3, together with strips of two columns).  On small
+// launches single precision, which waits on latency, leaves every SM a CTA; FP64, whose pipe every warp of an SM shares,
+// takes the largest number that puts at most a twentieth more groups on the fullest SM than any other (640 groups: 5 on
+// each of 128 SMs, where 4 per CTA would put 8 on some: 0.709 against 0.758 ms, 32x32, 24x24, N_T 3).
+template <typename T>
+int k4_groups_per_cta(March m, int nt, bool imp, int total)
+{
+    if (nt > K4_NT4) return 1;
+    const int most = std::min<int>(MAXNT / nt, SMEM_MAX / k4_smem_of<T>(m.cols, nt, imp));
+    if (sizeof(T) == 4) return std::max(1, std::min(most, total / GPU_SMS));
+    auto load = [&](int g) { return (long long)((total + g - 1) / g + GPU_SMS - 1) / GPU_SMS * g; };
+    long long least = load(1);
+    for (int g = 2; g <= most; ++g) least = std::min(least, load(g));
+    for (int g = most; g > 1; --g)
+        if (20 * load(g) <= 21 * least) return g;
+    return 1;
 }
 
 template <typename T>
@@ -458,7 +489,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
         fill_host(h, cases[k]);
         h.k4shape = pick_k4_shape<T>(h.nt);
         im.max_nt = std::max(im.max_nt, h.nt);
-        h.k1b = ((h.nx + K1_TX<T> - 1) / K1_TX<T>) * ((h.ny + K1_TY<T> - 1) / K1_TY<T>) * h.nt;
+        h.k1b = h.k1sep ? k1_blocks<T, true>(h.nx, h.ny, h.nt) : k1_blocks<T, false>(h.nx, h.ny, h.nt);
         if (cases[k].phys.spectral_implicit) im.any_implicit = true;
     }
     im.d_cases = cv.take<CaseDev<T>>(ncases);
@@ -469,7 +500,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
     im.d_tune_off = cv.take<int>(2);
     // launch specs: K1 per shape, K2, K3, K4 per shape; plus the step kernel (state setting only)
     im.specs.clear();
-    auto add = [&](int kind, int shape) { im.specs.push_back(LaunchSpec{kind, shape, (int)im.specs.size(), 0, 0, 0, {}}); };
+    auto add = [&](int kind, int shape) { im.specs.push_back(LaunchSpec{kind, shape, (int)im.specs.size(), 0, 0, 0, {}, 1}); };
     add(0, 0);
     add(0, 1);
     add(1, 0);
@@ -511,22 +542,25 @@ void fill_offsets(Impl<T>& im, int ncases)
     for (auto& sp : im.specs) {
         int acc = 0;
         size_t smem = 0;
+        auto march_here = [&](const HostCase& h) {
+            if (sp.kind != 4 || h.k4shape < 0 || h.nt != sp.nt) return false;
+            const March m = k4_march_of<T>(h.k4shape, h.nx, h.nt, h.nu + h.nv, im.any_implicit);
+            return m.cols == sp.march.cols && m.rows == sp.march.rows;
+        };
+        if (sp.kind == 4) {
+            int total = 0;
+            for (const HostCase& h : im.hc) total += march_here(h) ? k4_groups<T>(h, sp.march) : 0;
+            sp.groups = k4_groups_per_cta<T>(sp.march, sp.nt, im.any_implicit, total);
+        }
         for (int k = 0; k < ncases; ++k) {
             im.off_host[(size_t)sp.table * (ncases + 1) + k] = acc;
             const HostCase& h = im.hc[k];
             int nb = 0;
             switch (sp.kind) {
-                case 0: nb = h.k1sep == sp.shape ? h.k1b : 0; smem = k1_smem_of<T>(); break;
+                case 0: nb = h.k1sep == sp.shape ? h.k1b : 0; smem = sp.shape ? k1_smem_of<T, true>() : k1_smem_of<T, false>(); break;
                 case 1: nb = h.k2b; break;
                 case 2: nb = h.k3b; break;
-                case 4:
-                    if (h.k4shape >= 0 && h.nt == sp.nt) {
-                        const March m = k4_march_of<T>(h.k4shape, h.nx, h.nt, im.any_implicit);
-                        if (m.cols != sp.march.cols || m.rows != sp.march.rows) break;
-                        nb = k4_blocks<T>(h, m);
-                        smem = k4_smem_of<T>(m.cols, h.nt, im.any_implicit);
-                    }
-                    break;
+                case 4: nb = march_here(h) ? (k4_groups<T>(h, sp.march) + sp.groups - 1) / sp.groups : 0; break;
                 case 5: nb = h.ksb; break;
             }
             acc += nb;
@@ -605,8 +639,9 @@ cudaError_t upload_case(const HostCase& h, const CaseDev<T>& d, cudaStream_t s, 
     for (int i = 0; i + 1 < h.nx; ++i) rdx[i] = 1.0 / (xc[i + 1] - xc[i]);
     for (int j = 0; j + 1 < h.ny; ++j) rdy[j] = 1.0 / (yc[j + 1] - yc[j]);
     std::vector<double> vu(h.nvp, 0.0), vv(h.nvp, 0.0), vw(h.nvp, 0.0);
-    std::vector<T> tu(h.nvp, T(0)), tv(h.nvp, T(0)), tw(h.nvp, T(0)), th(h.nvp, T(0)), twu(h.nvp, T(0)),
-        twv(h.nvp, T(0));
+    std::vector<T> tu(h.nvp, T(0)), tv(h.nvp, T(0)), th(h.nvp, T(0)), twu(h.nvp, T(0));
+    const int wt = h.k1sep ? K1_WT<true> : K1_WT<false>;
+    std::vector<T> wrow((size_t)h.nvb * wt, T(0));
     double ref[5][13];
     memset(ref, 0, sizeof ref);
     std::vector<int> iu_(h.nvp, 0), iv_(h.nvp, 0);
@@ -616,8 +651,21 @@ cudaError_t upload_case(const HostCase& h, const CaseDev<T>& d, cudaStream_t s, 
         const int iu = can % h.nu, jv = can / h.nu;
         const double u = h.u[iu], v = h.v[jv], w = h.wu[iu] * h.wv[jv] * h.vfac[a];
         vu[a] = u; vv[a] = v; vw[a] = w;
-        tu[a] = T(u); tv[a] = T(v); tw[a] = T(w); th[a] = T((1.0 / M_PI) * exp(-(u * u + v * v)));
-        twu[a] = T(h.wu[iu]); twv[a] = T(h.wv[jv] * h.vfac[a]);
+        tu[a] = T(u); tv[a] = T(v); th[a] = T((1.0 / M_PI) * exp(-(u * u + v * v)));
+        twu[a] = T(h.wu[iu]);
+        T* wr = &wrow[(size_t)(a / VB) * wt];
+        const int l = a % VB;
+        if (h.k1sep) {
+            double z = h.wv[jv] * h.vfac[a];
+            for (int q = 0; q < 4; ++q, z *= v) wr[l * 4 + q] = T(z);
+            wr[4 * VB + l] = T(z);
+        } else {
+            const double r2 = u * u + v * v;
+            const double m[13] = {1, u, v, u * u, u * v, v * v, u * u * u, u * u * v, u * v * v, v * v * v, u * u * r2,
+                                  v * v * r2, u * v * r2};
+            for (int q = 0; q < 12; ++q) wr[(q / 4) * 4 * VB + l * 4 + q % 4] = T(w * m[q]);
+            wr[12 * VB + l] = T(w * m[12]);
+        }
         iu_[a] = iu; iv_[a] = jv;
     }
     for (int jv = 0; jv < h.nv; ++jv)
@@ -646,10 +694,9 @@ cudaError_t upload_case(const HostCase& h, const CaseDev<T>& d, cudaStream_t s, 
     if ((e = put(d.vw, vw.data(), sizeof(double) * h.nvp))) return e;
     if ((e = put(d.tu, tu.data(), sizeof(T) * h.nvp))) return e;
     if ((e = put(d.tv, tv.data(), sizeof(T) * h.nvp))) return e;
-    if ((e = put(d.tw, tw.data(), sizeof(T) * h.nvp))) return e;
     if ((e = put(d.thref, th.data(), sizeof(T) * h.nvp))) return e;
     if ((e = put(d.twu, twu.data(), sizeof(T) * h.nvp))) return e;
-    if ((e = put(d.twv, twv.data(), sizeof(T) * h.nvp))) return e;
+    if ((e = put(d.wrow, wrow.data(), sizeof(T) * wrow.size()))) return e;
     if ((e = put(d.u1, h.u.data(), sizeof(double) * h.nu))) return e;
     if ((e = put(d.wu1, h.wu.data(), sizeof(double) * h.nu))) return e;
     if ((e = put(d.v1, h.v.data(), sizeof(double) * h.nv))) return e;
@@ -726,19 +773,10 @@ __global__ void k_begin_call(CaseStatus* st, int ncases)
     st[k].iters_call = 0;
 }
 
-__global__ void k_set_int(int* p, int v) { *p = v; }
-
-// End of one pass of the device-side loop: one iteration fewer left; the loop goes on while iterations are left,
-// some case is still iterating (not converged, not diverged) and no device wait has failed.  Every pass
-// decrements the count, so the loop ends after at most the requested number of iterations.
-__global__ void k_loop_test(cudaGraphConditionalHandle hc, int* left, const CaseStatus* st, int ncases, const int* err)
+__global__ void k_set_loop(int* p, int v)
 {
-    if (threadIdx.x != 0) return;
-    const int r = *left - 1;
-    *left = r;
-    int any = 0;
-    for (int k = 0; k < ncases; ++k) any |= st[k].active;
-    cudaGraphSetConditional(hc, (r > 0 && any && *(volatile const int*)err == 0) ? 1u : 0u);
+    p[0] = v;
+    p[1] = 0;
 }
 
 // state of one case copied between handles of possibly different precision (same grid and velocity layout)
@@ -751,44 +789,56 @@ __global__ void k_convert_state(const P2<TS>* src, P2<TD>* dst, size_t n)
     dst[k] = pk(TD(a.x), TD(a.y));
 }
 
-template <typename T>
-void launch_k1(int shape, int total, size_t smem, Batch<T> b, cudaStream_t s)
+template <class P>
+void launch_k1(int shape, int total, size_t smem, const P& b, cudaStream_t s)
 {
-    if (shape == 1) k1_kernel<T, true>()<<<total, K1_TX<T> * K1_TY<T> * 32, smem, s>>>(b);
-    else k1_kernel<T, false>()<<<total, K1_TX<T> * K1_TY<T> * 32, smem, s>>>(b);
+    using T = typename P::value_type;
+    if (shape == 1) k1_kernel<P, true>()<<<total, K1Cfg<T, true>::TX * K1Cfg<T, true>::TY * 32, smem, s>>>(b);
+    else k1_kernel<P, false>()<<<total, K1Cfg<T, false>::TX * K1Cfg<T, false>::TY * 32, smem, s>>>(b);
 }
 
+// Whether the micro update takes its one case as a kernel parameter: explicit strips of two columns (the wider and the
+// implicit instances, short of registers, spill more that way: 8.7 against 10.3 ms, 128x128, 64x64, N_T 11)
+inline bool k4_one(int ncases, bool imp, March m) { return ncases == 1 && !imp && m.cols == 2; }
+
 // the explicit-only kernels unless a case of the handle takes the spectral source at the new iterate
-template <typename T>
-void launch_k4(bool imp, March m, int nt, int total, size_t smem, Batch<T> b, cudaStream_t s)
+template <class P>
+void launch_k4(bool imp, March m, int nt, int groups, int total, const P& b, cudaStream_t s)
 {
-    constexpr int P = K4_VPL<T>;
+    using T = typename P::value_type;
+    constexpr int L = K4_VPL<T>;
+    const size_t smem = groups * k4_smem_of<T>(m.cols, nt, imp);
     auto go = [&](auto plain, auto implicit) {
-        if (imp) implicit<<<total, nt * 32, smem, s>>>(b, m.rows);
-        else plain<<<total, nt * 32, smem, s>>>(b, m.rows);
+        if (imp) implicit<<<total, groups * nt * 32, smem, s>>>(b, m.rows, groups);
+        else plain<<<total, groups * nt * 32, smem, s>>>(b, m.rows, groups);
     };
-    if (m.cols == 2) go(k4_march<T, 2, P, false, K4_T2>, k4_march<T, 2, P, true, K4_T2>);
-    else if (nt <= K4_NT4) go(k4_march<T, 4, P, false, K4_T4>, k4_march<T, 4, P, true, K4_T4>);
-    else go(k4_march<T, 4, P, false, K4_T4L>, k4_march<T, 4, P, true, K4_T4L>);
+    if constexpr (!std::is_same<P, Batch<T>>::value) {
+        go(k4_march<P, 2, L, false, K4_T2>, k4_march<P, 2, L, false, K4_T2>);   // k4_one
+    } else {
+        if (m.cols == 2) go(k4_march<P, 2, L, false, K4_T2>, k4_march<P, 2, L, true, K4_T2>);
+        else if (nt <= K4_NT4) go(k4_march<P, 4, L, false, K4_T2>, k4_march<P, 4, L, true, K4_T2>);
+        else go(k4_march<P, 4, L, false, K4_T4L>, k4_march<P, 4, L, true, K4_T4L>);
+    }
 }
 
 // every K4 shape may be chosen later (autotuning), so each gets the largest dynamic shared memory it can use
-template <typename T>
+template <class P>
 cudaError_t set_smem_attributes()
 {
-    const int big = (int)SMEM_MAX;
-    cudaError_t e = cudaFuncSetAttribute(k1_kernel<T, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)k1_smem_of<T>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k1_kernel<T, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)k1_smem_of<T>());
-    auto set = [&](auto k) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+    using T = typename P::value_type;
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto k, size_t bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    constexpr int P = K4_VPL<T>;
-    set(k4_march<T, 2, P, false, K4_T2>); set(k4_march<T, 2, P, true, K4_T2>);
-    set(k4_march<T, 4, P, false, K4_T4>); set(k4_march<T, 4, P, true, K4_T4>);
-    set(k4_march<T, 4, P, false, K4_T4L>); set(k4_march<T, 4, P, true, K4_T4L>);
+    set(k1_kernel<P, false>(), k1_smem_of<T, false>());
+    set(k1_kernel<P, true>(), k1_smem_of<T, true>());
+    constexpr int L = K4_VPL<T>;
+    set(k4_march<P, 2, L, false, K4_T2>, SMEM_MAX);
+    if constexpr (std::is_same<P, Batch<T>>::value) {
+        set(k4_march<P, 2, L, true, K4_T2>, SMEM_MAX);
+        set(k4_march<P, 4, L, false, K4_T2>, SMEM_MAX); set(k4_march<P, 4, L, true, K4_T2>, SMEM_MAX);
+        set(k4_march<P, 4, L, false, K4_T4L>, SMEM_MAX); set(k4_march<P, 4, L, true, K4_T4L>, SMEM_MAX);
+    }
     return e;
 }
 
@@ -796,9 +846,35 @@ cudaError_t set_smem_attributes()
 // equilibrium tables), 3 micro update, 4 residual.
 inline int profile_slot(int kind) { return kind == 0 ? 0 : kind == 1 ? 1 : kind == 2 ? 2 : 3; }
 
+template <typename T>
+void launch_spec(Impl<T>& im, const LaunchSpec& sp, const Batch<T>& b, cudaStream_t s)
+{
+    const bool one = b.ncases == 1;
+    switch (sp.kind) {
+        case 0:
+            if (one) launch_k1(sp.shape, sp.total, sp.smem, One<T>{im.dc[0]}, s);
+            else launch_k1(sp.shape, sp.total, sp.smem, b, s);
+            break;
+        case 1: k2_face_params<T><<<sp.total, K2_ITEMS * K2_WARPS, 0, s>>>(b); break;
+        case 2: {
+            Range rt("k_tables");          // the same launch writes the equilibrium tables
+            k3_macro<T><<<sp.total, k3_threads(im.max_nt), 0, s>>>(b);
+            break;
+        }
+        case 4:
+            if (k4_one(b.ncases, im.any_implicit, sp.march))
+                launch_k4(im.any_implicit, sp.march, sp.nt, sp.groups, sp.total, One<T>{im.dc[0]}, s);
+            else
+                launch_k4(im.any_implicit, sp.march, sp.nt, sp.groups, sp.total, b, s);
+            break;
+        case 5: k_steps<T><<<sp.total, 128, 0, s>>>(b); break;
+    }
+}
+
 // one iteration; with `ev` (2 events per kernel kind, 5 kinds) each kind is bracketed by an event pair
 template <typename T>
-void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev = nullptr)
+void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev = nullptr,
+                       const cudaGraphConditionalHandle* loop = nullptr)
 {
     const int stride = ncases + 1;
     int open_slot = -1;
@@ -810,19 +886,10 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
             cudaEventRecord(ev[2 * slot], s);
             open_slot = slot;
         }
-        Batch<T> b{im.d_cases, ncases, im.d_off + (size_t)sp.table * stride};
         static const char* const names[5] = {"k1_cells", "k2_face_params", "k3_macro", "", "k4_cells"};
         Range r(names[sp.kind]);
-        switch (sp.kind) {
-            case 0: launch_k1<T>(sp.shape, sp.total, sp.smem, b, s); break;
-            case 1: k2_face_params<T><<<sp.total, K2_ITEMS * K2_WARPS, 0, s>>>(b); break;
-            case 2: {
-                Range rt("k_tables");          // the same launch writes the equilibrium tables
-                k3_macro<T><<<sp.total, k3_threads(im.max_nt), 0, s>>>(b);
-                break;
-            }
-            case 4: launch_k4<T>(im.any_implicit, sp.march, sp.nt, sp.total, sp.smem, b, s); break;
-        }
+        const Batch<T> b{im.d_cases, ncases, im.d_off + (size_t)sp.table * stride};
+        launch_spec(im, sp, b, s);
     }
     if (ev) {
         cudaEventRecord(ev[2 * open_slot + 1], s);
@@ -830,7 +897,12 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
     }
     {
         Range r("k5_finish");
-        k5_finish<T><<<ncases, K5_THREADS, 0, s>>>(im.d_cases, ncases, im.d_off + (size_t)im.k3_table * stride);
+        const int* off = im.d_off + (size_t)im.k3_table * stride;
+        if (loop)
+            k5_finish<T, true><<<ncases, K5_THREADS, 0, s>>>(im.d_cases, ncases, off,
+                                                             LoopTest{*loop, im.d_loop, im.d_status, im.d_err});
+        else
+            k5_finish<T, false><<<ncases, K5_THREADS, 0, s>>>(im.d_cases, ncases, off, LoopTest{});
     }
     if (ev) cudaEventRecord(ev[9], s);
 }
@@ -839,7 +911,7 @@ template <typename T>
 void enqueue_steps(Impl<T>& im, int ncases, cudaStream_t s)
 {
     const LaunchSpec& sp = im.specs[im.steps_table];
-    if (sp.total) k_steps<T><<<sp.total, 128, 0, s>>>(Batch<T>{im.d_cases, ncases, im.d_off + (size_t)sp.table * (ncases + 1)});
+    if (sp.total) launch_spec(im, sp, Batch<T>{im.d_cases, ncases, im.d_off + (size_t)sp.table * (ncases + 1)}, s);
 }
 
 hbugks_status begin(hbugks_t h)
@@ -872,7 +944,7 @@ hbugks_status capture(hbugks_t h, Impl<T>& im)
         (which == 0 ? h->g1 : h->gN) = ex;
     }
     // The pseudo-time loop on the device: a graph holding one conditional while node, whose body is one
-    // iteration followed by the loop test; one launch runs up to the requested number of iterations and stops
+    // iteration, the loop test in its last kernel; one launch runs up to the requested number of iterations and stops
     // by itself once every case has converged (or diverged, or a wait failed), with no host round trip.
     cudaGraph_t g;
     HB_CK(cudaGraphCreate(&g, 0));
@@ -894,8 +966,7 @@ hbugks_status capture(hbugks_t h, Impl<T>& im)
     HB_CK(cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &np));
     cudaGraph_t body = np.conditional.phGraph_out[0];
     HB_CK(cudaStreamBeginCaptureToGraph(h->s, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_iteration(im, h->ncases, h->s);
-    k_loop_test<<<1, 32, 0, h->s>>>(hc, im.d_loop, im.d_status, h->ncases, im.d_err);
+    enqueue_iteration(im, h->ncases, h->s, nullptr, &hc);
     HB_CK(cudaStreamEndCapture(h->s, &body));
     HB_CK(cudaGraphInstantiate(&h->gW, g, 0));
     return HBUGKS_OK;
@@ -980,14 +1051,18 @@ hbugks_status autotune(hbugks_t h, Impl<T>& im, int ncases)
             for (int sh = 0; sh < N_K4_SHAPES; ++sh) {
                 if (!k4_shape_ok<T>(sh, hc.nt, hc.pairs != 0)) continue;
                 const bool imp = im.any_implicit;
-                const March m = k4_march_of<T>(sh, hc.nx, hc.nt, imp);
-                const size_t smem = k4_smem_of<T>(m.cols, hc.nt, imp);
-                const int off[2] = {0, k4_blocks<T>(hc, m)};
+                const March m = k4_march_of<T>(sh, hc.nx, hc.nt, hc.nu + hc.nv, imp);
+                const int total = k4_groups<T>(hc, m), per = k4_groups_per_cta<T>(m, hc.nt, imp, total);
+                const int off[2] = {0, (total + per - 1) / per};
                 HB_CK(cudaMemcpyAsync(im.d_tune_off, off, sizeof off, cudaMemcpyHostToDevice, h->s));
                 const Batch<T> b{im.d_cases + k, 1, im.d_tune_off};
-                launch_k4<T>(imp, m, hc.nt, off[1], smem, b, h->s);
+                auto run = [&]() {
+                    if (k4_one(ncases, imp, m)) launch_k4(imp, m, hc.nt, per, off[1], One<T>{im.dc[k]}, h->s);
+                    else launch_k4(imp, m, hc.nt, per, off[1], b, h->s);
+                };
+                run();
                 HB_CK(cudaEventRecord(e0, h->s));
-                for (int r = 0; r < 3; ++r) launch_k4<T>(imp, m, hc.nt, off[1], smem, b, h->s);
+                for (int r = 0; r < 3; ++r) run();
                 HB_CK(cudaEventRecord(e1, h->s));
                 HB_CK(cudaEventSynchronize(e1));
                 float ms = 0.f;
@@ -1010,7 +1085,8 @@ hbugks_status do_create(hbugks_t h, Impl<T>& im, int ncases, const hbugks_case* 
     for (auto& hc : im.hc) {
         if (hc.k4shape < 0) return HBUGKS_EINVAL;
     }
-    HB_CK(set_smem_attributes<T>());
+    HB_CK(set_smem_attributes<Batch<T>>());
+    HB_CK(set_smem_attributes<One<T>>());
     std::vector<std::vector<char>> keep;
     for (int k = 0; k < ncases; ++k) HB_CK(upload_case(im.hc[k], im.dc[k], h->s, keep));
     HB_CK(cudaMemcpyAsync(im.d_cases, im.dc.data(), sizeof(CaseDev<T>) * ncases, cudaMemcpyHostToDevice, h->s));
@@ -1054,7 +1130,7 @@ template <typename T>
 hbugks_status launch_loop(hbugks_t h, Impl<T>& im, int n)
 {
     if (n <= 0) return HBUGKS_OK;
-    k_set_int<<<1, 1, 0, h->s>>>(im.d_loop, n);
+    k_set_loop<<<1, 1, 0, h->s>>>(im.d_loop, n);
     HB_CK(cudaGraphLaunch(h->gW, h->s));
     return HBUGKS_OK;
 }
@@ -1651,7 +1727,7 @@ int hbugks_launches_per_iteration(hbugks_t h)
 {
     if (!h) return -1;
     return dispatch(h, [&](auto& im) -> int {
-        int n = h->loop_mode == 0 ? 2 : 1;   // residual kernel (and the loop test of the device-side loop)
+        int n = 1;                           // residual kernel (with the loop test of the device-side loop)
         for (auto& sp : im.specs)
             if (sp.kind != 5 && sp.total) ++n;
         return n;

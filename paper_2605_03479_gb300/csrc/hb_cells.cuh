@@ -28,6 +28,8 @@ __device__ __forceinline__ float rcp_approx(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// (All products that feed a sum are written as fused ones here and in hb_micro.cuh, so that every instance of a kernel,
+// whether it finds its case in a table or as a parameter, rounds alike.)
 // The arguments are twice the one-sided slopes, so that the limited slope 2 s1 s2 / (s1 + s2) is their product over
 // their sum.
 __device__ __forceinline__ float2 vleer2(float2 s1, float2 s2)
@@ -97,6 +99,26 @@ __device__ __forceinline__ T lane_totals(T (&v)[N], int lane)
     return x[0];
 }
 
+// N parameters (a multiple of 4) from shared memory by 16-byte loads
+template <int N>
+__device__ __forceinline__ void load_par(const float* p, float (&o)[N])
+{
+#pragma unroll
+    for (int k = 0; k < N; k += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(p + k);
+        o[k] = x.x; o[k + 1] = x.y; o[k + 2] = x.z; o[k + 3] = x.w;
+    }
+}
+template <int N>
+__device__ __forceinline__ void load_par(const double* p, double (&o)[N])
+{
+#pragma unroll
+    for (int k = 0; k < N; k += 2) {
+        const double2 x = *reinterpret_cast<const double2*>(p + k);
+        o[k] = x.x; o[k + 1] = x.y;
+    }
+}
+
 // ------------------------------------------------------------------------------ K1: half-face sums
 
 // Velocity sums of one cell's reconstruction at its downwind faces.  Slots of the 23 sums (as for an
@@ -118,25 +140,32 @@ __device__ __forceinline__ T lane_totals(T (&v)[N], int lane)
 // w u^a v^b d factors into w_u u^a (the lane's) times sum over the lane's velocities of w_v v^b d, and the lane
 // keeps only those v-moments (20 sums: of f0 v^0..3 for h and v^0..1 for b, of s_x the same, of s_y v^0..4 and
 // v^0..2), multiplying by w_u u^a when the class changes.
-// Bound by FP64 instructions in FP64 (67 per velocity with SEP, the limiter's reciprocals included) and by
-// instruction issue in FP32.  Against 59 sums with the reconstruction formed per velocity and divisions in the
-// limiter: 36.98 -> 23.19 ms (twelve 64x64 cavities, 32x32 velocities, N_T 3, FP64, SEP), 18.22 -> 12.81 ms (64x64,
-// 48x48, N_T 7, FP64), 4.83 -> 4.19 ms (128x128, 64x64, N_T 11, FP32, SEP), 0.543 -> 0.518 ms (64x64, 48x48, FP32).
-template <typename T, int TX, int TY, int G, int S, bool SEP>
-__global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8) ? 2 : 1) k1_cells(Batch<T> B)
+// Bound by FP64 instructions in FP64 (62 per velocity with SEP, the limiter's reciprocals included); in FP32 by waiting
+// for the staged blocks (three times the tile's own cells pass from L2) at 56 % issue.  Against 59 sums with the
+// reconstruction formed per velocity, divisions in the limiter and weights formed per lane from two loads: 36.98 ->
+// 22.2 ms (twelve 64x64 cavities, 32x32 velocities, N_T 3, FP64, SEP), 18.22 -> 11.3 ms (64x64, 48x48, N_T 7, FP64),
+// 4.83 -> 3.34 ms (128x128, 64x64, N_T 11, FP32, SEP), 0.543 -> 0.463 ms (64x64, 48x48, FP32).  Tiles of 4x2 cells:
+// 4x4 4.11 ms, 6x4 3.96, 8x3 4.14 on the 128x128 case, whose larger CTAs wait for their slowest warp.
+// Weights of a velocity block in global and shared memory, T [K1_WT]: SEP four per lane (w_v v^0..3), then w_v v^4 per
+// lane; general four, four and four per lane (w times 1, u, v, uu; uv, vv, uuu, uuv; uvv, vvv, uu|u|^2, vv|u|^2), then
+// w uv|u|^2 per lane.  Products formed in FP64 when the case is uploaded.
+template <bool SEP> constexpr int K1_WT = SEP ? 160 : 416;
+
+template <class P, int TX, int TY, int G, int S, bool SEP, int CTAS>
+__global__ void __launch_bounds__(TX * TY * 32, CTAS) k1_cells(const __grid_constant__ P B)
 {
+    using T = typename P::value_type;
     using V = P2<T>;
     constexpr int PX = TX + 2, PY = TY + 2, NR = PX * PY, NWC = TX * TY;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ uint64_t bars[S], empty[S];
     __shared__ T sacc[NWC][4][NM];
     __shared__ int abort_flag;                               // set by the first warp whose wait runs out
-    const int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
+    int lb;
+    const CaseDev<T>& cd = B.find(blockIdx.x, lb);
     if (!cd.st->active) return;
     // another CTA may set the error word while this one starts: decide for the whole CTA at once
     if (__syncthreads_or(*(volatile int*)cd.err != 0)) return;
-    const int lb = blockIdx.x - B.off[cs];
     const int ntx = (cd.nx + TX - 1) / TX, nty = (cd.ny + TY - 1) / TY;
     const int tx = lb % ntx, ty = (lb / ntx) % nty, n = lb / (ntx * nty);
     const int i0 = tx * TX, j0 = ty * TY;
@@ -150,9 +179,10 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
         for (int k = 0; k < S; ++k) mbar_init(empty + k, NWC);   // one arrival per warp: slot read
     }
     mbar_setup(bars, S);
-    // staged rectangle: columns i0-1 .. i0+TX, rows j0-1 .. j0+TY; S buffers [G][NR][32] of (h, b) pairs
+    // staged rectangle: columns i0-1 .. i0+TX, rows j0-1 .. j0+TY; S slots of [G][NR][32] (h, b) pairs
     constexpr size_t blk = (size_t)NR * VB;
-    V* buf = reinterpret_cast<V*>(smem_raw);
+    constexpr int WT = K1_WT<SEP>;
+    constexpr size_t SLOT = G * (blk * sizeof(V) + WT * sizeof(T));   // bytes: G blocks, then their weights
     const int p = cd.st->parity;
     const V* gf = cd.f[p];
     const int c0 = max(i0 - 1, 0), c1 = min(i0 + TX + 1, nx);
@@ -162,20 +192,33 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
         const int jj = j0 - 1 + r;
         if (jj >= 0 && jj < ny) rbytes += row_b;
     }
-    const int nchunk = (nvb + G - 1) / G;
+    // chunks of up to G blocks of one sign class (the classes occupy consecutive blocks)
+    int nchunk = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) nchunk += (cd.cls_end[c] - (c ? cd.cls_end[c - 1] : 0) + G - 1) / G;
     int* err = cd.err;
+    int pvb = 0, pcls = 0;                                   // next block to copy and its class (warp 0)
     auto issue = [&](int k) {
-        const int vb0 = k * G, gk = min(G, nvb - vb0);
-        V* dst = buf + (size_t)(k % S) * G * blk;
-        if (lane == 0) mbar_arrive_expect(&bars[k % S], (uint32_t)gk * rbytes);
+        while (pvb >= cd.cls_end[pcls]) ++pcls;
+        const int gk = min(G, cd.cls_end[pcls] - pvb);
+        unsigned char* dst = smem_raw + (size_t)(k % S) * SLOT;
+        const uint32_t wb = (uint32_t)(gk * WT * (int)sizeof(T));
+        if (lane == 0) mbar_arrive_expect(&bars[k % S], (uint32_t)gk * rbytes + wb);
         __syncwarp();
-        for (int q = lane; q < gk * PY; q += 32) {
+        for (int q = lane; q <= gk * PY; q += 32) {
+            if (q == gk * PY) {
+                bulk_g2s(dst + G * blk * sizeof(V), cd.wrow + (size_t)pvb * WT, wb, &bars[k % S]);
+                break;
+            }
             const int r = q % PY, g = q / PY;
             const int jj = j0 - 1 + r;
             if (jj < 0 || jj >= ny) continue;
-            const size_t src = ((size_t)(vb0 + g) * nt + n) * nc * VB + ((size_t)jj * nx + c0) * VB;
-            bulk_g2s(dst + (size_t)g * blk + (size_t)(r * PX + c0 - (i0 - 1)) * VB, gf + src, row_b, &bars[k % S]);
+            const size_t src = ((size_t)(pvb + g) * nt + n) * nc * VB + ((size_t)jj * nx + c0) * VB;
+            bulk_g2s(dst + ((size_t)g * blk + (size_t)(r * PX + c0 - (i0 - 1)) * VB) * sizeof(V), gf + src, row_b,
+                     &bars[k % S]);
         }
+        __syncwarp();
+        pvb += gk;
     };
     if (warp == 0)
         for (int k = 0; k < S - 1 && k < nchunk; ++k) issue(k);
@@ -194,10 +237,6 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
     const T hxh = valid ? T(cd.hx[i]) : T(0), hyh = valid ? T(cd.hy[j]) : T(0);
     const bool inner = hm && hp && vm && vp;                 // every neighbour present: no wall branches
     const int kc = (tj + 1) * PX + ti + 1;
-    const T* __restrict__ tu = cd.tu;
-    const T* __restrict__ tv = cd.tv;
-    const T* __restrict__ tw = SEP ? cd.twv : cd.tw;       // SEP: the v-factor w_v of each weight
-
     // A sum of h and the sum of b with the same weight are kept as one pair (one packed FMA), the others of h alone:
     //   SEP      f: pairs v^0 v^1, h v^2 v^3;  x: the same;  y: pairs v^0 v^1 v^2, h v^3 v^4
     //   general  f: pairs 1 u v, h uu uv vv uuu uuv uvv vvv;  x: pairs 1 u v uu uv, h vv uuu uuv uvv vvv uu|u|^2 uv|u|^2;
@@ -227,7 +266,7 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
     zero_sums();
 #pragma unroll
     for (int q = 0; q < NCM; ++q) ac[q] = T(0);
-    int cur = -1, cend = 0;                                  // current sign class, the first block past it
+    int cur = 0;                                             // current sign class
     T ul = T(0), wul = T(0);                                 // SEP: the lane's u and w_u in the current class
     // the 23 face sums of one face from its v-moments (SEP): D, DB of d0 and e0, S, SB tangential slopes, N, NB normal
     auto unfold = [&](const T (&D)[4], const T (&DB)[2], const T (&S_)[3], T SB, const T (&N)[3], T NB, T (&o)[NM]) {
@@ -235,9 +274,9 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
         o[0] = w1 * D[0]; o[1] = w2 * D[0]; o[2] = w1 * D[1]; o[3] = w3 * D[0]; o[4] = w2 * D[1];
         o[5] = w1 * D[2]; o[6] = w4 * D[0]; o[7] = w3 * D[1]; o[8] = w2 * D[2]; o[9] = w1 * D[3];
         o[10] = w1 * DB[0]; o[11] = w2 * DB[0]; o[12] = w1 * DB[1];
-        o[13] = w1 * S_[0]; o[14] = w2 * S_[0]; o[15] = w1 * S_[1]; o[16] = w3 * S_[0] + w1 * S_[2];
+        o[13] = w1 * S_[0]; o[14] = w2 * S_[0]; o[15] = w1 * S_[1]; o[16] = pfma(w3, S_[0], w1 * S_[2]);
         o[17] = w1 * SB;
-        o[18] = w1 * N[0]; o[19] = w2 * N[0]; o[20] = w1 * N[1]; o[21] = w3 * N[0] + w1 * N[2];
+        o[18] = w1 * N[0]; o[19] = w2 * N[0]; o[20] = w1 * N[1]; o[21] = pfma(w3, N[0], w1 * N[2]);
         o[22] = w1 * NB;
     };
     // add the sums of the current sign class to its two half-face slots and to the cell's moments
@@ -250,24 +289,24 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
             const T Y[5] = {yp[0].x, yp[1].x, yp[2].x, ys[0], ys[1]}, YB[3] = {yp[0].y, yp[1].y, yp[2].y};
             T D[4], DB[2], S_[3], N[3];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) D[q] = F[q] + sx_ * X[q];
+            for (int q = 0; q < 4; ++q) D[q] = pfma(sx_, X[q], F[q]);
 #pragma unroll
-            for (int q = 0; q < 2; ++q) DB[q] = FB[q] + sx_ * XB[q];
+            for (int q = 0; q < 2; ++q) DB[q] = pfma(sx_, XB[q], FB[q]);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) { S_[q] = Y[q]; N[q] = ul * (ul * X[q] + Y[q + 1]); }
-            unfold(D, DB, S_, YB[0], N, ul * (ul * XB[0] + YB[1]), ox);
+            for (int q = 0; q < 3; ++q) { S_[q] = Y[q]; N[q] = ul * pfma(ul, X[q], Y[q + 1]); }
+            unfold(D, DB, S_, YB[0], N, ul * pfma(ul, XB[0], YB[1]), ox);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) D[q] = F[q] + sy_ * Y[q];
+            for (int q = 0; q < 4; ++q) D[q] = pfma(sy_, Y[q], F[q]);
 #pragma unroll
-            for (int q = 0; q < 2; ++q) DB[q] = FB[q] + sy_ * YB[q];
+            for (int q = 0; q < 2; ++q) DB[q] = pfma(sy_, YB[q], FB[q]);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) { S_[q] = X[q]; N[q] = ul * X[q + 1] + Y[q + 2]; }
-            unfold(D, DB, S_, XB[0], N, ul * XB[1] + YB[2], oy);
+            for (int q = 0; q < 3; ++q) { S_[q] = X[q]; N[q] = pfma(ul, X[q + 1], Y[q + 2]); }
+            unfold(D, DB, S_, XB[0], N, pfma(ul, XB[1], YB[2]), oy);
             const T w1 = wul, w2 = w1 * ul, w3 = w2 * ul, w4 = w3 * ul;
-            ac[0] += w1 * F[0]; ac[1] += w2 * F[0]; ac[2] += w1 * F[1]; ac[3] += w3 * F[0];
-            ac[4] += w2 * F[1]; ac[5] += w1 * F[2]; ac[6] += w4 * F[0]; ac[7] += w3 * F[1];
-            ac[8] += w2 * F[2]; ac[9] += w1 * F[3];
-            ac[10] += w1 * FB[0]; ac[11] += w2 * FB[0]; ac[12] += w1 * FB[1];
+            ac[0] = pfma(w1, F[0], ac[0]); ac[1] = pfma(w2, F[0], ac[1]); ac[2] = pfma(w1, F[1], ac[2]); ac[3] = pfma(w3, F[0], ac[3]);
+            ac[4] = pfma(w2, F[1], ac[4]); ac[5] = pfma(w1, F[2], ac[5]); ac[6] = pfma(w4, F[0], ac[6]); ac[7] = pfma(w3, F[1], ac[7]);
+            ac[8] = pfma(w2, F[2], ac[8]); ac[9] = pfma(w1, F[3], ac[9]);
+            ac[10] = pfma(w1, FB[0], ac[10]); ac[11] = pfma(w2, FB[0], ac[11]); ac[12] = pfma(w1, FB[1], ac[12]);
         } else {
             // monomials 1, u, v, uu, uv, vv, uuu, uuv, uvv, vvv
             const T F[10] = {fp_[0].x, fp_[1].x, fp_[2].x, fs_[0], fs_[1], fs_[2], fs_[3], fs_[4], fs_[5], fs_[6]};
@@ -275,14 +314,14 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
             const T Y[10] = {yp[0].x, yp[1].x, yp[2].x, ys[0], yp[3].x, yp[4].x, ys[1], ys[2], ys[3], ys[4]};
 #pragma unroll
             for (int q = 0; q < 10; ++q) {
-                ox[q] = F[q] + sx_ * X[q];
-                oy[q] = F[q] + sy_ * Y[q];
+                ox[q] = pfma(sx_, X[q], F[q]);
+                oy[q] = pfma(sy_, Y[q], F[q]);
                 ac[q] += F[q];
             }
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                ox[10 + q] = fp_[q].y + sx_ * xp[q].y;
-                oy[10 + q] = fp_[q].y + sy_ * yp[q].y;
+                ox[10 + q] = pfma(sx_, xp[q].y, fp_[q].y);
+                oy[10 + q] = pfma(sy_, yp[q].y, fp_[q].y);
                 ac[10 + q] += fp_[q].y;
                 ox[13 + q] = Y[q];
                 oy[13 + q] = X[q];
@@ -307,110 +346,109 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
     // Ring of S slots: chunk k lands in slot k % S (mbarrier bars); each warp arrives on empty once it has
     // read the slot, and warp 0 refills a slot only after every warp has released it, so warps run up to
     // S - 1 chunks apart instead of meeting at a CTA barrier per chunk.
-    for (int k = 0; k < nchunk; ++k) {
-        if (warp == 0 && k + S - 1 < nchunk) {
-            const int kk = k + S - 1;
-            if (kk >= S && !mbar_wait(&empty[kk % S], (uint32_t)((kk / S - 1) & 1), err, &abort_flag)) {
+    int k = 0, slot = 0, vb = 0;                             // chunk, its slot, its first block
+    uint32_t ph = 0;                                         // phase of the slot's barrier
+    for (cur = 0; cur < 4; ++cur) {
+        const int vend = cd.cls_end[cur];
+        if (vb >= vend) continue;
+        if (SEP) {
+            ul = __ldg(cd.tu + vb * VB + lane);
+            wul = __ldg(cd.twu + vb * VB + lane);
+        }
+        for (; vb < vend; vb += G, ++k) {
+            if (warp == 0 && k + S - 1 < nchunk) {
+                const int kk = k + S - 1;
+                if (kk >= S && !mbar_wait(&empty[kk % S], (uint32_t)((kk / S - 1) & 1), err, &abort_flag)) {
+                    give_up(k);
+                    return;
+                }
+                issue(kk);
+                issued = kk + 1;
+            }
+            if (!mbar_wait(&bars[slot], ph, err, &abort_flag)) {
                 give_up(k);
                 return;
             }
-            issue(kk);
-            issued = kk + 1;
-        }
-        if (!mbar_wait(&bars[k % S], (uint32_t)((k / S) & 1), err, &abort_flag)) {
-            give_up(k);
-            return;
-        }
-        const V* cb = buf + (size_t)(k % S) * G * blk;
-        const int vb0 = k * G, gk = min(G, nvb - vb0);
-        // the blocks of the chunk; INNER: every neighbour of the warp's cell exists (no wall branches)
-        auto run_blocks = [&](auto inner_tag) {
-            constexpr bool INNER = decltype(inner_tag)::value;
-            // the velocities of block g + 1 are loaded while block g is summed
-            // (SEP reads u only where the class changes)
-            T nu_ = SEP ? T(0) : __ldg(tu + vb0 * VB + lane), nv_ = __ldg(tv + vb0 * VB + lane),
-              nw_ = __ldg(tw + vb0 * VB + lane);
-            for (int g = 0; g < gk; ++g) {
-                [[maybe_unused]] const T u = nu_;
-                const T v = nv_, w = nw_;
-                if (g + 1 < gk) {
-                    const int a1 = (vb0 + g + 1) * VB + lane;
-                    if (!SEP) nu_ = __ldg(tu + a1);
-                    nv_ = __ldg(tv + a1); nw_ = __ldg(tw + a1);
-                }
-                // the classes occupy consecutive blocks: a new one starts where the current one ends
-                if (vb0 + g >= cend) {
-                    if (cur >= 0) flush();
-                    do {
-                        ++cur;
-                        cend = cd.cls_end[cur];
-                    } while (vb0 + g >= cend);
-                    if (SEP) {
-                        ul = __ldg(tu + (vb0 + g) * VB + lane);
-                        wul = __ldg(cd.twu + (vb0 + g) * VB + lane);
-                    }
-                }
-                const V* ph = cb + (size_t)g * blk + (size_t)kc * VB + lane;
-                const V f0 = ph[0];
+            const unsigned char* cb = smem_raw + (size_t)slot * SLOT;
+            const int gk = min(G, vend - vb);
+            // one block of the chunk; INNER: every neighbour of the warp's cell exists (no wall branches)
+            auto block = [&](auto inner_tag, const V* pc, const T* wp) {
+                constexpr bool INNER = decltype(inner_tag)::value;
+                const V f0 = pc[0];
                 V sxv, syv;
                 if constexpr (INNER) {
-                    sxv = slope2i(ph[-VB], f0, ph[VB], wxm, wxp);
-                    syv = slope2i(ph[-PX * VB], f0, ph[PX * VB], wym, wyp);
+                    sxv = slope2i(pc[-VB], f0, pc[VB], wxm, wxp);
+                    syv = slope2i(pc[-PX * VB], f0, pc[PX * VB], wym, wyp);
                 } else {
-                    sxv = slope2(ph[-VB], f0, ph[VB], wxm, wxp, hm, hp, sx);
-                    syv = slope2(ph[-PX * VB], f0, ph[PX * VB], wym, wyp, vm, vp, sy);
+                    sxv = slope2(pc[-VB], f0, pc[VB], wxm, wxp, hm, hp, sx);
+                    syv = slope2(pc[-PX * VB], f0, pc[PX * VB], wym, wyp, vm, vp, sy);
                 }
-                const T c1 = w * v, c2 = c1 * v, c3 = c2 * v;
+                T a[4];
+                load_par(wp + lane * 4, a);
                 if constexpr (SEP) {
-                    // w is w_v here; v-moments of every summand
-                    const V bw = bc(w), bc1 = bc(c1);
+                    const T c4 = wp[4 * VB + lane];
+                    const V bw = bc(a[0]), bc1 = bc(a[1]);
                     fp_[0] = pfma(f0, bw, fp_[0]); fp_[1] = pfma(f0, bc1, fp_[1]);
                     xp[0] = pfma(sxv, bw, xp[0]); xp[1] = pfma(sxv, bc1, xp[1]);
-                    yp[0] = pfma(syv, bw, yp[0]); yp[1] = pfma(syv, bc1, yp[1]); yp[2] = pfma(syv, bc(c2), yp[2]);
-                    fs_[0] += f0.x * c2; fs_[1] += f0.x * c3;
-                    xs[0] += sxv.x * c2; xs[1] += sxv.x * c3;
-                    ys[0] += syv.x * c3; ys[1] += syv.x * (c3 * v);
+                    yp[0] = pfma(syv, bw, yp[0]); yp[1] = pfma(syv, bc1, yp[1]); yp[2] = pfma(syv, bc(a[2]), yp[2]);
+                    fs_[0] = pfma(f0.x, a[2], fs_[0]); fs_[1] = pfma(f0.x, a[3], fs_[1]);
+                    xs[0] = pfma(sxv.x, a[2], xs[0]); xs[1] = pfma(sxv.x, a[3], xs[1]);
+                    ys[0] = pfma(syv.x, a[3], ys[0]); ys[1] = pfma(syv.x, c4, ys[1]);
                 } else {
-                    const T wu = w * u, wuu = wu * u, wuv = wu * v, wuuu = wuu * u, wuuv = wuu * v, wuvv = wuv * v;
-                    const T r2 = u * u + v * v;
-                    const V bw = bc(w), bu = bc(wu), bv = bc(c1), buv = bc(wuv);
+                    T d[4], e[4];                            // a: 1 u v uu, d: uv vv uuu uuv, e: uvv vvv uu|u|^2 vv|u|^2
+                    load_par(wp + 4 * VB + lane * 4, d);
+                    load_par(wp + 8 * VB + lane * 4, e);
+                    const T wr = wp[12 * VB + lane];
+                    const V bw = bc(a[0]), bu = bc(a[1]), bv = bc(a[2]), buv = bc(d[0]);
                     fp_[0] = pfma(f0, bw, fp_[0]); fp_[1] = pfma(f0, bu, fp_[1]); fp_[2] = pfma(f0, bv, fp_[2]);
                     xp[0] = pfma(sxv, bw, xp[0]); xp[1] = pfma(sxv, bu, xp[1]); xp[2] = pfma(sxv, bv, xp[2]);
-                    xp[3] = pfma(sxv, bc(wuu), xp[3]); xp[4] = pfma(sxv, buv, xp[4]);
+                    xp[3] = pfma(sxv, bc(a[3]), xp[3]); xp[4] = pfma(sxv, buv, xp[4]);
                     yp[0] = pfma(syv, bw, yp[0]); yp[1] = pfma(syv, bu, yp[1]); yp[2] = pfma(syv, bv, yp[2]);
-                    yp[3] = pfma(syv, buv, yp[3]); yp[4] = pfma(syv, bc(c2), yp[4]);
-                    fs_[0] += f0.x * wuu; fs_[1] += f0.x * wuv; fs_[2] += f0.x * c2; fs_[3] += f0.x * wuuu;
-                    fs_[4] += f0.x * wuuv; fs_[5] += f0.x * wuvv; fs_[6] += f0.x * c3;
-                    xs[0] += sxv.x * c2; xs[1] += sxv.x * wuuu; xs[2] += sxv.x * wuuv; xs[3] += sxv.x * wuvv;
-                    xs[4] += sxv.x * c3; xs[5] += sxv.x * (wuu * r2); xs[6] += sxv.x * (wuv * r2);
-                    ys[0] += syv.x * wuu; ys[1] += syv.x * wuuu; ys[2] += syv.x * wuuv; ys[3] += syv.x * wuvv;
-                    ys[4] += syv.x * c3; ys[5] += syv.x * (c2 * r2); ys[6] += syv.x * (wuv * r2);
+                    yp[3] = pfma(syv, buv, yp[3]); yp[4] = pfma(syv, bc(d[1]), yp[4]);
+                    fs_[0] = pfma(f0.x, a[3], fs_[0]); fs_[1] = pfma(f0.x, d[0], fs_[1]); fs_[2] = pfma(f0.x, d[1], fs_[2]); fs_[3] = pfma(f0.x, d[2], fs_[3]);
+                    fs_[4] = pfma(f0.x, d[3], fs_[4]); fs_[5] = pfma(f0.x, e[0], fs_[5]); fs_[6] = pfma(f0.x, e[1], fs_[6]);
+                    xs[0] = pfma(sxv.x, d[1], xs[0]); xs[1] = pfma(sxv.x, d[2], xs[1]); xs[2] = pfma(sxv.x, d[3], xs[2]); xs[3] = pfma(sxv.x, e[0], xs[3]);
+                    xs[4] = pfma(sxv.x, e[1], xs[4]); xs[5] = pfma(sxv.x, e[2], xs[5]); xs[6] = pfma(sxv.x, wr, xs[6]);
+                    ys[0] = pfma(syv.x, a[3], ys[0]); ys[1] = pfma(syv.x, d[2], ys[1]); ys[2] = pfma(syv.x, d[3], ys[2]); ys[3] = pfma(syv.x, e[0], ys[3]);
+                    ys[4] = pfma(syv.x, e[1], ys[4]); ys[5] = pfma(syv.x, e[3], ys[5]); ys[6] = pfma(syv.x, wr, ys[6]);
                     if constexpr (!INNER) {
-                        // a velocity parallel to a wall carries nothing into it
+                        // a velocity parallel to a wall (u^2 w = 0) carries nothing into it
                         const bool xn = (cur & 1) != 0, yn = (cur & 2) != 0;
-                        if ((xn ? !hm : !hp) && u == T(0)) {
-                            const V d = pfma(sxv, bc(xn ? -hxh : hxh), f0);
-                            zxp[0] = pfma(d, bw, zxp[0]); zxp[1] = pfma(d, bv, zxp[1]);
-                            zxs[0] += d.x * c2; zxs[1] += d.x * c3;
+                        if ((xn ? !hm : !hp) && a[3] == T(0)) {
+                            const V z = pfma(sxv, bc(xn ? -hxh : hxh), f0);
+                            zxp[0] = pfma(z, bw, zxp[0]); zxp[1] = pfma(z, bv, zxp[1]);
+                            zxs[0] = pfma(z.x, d[1], zxs[0]); zxs[1] = pfma(z.x, e[1], zxs[1]);
                         }
-                        if ((yn ? !vm : !vp) && v == T(0)) {
-                            const V d = pfma(syv, bc(yn ? -hyh : hyh), f0);
-                            zyp[0] = pfma(d, bw, zyp[0]); zyp[1] = pfma(d, bu, zyp[1]);
-                            zys[0] += d.x * wuu; zys[1] += d.x * wuuu;
+                        if ((yn ? !vm : !vp) && d[1] == T(0)) {
+                            const V z = pfma(syv, bc(yn ? -hyh : hyh), f0);
+                            zyp[0] = pfma(z, bw, zyp[0]); zyp[1] = pfma(z, bu, zyp[1]);
+                            zys[0] = pfma(z.x, a[3], zys[0]); zys[1] = pfma(z.x, d[2], zys[1]);
                         }
                     }
                 }
+            };
+            auto run_blocks = [&](auto inner_tag) {
+                const V* pc = reinterpret_cast<const V*>(cb) + (size_t)kc * VB + lane;
+                const T* wp = reinterpret_cast<const T*>(cb + G * blk * sizeof(V));
+                if (gk == G) {
+#pragma unroll
+                    for (int g = 0; g < G; ++g) block(inner_tag, pc + g * blk, wp + g * WT);
+                } else {
+                    for (int g = 0; g < gk; ++g) block(inner_tag, pc + g * blk, wp + g * WT);
+                }
+            };
+            if (valid) {
+                if (inner) run_blocks(std::true_type{});
+                else run_blocks(std::false_type{});
             }
-        };
-        if (valid) {
-            if (inner) run_blocks(std::true_type{});
-            else run_blocks(std::false_type{});
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[slot]);
+            if (++slot == S) { slot = 0; ph ^= 1; }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[k % S]);
+        vb = vend;
+        if (valid) flush();
     }
     if (!valid) return;
-    if (cur >= 0) flush();
     const T cm = lane_totals<NCM>(ac, lane);
     __syncwarp();
     const int c = j * nx + i;
@@ -419,10 +457,10 @@ __global__ void __launch_bounds__(TX * TY * 32, (sizeof(T) == 4 && TX * TY == 8)
     for (int k = lane; k < 4 * NM; k += 32) hmo[k] = (double)sacc[warp][k / NM][k % NM];
 }
 
-template <typename T, int TX, int TY, int G, int S>
+template <typename T, int TX, int TY, int G, int S, bool SEP>
 constexpr size_t k1_cells_smem()
 {
-    return (size_t)S * G * (TX + 2) * (TY + 2) * VB * sizeof(P2<T>);
+    return (size_t)S * G * ((TX + 2) * (TY + 2) * VB * sizeof(P2<T>) + K1_WT<SEP> * sizeof(T));
 }
 
 }  // namespace hb

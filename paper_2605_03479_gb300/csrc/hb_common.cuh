@@ -61,6 +61,15 @@ __device__ __forceinline__ float2 psub(float2 a, float2 b)
 }
 __device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
+// the same on one value
+__device__ __forceinline__ float pfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double pfma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float pmul(float a, float b) { return a * b; }
+// (kept apart from a following addition, so that every instance of the kernel rounds alike)
+__device__ __forceinline__ double pmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float padd(float a, float b) { return a + b; }
+__device__ __forceinline__ double padd(double a, double b) { return __dadd_rn(a, b); }
+
 // Face parameter slots of the micro flux (delta form).  For an interface velocity u = (u, v) with normal
 // component u_n, the Maxwellian part of the time-integrated flux divided by dG_f is
 //   h: C1' dH + H Q(u, v),   b: C1' dB + B (Q(u, v) + l0 + l1 u + l2 v)
@@ -70,7 +79,7 @@ __device__ __forceinline__ double2 psub(double2 a, double2 b) { return make_doub
 // Cubic monomial order: 1, u, v, u^2, uv, v^2, u^3, u^2 v, u v^2, v^3.  Blocks start on multiples of 4.
 enum FP {
     F_QL = 0, F_QR = 12, F_LBL = 24, F_LBR = 28, F_RM1 = 32, F_R = 33, F_I2L = 34, F_DI2L = 35,
-    F_C1 = 36, F_C4 = 37, F_C5 = 38, F_NIN = 39, F_WRM1 = 40, F_WR = 41, F_WI2L = 42, F_WDI2L = 43
+    F_C1 = 36, F_C4 = 37, F_C5 = 38, F_C1D = 39, F_WRM1 = 40, F_WR = 41, F_WI2L = 42, F_WDI2L = 43
 };
 // Cell parameter slots: equilibrium of W^k at 0..11, of W^{k+1} at 12..23, each: r - 1, r, 1/(2 lam),
 // 1/(2 lam) - 1/(2 lam0), then the Shakhov factor s (c.q)(2 lam |c|^2 - 4) = L(u, v) Q(u, v) as
@@ -106,8 +115,9 @@ struct CaseDev {
     const double* wall;                // [4][nslot][3]  U_w, V_w, T_w per level (per step in time-domain mode)
     const double *xn, *yn, *xc, *yc, *hx, *hy, *rdx, *rdy;   // rdx[i] = 1/(xc[i+1]-xc[i])
     const double *vu, *vv, *vw;        // per padded velocity
-    const T *tu, *tv, *tw, *thref;     // per padded velocity
-    const T *twu, *twv;                // per padded velocity: the factors w_u, w_v of its weight (0 for padding)
+    const T *tu, *tv, *thref;          // per padded velocity
+    const T* twu;                      // per padded velocity: the factor w_u of its weight (0 for padding)
+    const T* wrow;                     // per velocity block: weights of the face sums (K1_WT)
     const double *u1, *wu1, *v1, *wv1; // 1-D grids
     const T *tu1, *tv1;                // 1-D nodes in the storage precision
     const double* refmom;              // [5][13]: full, u>0, u<0, v>0, v<0 moments of (H_ref, B_ref)
@@ -148,24 +158,49 @@ struct CaseDev {
                                        // first completed wait as expired (no copy in flight is abandoned)
 };
 
+// Which case a CTA works on, and its index among the case's CTAs.  Batch: the cases' descriptions lie in global memory,
+// found through a per-case block offset table.  One: a handle of a single case passes its description as a kernel
+// parameter, whose fields the kernels read from the constant bank as uniform values (registers and address arithmetic
+// off the vector pipes): micro update 1.02 -> 0.92 ms (64x64, 48x48, N_T 7).
 template <typename T>
 struct Batch {
+    using value_type = T;
     const CaseDev<T>* cases;
     int ncases;
     const int* off;   // block offsets per case for this kernel, ncases + 1 entries
+    __device__ __forceinline__ const CaseDev<T>& find(int blk, int& local) const
+    {
+        int lo = 0, hi = ncases - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (off[mid] <= blk) lo = mid; else hi = mid - 1;
+        }
+        local = blk - off[lo];
+        return cases[lo];
+    }
+};
+// the description copied to shared memory by the whole CTA: one round of loads instead of a chain of dependent ones
+template <typename T>
+__device__ __forceinline__ void copy_case(const CaseDev<T>& from, CaseDev<T>& to)
+{
+    static_assert(sizeof(CaseDev<T>) % 8 == 0, "copied in words of 8 bytes");
+    const unsigned long long* a = reinterpret_cast<const unsigned long long*>(&from);
+    unsigned long long* b = reinterpret_cast<unsigned long long*>(&to);
+    for (int k = threadIdx.x; k < (int)(sizeof(CaseDev<T>) / 8); k += blockDim.x) b[k] = a[k];
+    __syncthreads();
+}
+template <typename T>
+struct One {
+    using value_type = T;
+    CaseDev<T> c;
+    __device__ __forceinline__ const CaseDev<T>& find(int blk, int& local) const
+    {
+        local = blk;
+        return c;
+    }
 };
 
 // --------------------------------------------------------------------------------- small helpers
-
-__device__ __forceinline__ int find_case(const int* off, int ncases, int blk)
-{
-    int lo = 0, hi = ncases - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= blk) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
 
 // wall-state slot of level n in the current iteration: the level itself, or in time-domain mode the step
 // within the forcing period

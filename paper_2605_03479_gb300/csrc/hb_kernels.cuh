@@ -164,8 +164,9 @@ __device__ __forceinline__ void mom4(const P (&c)[10], P d0, P dn, P dt, const P
 template <typename T>
 __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B)
 {
-    const int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
+    __shared__ CaseDev<T> cd;
+    int lb;
+    copy_case(B.find(blockIdx.x, lb), cd);
     // uniform over the CTA: neither word changes while this kernel runs
     if (!cd.st->active || *(volatile int*)cd.err) return;
     __shared__ T pL[5][K2_ITEMS], pR[5][K2_ITEMS], pt[5][K2_ITEMS], pA[5][K2_ITEMS], shk_[13][K2_ITEMS], Cw[5][K2_ITEMS];
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
     __shared__ double dF1[4][K2_ITEMS], sdG[K2_ITEMS], st[10][K2_ITEMS];
     const int nt = cd.nt, nu = cd.nu, nv = cd.nv, nuv = nu + nv, nitems = cd.nf * nt;
     const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
-    const int base = (blockIdx.x - B.off[cs]) * K2_ITEMS;
+    const int base = lb * K2_ITEMS;
     const bool valid = base + lane < nitems;
     const int item = valid ? base + lane : nitems - 1;       // lanes past the end repeat the last item and store nothing
     const int f = item / nt, n = item - f * nt;
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
         pp[F_C1] = T((double)Cw[0][lane] * idG);
         pp[F_C4] = T((double)Cw[3][lane] * idG);
         pp[F_C5] = T((double)Cw[4][lane] * idG);
-        pp[F_NIN] = T(nin);
+        pp[F_C1D] = T((double)Cw[0][lane] * idG * (i2ld - 0.5 * il0));
     }
 }
 
@@ -510,9 +511,9 @@ __device__ __forceinline__ double local_step(const CaseDev<T>& cd, double numax)
 template <typename T>
 __global__ void k_steps(Batch<T> B)
 {
-    int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
-    int c = (blockIdx.x - B.off[cs]) * blockDim.x + threadIdx.x;
+    int lb;
+    const CaseDev<T>& cd = B.find(blockIdx.x, lb);
+    int c = lb * blockDim.x + threadIdx.x;
     if (c >= cd.nc) return;
     const double rdx = rcp64(2.0 * cd.hx[c % cd.nx]), rdy = rcp64(2.0 * cd.hy[c / cd.nx]);
     double numax = 0.0;
@@ -544,15 +545,15 @@ __host__ __device__ constexpr int k3_threads(int nt) { return 2 * k3_half(nt) < 
 template <typename T>
 __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
 {
-    const int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
+    __shared__ CaseDev<T> cd;
+    int lb;
+    copy_case(B.find(blockIdx.x, lb), cd);
     // uniform over the CTA: neither word changes while this kernel runs
     if (!cd.st->active || *(volatile int*)cd.err) return;
     __shared__ T coef[K3_CELLS * MAXNT * 2][5];            // exponent coefficients of the tables, row (cell, level, e)
     __shared__ double sq[MAXNT * K3_CELLS][2], stau[MAXNT * K3_CELLS], snu[MAXNT * K3_CELLS];
     __shared__ double srhs[MAXNT * K3_CELLS][4], sinv[MAXNT * K3_CELLS];
     __shared__ double sM[MAXNT][MAXNT][K3_CELLS];
-    const int lb = blockIdx.x - B.off[cs];
     const int nt = cd.nt, nc = cd.nc, half = k3_half(nt);
     const int role = (int)threadIdx.x / half;              // 0: W^k, 1: W^{k+1}, 2: helps with the tables only
     const int r = (int)threadIdx.x - role * half;
@@ -745,15 +746,12 @@ __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
 
 constexpr int K5_THREADS = 128;
 
+// residual, history and status of one case from nb partials; ends the iteration (swaps the state buffers)
 template <typename T>
-__global__ void __launch_bounds__(K5_THREADS) k5_finish(const CaseDev<T>* cases, int ncases, const int* k3off)
+__device__ __forceinline__ void finish_case(const CaseDev<T>& cd, int nb)
 {
-    int cs = blockIdx.x;
-    if (cs >= ncases) return;
-    const CaseDev<T>& cd = cases[cs];
     CaseStatus* st = cd.st;
     if (!st->active || *(volatile int*)cd.err) return;   // a failed wait leaves the iteration unfinished
-    const int nb = k3off[cs + 1] - k3off[cs];
     // thread t sums variable t & 3 of every 32nd partial; then a fixed tree over lanes and warps
     __shared__ double part[K5_THREADS / 32][4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -784,6 +782,35 @@ __global__ void __launch_bounds__(K5_THREADS) k5_finish(const CaseDev<T>* cases,
                 st->active = 0;
             }
         }
+    }
+}
+
+// LOOP: the last CTA also ends the pass of the device-side loop: one iteration fewer left; the loop goes on while
+// iterations are left, some case is still iterating (not converged, not diverged) and no device wait has failed.  Every
+// pass decrements the count, so the loop ends after at most the requested number of iterations.
+struct LoopTest {
+    cudaGraphConditionalHandle handle;
+    int* left;                          // [0] iterations left, [1] CTAs of this pass that are done
+    const CaseStatus* st;
+    const int* err;
+};
+
+template <typename T, bool LOOP>
+__global__ void __launch_bounds__(K5_THREADS) k5_finish(const CaseDev<T>* cases, int ncases, const int* k3off, LoopTest loop)
+{
+    finish_case(cases[blockIdx.x], k3off[blockIdx.x + 1] - k3off[blockIdx.x]);
+    if constexpr (LOOP) {
+        __syncthreads();
+        if (threadIdx.x != 0) return;
+        __threadfence();
+        if (atomicAdd(loop.left + 1, 1) != ncases - 1) return;
+        __threadfence();
+        loop.left[1] = 0;
+        const int r = loop.left[0] - 1;
+        loop.left[0] = r;
+        int any = 0;
+        for (int k = 0; k < ncases; ++k) any |= *(volatile const int*)&loop.st[k].active;
+        cudaGraphSetConditional(loop.handle, (r > 0 && any && *(volatile const int*)loop.err == 0) ? 1u : 0u);
     }
 }
 

@@ -1,8 +1,9 @@
 // Micro update of one HB-UGKS iteration (K4): interface micro fluxes (Eq. micro_flux), spectral source and the
 // semi-implicit collision update (Eq. fv_h) of every cell, level and velocity.
 //
-// A CTA takes a strip of TX columns, a segment of rows, VPL blocks of 32 velocities of one sign class, and all
-// levels, one warp per level.  Its warps march along the rows in the direction of v and, within a row, along the
+// A group of warps, one per level, takes a strip of TX columns, a segment of rows and VPL blocks of 32 velocities of
+// one sign class; a CTA holds one or several groups, which share nothing (registers are given to a CTA for four warps
+// at a time, so CTAs of three or five warps would waste a quarter or more of them).  A group's warps march along the rows in the direction of v and, within a row, along the
 // columns in the direction of u: a cell's upwind fluxes are then the ones the same lane has just computed (the
 // x-flux of the cell before, the y-flux of the row before), so no flux and no slope passes through shared memory and
 // no CTA barrier separates levels.  Columns and rows are counted from the upwind side ("mirrored": column p is
@@ -10,13 +11,16 @@
 // with it, and u s_x, u (F_downwind - F_upwind) keep theirs, so one code serves the four sign classes.  Only the
 // strip's upwind column and the segment's upwind row are computed twice (one flux each).
 //
-// Bound by instruction issue: 238 warp instructions per 32 updates in single precision (128x128, 64x64, N_T 11), 130 of
-// them floating point, where the previous kernel (a tile of cells per CTA, fluxes through shared memory, one barrier per
-// level) needed 422.  The shared-memory loads serve two velocities per lane, the expm1 factors are loaded one cell ahead
-// (their L2 latency was 46 % of the stalls), and the x direction is a template parameter so that all offsets within a
-// row are constants.  Measured, previous kernel -> this one: 16.25 -> 8.73 ms (128x128, 64x64, N_T 11), 1.50 -> 1.02 ms
-// (64x64, 48x48, N_T 7), 44.5 -> 29.2 ms (48 uneven cavities), 0.60 -> 0.42 ms (90x90, 28x28, N_T 3); FP64, bound by
-// its pipe, 58.1 -> 50.1 ms (twelve 64x64, 32x32, N_T 3), 25.8 -> 21.9 ms (64x64, 48x48, N_T 7).
+// Bound by instruction issue in single precision: about 235 warp instructions per 32 updates, 130 of them floating
+// point, where the previous kernel (a tile of cells per CTA, fluxes through shared memory, one barrier per level) needed
+// 422.  The shared-memory loads serve two velocities per lane, the expm1 factors are loaded ahead of their use (their L2
+// latency was 46 % of the stalls), and the x direction is a template parameter so that all offsets within a row are
+// constants.  Strips of two columns with 128 registers hold more warps per SM and win up to 7 levels (0.83 against
+// 1.02 ms, 64x64, 48x48, N_T 7), strips of four with 168 recompute less and win above (8.3 ms, 128x128, 64x64, N_T 11).
+// Bound by the FP64 pipe in FP64: everything relative to H_ref saves 9 of 178 instructions per update.  Previous kernel
+// -> this one: 16.25 -> 8.27 ms (128x128, 64x64, N_T 11), 1.50 -> 0.83 ms (64x64, 48x48, N_T 7), 44.5 -> 25.8 ms (48
+// uneven cavities), 0.60 -> 0.32 ms (90x90, 28x28, N_T 3); FP64 58.1 -> 46.4 ms (twelve 64x64, 32x32, N_T 3) and 25.8 ->
+// 20.8 ms (64x64, 48x48, N_T 7).
 #pragma once
 #include "hb_cells.cuh"
 
@@ -26,32 +30,6 @@ namespace hb {
 template <typename T, int VPL> struct LanesOf { using type = T; };
 template <> struct LanesOf<float, 2> { using type = float2; };
 
-__device__ __forceinline__ float pfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double pfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float pmul(float a, float b) { return a * b; }
-// (kept apart from a following addition, so that every instance of the kernel rounds alike)
-__device__ __forceinline__ double pmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float padd(float a, float b) { return a + b; }
-__device__ __forceinline__ double padd(double a, double b) { return __dadd_rn(a, b); }
-// N parameters (a multiple of 4) from shared memory by 16-byte loads
-template <int N>
-__device__ __forceinline__ void load_par(const float* p, float (&o)[N])
-{
-#pragma unroll
-    for (int k = 0; k < N; k += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(p + k);
-        o[k] = x.x; o[k + 1] = x.y; o[k + 2] = x.z; o[k + 3] = x.w;
-    }
-}
-template <int N>
-__device__ __forceinline__ void load_par(const double* p, double (&o)[N])
-{
-#pragma unroll
-    for (int k = 0; k < N; k += 2) {
-        const double2 x = *reinterpret_cast<const double2*>(p + k);
-        o[k] = x.x; o[k + 1] = x.y;
-    }
-}
 template <typename L> struct Lane1;
 template <> struct Lane1<float> {
     static __device__ __forceinline__ float all(float x) { return x; }
@@ -69,25 +47,21 @@ template <> struct Lane1<float2> {
     static __device__ __forceinline__ float2 of(const float* x) { return make_float2(x[0], x[1]); }
 };
 
-// Maxwellian part of the micro flux divided by dG_f and u_n (delta form), C1' dH + H Q for h and C1' dB + B (Q + lin)
-// for b, from the face's parameters fp (shared memory; cubic at qo, linear term at lo: the upwind side's) and the
-// expm1 factors (ex, ey) of the interface Maxwellian at the lane's velocities; c4, c5: C4', C5'
+// Maxwellian part of the micro flux divided by dG_f, u_n and H_ref (delta form).  With G = H/H_ref - 1 it is
+// C1' G + (1 + G) Q = Q + G (Q + C1') for h, and i2l [Qb + G (Qb + C1')] + C1' (i2l - i2l0) for b (Qb = Q + lin), from
+// the face's parameters fp (shared memory; cubic at qo, linear term at lo: the upwind side's) and the expm1 factors
+// (ex, ey) of the interface Maxwellian at the lane's velocities; c4, c5: C4', C5'
 template <typename T, typename L>
-__device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L ey, L href, L u, L v, L& mh, L& mb, T& c4,
-                                          T& c5)
+__device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L ey, L u, L v, L& mh, L& mb, T& c4, T& c5)
 {
     using A = Lane1<L>;
-    T sc[8], c[12], l[4];          // sc: r - 1, r, 1/(2 lam), 1/(2 lam) - 1/(2 lam0), C1', C4', C5', nin
+    T sc[8], c[12], l[4];          // sc: r - 1, r, 1/(2 lam), 1/(2 lam) - 1/(2 lam0), C1', C4', C5', C1' times slot 3
     load_par(fp + F_RM1, sc);
     load_par(fp + qo, c);
     load_par(fp + lo, l);
     c4 = sc[5];
     c5 = sc[6];
-    const L E = pfma(ex, ey, padd(ex, ey));
-    const L dH = pmul(href, pfma(A::all(sc[1]), E, A::all(sc[0])));
-    const L H = padd(href, dH);
-    const L i2l = A::all(sc[2]);
-    const L dB = pfma(dH, i2l, pmul(href, A::all(sc[3])));
+    const L G = pfma(A::all(sc[1]), pfma(ex, ey, padd(ex, ey)), A::all(sc[0]));
     // Horner form of the bivariate cubic with monomials 1, u, v, u^2, uv, v^2, u^3, u^2 v, u v^2, v^3
     const L y0 = pfma(v, pfma(v, pfma(v, A::all(c[9]), A::all(c[5])), A::all(c[2])), A::all(c[0]));
     const L y1 = pfma(v, pfma(v, A::all(c[8]), A::all(c[4])), A::all(c[1]));
@@ -95,38 +69,38 @@ __device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L e
     const L Q = pfma(u, pfma(u, y2, y1), y0);
     const L Qb = pfma(v, A::all(l[2]), pfma(u, A::all(l[1]), padd(Q, A::all(l[0]))));
     const L c1 = A::all(sc[4]);
-    mh = pfma(H, Q, pmul(c1, dH));
-    mb = pfma(pmul(H, i2l), Qb, pmul(c1, dB));
+    mh = pfma(G, padd(Q, c1), Q);
+    mb = pfma(A::all(sc[2]), pfma(G, padd(Qb, c1), Qb), A::all(sc[7]));
 }
 
-// Equilibrium (H+ - H_ref, B+ - B_ref) of one cell-parameter slot q at the lane's velocities: the Maxwellian from the
-// cell table factors (ex, ey), and with the Shakhov model the correction (L Q) H for h and (L Q + 2 L) B for b (L, Q
-// the linear and quadratic factors of s (c.q)(2 lam |c|^2 - 4); r2 = u^2 + v^2)
+// Equilibrium (H+ - H_ref, B+ - B_ref) divided by H_ref of one cell-parameter slot q at the lane's velocities: G and
+// i2l G + (i2l - i2l0) of the Maxwellian (cell table factors ex, ey), and with the Shakhov model
+// G + (1 + G) sk = sk + G (1 + sk), sk = L Q, for h and the same with sk + 2 L for b (L, Q the linear and quadratic
+// factors of s (c.q)(2 lam |c|^2 - 4); r2 = u^2 + v^2)
 template <bool SHAKHOV, typename T, typename L>
-__device__ __forceinline__ void eq_core(const T* qp, L ex, L ey, L href, L u, L v, L r2, L& mh, L& mb)
+__device__ __forceinline__ void eq_core(const T* qp, L ex, L ey, L u, L v, L r2, L& mh, L& mb)
 {
     using A = Lane1<L>;
     T q[12];
     load_par(qp, q);
-    const L E = pfma(ex, ey, padd(ex, ey));
-    const L dH = pmul(href, pfma(A::all(q[E_R]), E, A::all(q[E_RM1])));
-    const L i2l = A::all(q[E_I2L]);
-    const L dB = pfma(dH, i2l, pmul(href, A::all(q[E_DI2L])));
+    const L G = pfma(A::all(q[E_R]), pfma(ex, ey, padd(ex, ey)), A::all(q[E_RM1]));
+    const L i2l = A::all(q[E_I2L]), di2l = A::all(q[E_DI2L]);
     if constexpr (!SHAKHOV) {
-        mh = dH;
-        mb = dB;
+        mh = G;
+        mb = pfma(i2l, G, di2l);
         return;
     }
-    const L H = padd(href, dH);
     const L Lf = pfma(A::all(q[E_L + 2]), v, pfma(A::all(q[E_L + 1]), u, A::all(q[E_L])));
     const L Qs = pfma(A::all(q[E_Q + 3]), r2,
                       pfma(A::all(q[E_Q + 2]), v, pfma(A::all(q[E_Q + 1]), u, A::all(q[E_Q]))));
-    const L sk = pmul(Lf, Qs);
-    mh = pfma(H, sk, dH);
-    mb = pfma(pmul(H, i2l), pfma(A::all(T(2)), Lf, sk), dB);
+    const L sk = pmul(Lf, Qs), sb = pfma(A::all(T(2)), Lf, sk), one = A::all(T(1));
+    mh = pfma(G, padd(one, sk), sk);
+    mb = pfma(i2l, pfma(G, padd(one, sb), sb), di2l);
 }
 
-// Shared memory of one CTA of k4_march for nt levels (bytes): three rows of the strip with its halo on every level
+constexpr int K4_MAXROWS = 32;   // rows per segment
+
+// Shared memory of one group of k4_march for nt levels (bytes): three rows of the strip with its halo on every level
 // (two columns upwind, one downwind), two rows of parameters (x-faces, y-faces downwind, cells) on every level, and
 // with the spectral source at the new iterate one row of right-hand sides.
 template <typename T, int TX, int VPL>
@@ -136,16 +110,18 @@ struct K4Layout {
     static constexpr uint32_t COL = VB * sizeof(V), BLK = NCOL * COL, ROW = VPL * BLK;
     static constexpr uint32_t PX = (TX + 1) * NP * sizeof(T), PY = TX * NP * sizeof(T), PC = TX * NCP * sizeof(T);
     static constexpr uint32_t PAR = PX + PY + PC;
+    // spacings: widths and inverse distances of the strip's columns, then of the segment's rows
+    static constexpr int GX = TX + 2, GH = TX + 1, GY = K4_MAXROWS + 3;
+    static constexpr size_t GEO = ((GX + GH + 2 * GY) * sizeof(T) + 15) / 16 * 16;
     static constexpr size_t bytes(int nt, bool imp)
     {
-        return (size_t)nt * (3 * ROW + 2 * PAR + (imp ? (uint32_t)(VPL * TX) * COL : 0u));
+        return (size_t)nt * (3 * ROW + 2 * PAR + (imp ? (uint32_t)(VPL * TX) * COL : 0u)) + GEO;
     }
 };
 
-constexpr int K4_MAXROWS = 32;   // rows per segment
-// threads the instances are compiled for, and so their registers: strips of two columns for every level count, strips
-// of four for up to 7 levels (144 registers: two CTAs of 7 warps per SM) and up to 11 (184)
-constexpr int K4_T2 = MAXNT * 32, K4_T4 = 14 * 32, K4_T4L = 11 * 32;
+// Threads the instances are compiled for, and so their registers: 128 for up to 15 warps (every level count with strips
+// of two columns, up to 7 levels with strips of four), 168 for strips of four columns on up to 11 levels, one CTA per SM.
+constexpr int K4_T2 = MAXNT * 32, K4_T4L = 11 * 32;
 constexpr int K4_NT4 = 7, K4_NT4L = 11;
 
 // spectral source of NC consecutive cells of a row on level n: sum_d e_d (f_{n-d} - f_{n+d}) for (h, b) (Eq. D_explicit in paired
@@ -173,6 +149,12 @@ __device__ __forceinline__ void spectral_cells(const char* row, uint32_t ls, int
     }
 }
 
+// barrier of one group's warps (named barrier 1 + group; at most 15 groups)
+__device__ __forceinline__ void group_sync(int group, int threads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(threads) : "memory");
+}
+
 // One bulk copy of the per-row batches, formed once per warp: in batch b (lo <= b <= hi) it reads src + (b - 1) stride
 // and lands at dst, plus the slot of the row it belongs to.
 struct alignas(16) K4Copy {
@@ -182,9 +164,10 @@ struct alignas(16) K4Copy {
     int lo, hi, pad;
 };
 
-template <typename T, int TX, int VPL, bool IMP, int MAXT>
-__global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
+template <class P, int TX, int VPL, bool IMP, int MAXT>
+__global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, int rows, int groups)
 {
+    using T = typename P::value_type;
     using Y = K4Layout<T, TX, VPL>;
     using V = P2<T>;
     using L = typename LanesOf<T, VPL>::type;
@@ -194,25 +177,29 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
     constexpr bool FULL = TX == 4;
     constexpr int NCOPY = VPL + 3;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t full[2], done;
+    __shared__ uint64_t full_[MAXNT][2], done_[MAXNT];       // per group
     __shared__ int abort_flag;                               // set by the first warp whose wait runs out
-    __shared__ T gxw[TX + 2], gxh[TX + 1], gyw[K4_MAXROWS + 3], gyh[K4_MAXROWS + 3];
-    __shared__ K4Copy copies[MAXNT][NCOPY];
-    const int cs = find_case(B.off, B.ncases, blockIdx.x);
-    const CaseDev<T>& cd = B.cases[cs];
+    __shared__ K4Copy copies[MAXNT][NCOPY];                  // per warp
+    int lb;
+    const CaseDev<T>& cd = B.find(blockIdx.x, lb);
     if (!cd.st->active) return;
     // another CTA may set the error word while this one starts: decide for the whole CTA at once
     if (__syncthreads_or(*(volatile int*)cd.err != 0)) return;
     const bool expire = *(volatile const int*)cd.expire != 0;
     const int nx = cd.nx, ny = cd.ny, nt = cd.nt, nc = cd.nc, nfx = cd.nfx, nuv = cd.nu + cd.nv;
     const int lane = threadIdx.x & 31;
-    const int n = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // the warp's level
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+    constexpr bool ALONE = MAXT == K4_T4L;                   // one group per CTA
+    const int gi = ALONE ? 0 : warp / nt, n = ALONE ? warp : warp - gi * nt;   // the warp's group and level
+    const int tid = (int)threadIdx.x - gi * nt * 32, nthreads = nt * 32;   // in the group
+    uint64_t* const full = full_[gi];
+    uint64_t* const done = &done_[gi];
     // CTA order: velocity group fastest (the CTAs of one strip share its parameters in L2), then strips, segments
     int ng = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) ng += (cd.cls_end[c] - (c ? cd.cls_end[c - 1] : 0) + VPL - 1) / VPL;
-    const int lb = blockIdx.x - B.off[cs], tile = lb / ng;
-    int g = lb - tile * ng, cls = 0, vb = 0, vend = 0;
+    const int work = ALONE ? lb : lb * groups + gi, tile = work / ng;
+    int g = work - tile * ng, cls = 0, vb = 0, vend = 0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const int first = c ? cd.cls_end[c - 1] : 0, cnt = (cd.cls_end[c] - first + VPL - 1) / VPL;
@@ -223,26 +210,30 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
     const int nstrip = (nx + TX - 1) / TX;
     const int p0 = FULL ? min((tile % nstrip) * TX, nx - TX) : (tile % nstrip) * TX;
     const int q0 = (tile / nstrip) * rows, nr = min(rows, ny - q0);
-    char* const srow = reinterpret_cast<char*>(smem_raw);
+    const bool idle = !ALONE && q0 >= ny;                    // past the case's last group
+    char* const srow = reinterpret_cast<char*>(smem_raw) + (ALONE ? 0 : (size_t)gi * Y::bytes(nt, IMP));
     char* const spar = srow + (size_t)3 * nt * Y::ROW;
     V* const srhs = reinterpret_cast<V*>(spar + (size_t)2 * nt * Y::PAR);   // right-hand sides (implicit source)
+    __shared__ T geo[ALONE ? Y::GEO / sizeof(T) : 1];        // (a fixed address saves the lone group's registers)
+    T* const gxw = ALONE ? geo : reinterpret_cast<T*>(srow + Y::bytes(nt, IMP) - Y::GEO);
+    T *const gxh = gxw + Y::GX, *const gyw = gxh + Y::GH, *const gyh = gyw + Y::GY;
     const uint32_t slot_b = (uint32_t)nt * Y::ROW, pslot_b = (uint32_t)nt * Y::PAR;
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
+    if (threadIdx.x == 0) abort_flag = 0;
+    if (tid == 0) {
         mbar_init(&full[0], nt);
         mbar_init(&full[1], nt);
-        mbar_init(&done, nt);
+        mbar_init(done, nt);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // spacings in mirrored order: gxw[k] twice the inverse distance of columns p0 - 2 + k and p0 - 1 + k, gxh[k] half
     // the width of column p0 - 1 + k; gyw[r], gyh[r] of stream rows r (row q = q0 - 2 + r) and r, r + 1
-    for (int k = threadIdx.x; k < TX + 2; k += blockDim.x) {
+    for (int k = tid; k < TX + 2; k += nthreads) {
         const int p = p0 - 2 + k, i = xneg ? nx - 2 - p : p;
         gxw[k] = (i >= 0 && i < nx - 1) ? T(2) * T(cd.rdx[i]) : T(0);
         const int ph = p + 1, ih = xneg ? nx - 1 - ph : ph;
         if (k < TX + 1) gxh[k] = (ih >= 0 && ih < nx) ? T(cd.hx[ih]) : T(0);
     }
-    for (int r = threadIdx.x; r < nr + 3; r += blockDim.x) {
+    for (int r = tid; r < nr + 3; r += nthreads) {
         const int q = q0 - 2 + r, j = yneg ? ny - 2 - q : q, jh = yneg ? ny - 1 - q : q;
         gyw[r] = (j >= 0 && j < ny - 1) ? T(2) * T(cd.rdy[j]) : T(0);
         gyh[r] = (jh >= 0 && jh < ny) ? T(cd.hy[jh]) : T(0);
@@ -294,9 +285,10 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
             c.lo = lane == VPL + 1 ? 1 : 2;
             c.hi = nr + 1;
         }
-        copies[n][lane] = c;
+        copies[warp][lane] = c;
     }
     __syncthreads();
+    if (idle) return;
 
     // this warp's part of batch b >= 1, its row into row slot `slot`
     auto issue = [&](int b, uint32_t slot) {
@@ -304,7 +296,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
         if (lane == 0) mbar_arrive_expect(bar, (b <= ny - q0 ? VPL * rb : 0u) + yb + (b >= 2 ? xb + cb : 0u));
         __syncwarp();
         if (lane < NCOPY) {
-            const K4Copy c = copies[n][lane];
+            const K4Copy c = copies[warp][lane];
             if (b >= c.lo && b <= c.hi)
                 bulk_g2s_at(c.dst + (lane < VPL ? slot * slot_b : (uint32_t)(b & 1) * pslot_b),
                             c.src + (long long)(b - 1) * c.stride, c.bytes, bar);
@@ -319,7 +311,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
     __syncwarp();
     if (lane < 2 * VPL) {
         const int row = lane / VPL;
-        const K4Copy c = copies[n][lane % VPL];
+        const K4Copy c = copies[warp][lane % VPL];
         if (q0 + row >= 2)
             bulk_g2s_at(c.dst + (uint32_t)row * slot_b, c.src + (long long)(row - 2) * c.stride, c.bytes, &full[0]);
     }
@@ -328,7 +320,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
 
     // the lane's velocities
     T u[VPL], v[VPL];
-    V um[VPL], vm[VPL];                                      // |u|, |v| as pairs
+    T um[VPL], vm[VPL];                                      // |u|, |v|
     T hr[VPL], rr2[VPL];
     uint32_t iu[VPL], iv[VPL];                               // byte offsets of the lane's entries in a table row
 #pragma unroll
@@ -336,14 +328,14 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
         const int av = (vb + (two ? h : 0)) * VB + lane;
         u[h] = __ldg(cd.tu + av);
         v[h] = __ldg(cd.tv + av);
-        um[h] = bc(xneg ? -u[h] : u[h]);
-        vm[h] = bc(yneg ? -v[h] : v[h]);
+        um[h] = xneg ? -u[h] : u[h];
+        vm[h] = yneg ? -v[h] : v[h];
         hr[h] = __ldg(cd.thref + av);
         rr2[h] = pfma(u[h], u[h], pmul(v[h], v[h]));
         iu[h] = (uint32_t)__ldg(cd.viu + av) * (uint32_t)sizeof(T);
         iv[h] = (uint32_t)(cd.nu + __ldg(cd.viv + av)) * (uint32_t)sizeof(T);
     }
-    const L uL = A::of(u), vL = A::of(v), hrefL = A::of(hr), r2L = A::of(rr2);
+    const L uL = A::of(u), vL = A::of(v), r2L = A::of(rr2);
     const bool shakhov = cd.shakhov != 0;
     const bool implicit = IMP && cd.spectral_implicit != 0;
     const int nh = implicit ? 0 : cd.nh;
@@ -383,9 +375,10 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
     auto face_flux = [&](const char* fp, int qo, int lo, L ex, L ey, const V (&d0)[VPL], const V (&gr)[VPL], V (&F)[VPL]) {
         L mh, mb;
         T c4, c5;
-        flux_core<T, L>(reinterpret_cast<const T*>(fp), qo, lo, ex, ey, hrefL, uL, vL, mh, mb, c4, c5);
+        flux_core<T, L>(reinterpret_cast<const T*>(fp), qo, lo, ex, ey, uL, vL, mh, mb, c4, c5);
 #pragma unroll
-        for (int h = 0; h < VPL; ++h) F[h] = pfma(bc(c5), gr[h], pfma(bc(c4), d0[h], pk(A::at(mh, h), A::at(mb, h))));
+        for (int h = 0; h < VPL; ++h)
+            F[h] = pfma(bc(hr[h]), pk(A::at(mh, h), A::at(mb, h)), pfma(bc(c4), d0[h], pmul(bc(c5), gr[h])));
     };
     // a wait ran out: this warp waits (bounded) for the batches from b on that it has issued and not seen complete, so
     // that none still lands in shared memory after the CTA exits
@@ -409,7 +402,11 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
         constexpr int FY0 = (int)Y::PX + (XN ? (TX - 1) * (int)(NP * sizeof(T)) : 0);
         constexpr int CE0 = (int)(Y::PX + Y::PY) + (XN ? (TX - 1) * (int)(NCP * sizeof(T)) : 0);
         const int i0 = XN ? nx - 1 - p0 : p0, fi0 = XN ? nx - p0 : p0;
-        const long long tstep = (long long)(SG * nt * nuv) * (int)sizeof(T); // table bytes between consecutive faces
+        // Bytes between the table rows of consecutive faces.  The lone-group instance, short of registers, keeps them in 32
+        // bits (its launch rule sees to it that eight of them fit).
+        using Off = std::conditional_t<ALONE, int, long long>;
+        const Off tstep = (Off)SG * nt * nuv * (int)sizeof(T);
+        auto ahead = [tstep](const char* tb, int k) { return tb + k * tstep; };
         char* const rown = srow + n * Y::ROW + lane * sizeof(V) + COL0;      // row slot 0, this level and lane
         auto at = [](const char* row, int c, int h) -> V {                   // mirrored column c (2 is p0) of block h
             return *reinterpret_cast<const V*>(row + c * CS + h * (int)Y::BLK);
@@ -428,7 +425,9 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
                 for (int h = 0; h < VPL; ++h) dyp[k][h] = pmul(psub(at(rb2, k + 1, h), at(ra, k + 1, h)), bc(gyw[r]));
         };
         // The table entries of a face or cell come from L2 and are loaded one cell ahead: xe, xv of the next x-face, ye,
-        // yv of the next y-face, ce, cv (and those of W^{k+1}) of the next cell, in the order they are used.
+        // yv of the next y-face, and with registers to spare (one CTA per SM) ce, cv (and those of W^{k+1}) of the next
+        // cell, in the order they are used.
+        constexpr bool EARLY = ALONE;
         L xe, xv, ye, yv, ce0, cv0, ce1, cv1;
         auto load_x = [&](const char* tb) { xe = pair_at(tb, iu); xv = pair_at(tb, iv); };
         auto load_y = [&](const char* tb) { ye = pair_at(tb, iu); yv = pair_at(tb, iv); };
@@ -442,12 +441,12 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
         };
         const char *tx0, *ty0, *tc0;
         row_tables(q0, tx0, ty0, tc0);
-        load_x(p0 > 0 ? tx0 : tx0 + tstep);
+        load_x(p0 > 0 ? tx0 : ahead(tx0, 1));
         load_y(ty0);
-        load_c(tc0);
+        if (EARLY) load_c(tc0);
         row_diff(rown, rown + slot_b, 0);                    // (unused where the segment starts at a wall)
         __syncwarp();
-        if (lane == 0) mbar_arrive(&done);
+        if (lane == 0) mbar_arrive(done);
 
         uint32_t slot = 0;
         for (int r = 1; r <= nr + 1; ++r) {
@@ -461,7 +460,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
             // the next batch: once every warp has left row r - 1, whose slots it refills
             auto refill = [&]() -> bool {
                 if (r > nr) return true;
-                if (!mbar_wait(&done, (uint32_t)((r - 1) & 1), err, &abort_flag)) return false;
+                if (!mbar_wait(done, (uint32_t)((r - 1) & 1), err, &abort_flag)) return false;
                 issue(r + 1, nslot == 2 ? 0 : nslot + 1);
                 issued = r + 1;
                 return true;
@@ -524,11 +523,11 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
                             if ((!FULL || t == TX - 1) && p0 + t == nx - 1) dxn = dxp[h];
                             const V sx = vleer2(dxp[h], dxn), sy = yslope(t + 2, h, fc[h], dyp[t + 1][h]);
                             d0[h] = pfma(sy, bc(gyh[r]), fc[h]);
-                            gr[h] = pfma(um[h], sx, pmul(vm[h], sy));
+                            gr[h] = pfma(bc(um[h]), sx, pmul(bc(vm[h]), sy));
                             dxp[h] = dxn;
                             fc[h] = fe;
                         }
-                        face_flux(pr + FY0 + t * FS, qy_, ly_, pair_at(th + t * tstep, iu), pair_at(th + t * tstep, iv), d0,
+                        face_flux(pr + FY0 + t * FS, qy_, ly_, pair_at(ahead(th, t), iu), pair_at(ahead(th, t), iv), d0,
                                   gr, Fy[t]);
                     }
                 }
@@ -547,10 +546,10 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
                         if (p0 == 1) dxm = dxp[h];           // (an overlapping strip next to the wall)
                         const V sx = vleer2(dxm, dxp[h]), sy = yslope(1, h, fw, dyp[0][h]);
                         d0[h] = pfma(sx, bc(gxh[0]), fw);
-                        gr[h] = pfma(um[h], sx, pmul(vm[h], sy));
+                        gr[h] = pfma(bc(um[h]), sx, pmul(bc(vm[h]), sy));
                     }
                     face_flux(pr + FX0, qx_, lx_, xe, xv, d0, gr, Fx);
-                    load_x(tx0 + tstep);
+                    load_x(ahead(tx0, 1));
                 } else {
                     wall_flux(pr + FX0, XN ? 1 : 3, Fx);
 #pragma unroll
@@ -587,51 +586,53 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
                         const V sx = vleer2(dxp[h], dxn), sy = yslope(t + 2, h, f0[h], dyp[t + 1][h]);
                         dx0[h] = pfma(sx, bc(gxh[t + 1]), f0[h]);
                         dy0[h] = pfma(sy, bc(gyh[r]), f0[h]);
-                        gr[h] = pfma(um[h], sx, pmul(vm[h], sy));
+                        gr[h] = pfma(bc(um[h]), sx, pmul(bc(vm[h]), sy));
                         dxp[h] = dxn;
                     }
                     const bool more = t + 1 < TX && (FULL || p0 + t + 1 < nx);   // another cell in this row
+                    const char* tcell = ahead(tc0, 2 * t);
                     if (!more) {
                         // the tables of the next row from here on (after the segment's last row: its own, unused)
                         row_tables(min(q + 1, q0 + nr - 1), tx0, ty0, tc0);
                     }
                     face_flux(pr + FX0 + (t + 1) * FS, qx_, lx_, xe, xv, dx0, gr, Fn);
-                    load_x(more ? tx0 + (t + 2) * tstep : p0 > 0 ? tx0 : tx0 + tstep);
+                    load_x(more ? ahead(tx0, t + 2) : p0 > 0 ? tx0 : ahead(tx0, 1));
 #pragma unroll
                     for (int h = 0; h < VPL; ++h) { dX[h] = psub(Fn[h], Fx[h]); Fx[h] = Fn[h]; }
                     face_flux(pr + FY0 + t * FS, qy_, ly_, ye, yv, dy0, gr, Fn);
-                    load_y(more ? ty0 + (t + 1) * tstep : ty0);
+                    load_y(more ? ahead(ty0, t + 1) : ty0);
 #pragma unroll
                     for (int h = 0; h < VPL; ++h) { dY[h] = psub(Fn[h], Fy[t][h]); Fy[t][h] = Fn[h]; }
                     // ---- Eq. fv_h (delta form) with the equilibria of W^{k+1} (slot 1) and W^k (slot 0)
                     const T* cp = reinterpret_cast<const T*>(pr + CE0 + t * ES);
+                    if (!EARLY) load_c(tcell);
                     const L ex0 = ce0, ey0 = cv0, ex1 = ce1, ey1 = cv1;
-                    load_c(more ? tc0 + 2 * (t + 1) * tstep : tc0);
+                    if (EARLY) load_c(more ? ahead(tc0, 2 * (t + 1)) : tc0);
                     L h1, b1, h0, b0;
                     if (shakhov) {
-                        eq_core<true, T, L>(cp + C_EQ1, ex1, ey1, hrefL, uL, vL, r2L, h1, b1);
-                        eq_core<true, T, L>(cp + C_EQ0, ex0, ey0, hrefL, uL, vL, r2L, h0, b0);
+                        eq_core<true, T, L>(cp + C_EQ1, ex1, ey1, uL, vL, r2L, h1, b1);
+                        eq_core<true, T, L>(cp + C_EQ0, ex0, ey0, uL, vL, r2L, h0, b0);
                     } else {
-                        eq_core<false, T, L>(cp + C_EQ1, ex1, ey1, hrefL, uL, vL, r2L, h1, b1);
-                        eq_core<false, T, L>(cp + C_EQ0, ex0, ey0, hrefL, uL, vL, r2L, h0, b0);
+                        eq_core<false, T, L>(cp + C_EQ1, ex1, ey1, uL, vL, r2L, h1, b1);
+                        eq_core<false, T, L>(cp + C_EQ0, ex0, ey0, uL, vL, r2L, h0, b0);
                     }
                     T kp[12];                                // kself, -kE, kp1, kp0, -kdx, -kdy, each twice
                     load_par(cp + C_K, kp);
 #pragma unroll
                     for (int h = 0; h < VPL; ++h) {
                         V x = pmul(pk(kp[0], kp[1]), f0[h]);
-                        x = pfma(pmul(pk(kp[8], kp[9]), um[h]), dX[h], x);
-                        x = pfma(pmul(pk(kp[10], kp[11]), vm[h]), dY[h], x);
+                        x = pfma(bc(kp[8] * um[h]), dX[h], x);
+                        x = pfma(bc(kp[10] * vm[h]), dY[h], x);
                         x = pfma(pk(kp[2], kp[3]), e[t & 1][h], x);
-                        x = pfma(pk(kp[4], kp[5]), pk(A::at(h1, h), A::at(b1, h)), x);
-                        x = pfma(pk(kp[6], kp[7]), pk(A::at(h0, h), A::at(b0, h)), x);
+                        x = pfma(bc(kp[4] * hr[h]), pk(A::at(h1, h), A::at(b1, h)), x);
+                        x = pfma(bc(kp[6] * hr[h]), pk(A::at(h0, h), A::at(b0, h)), x);
                         if (implicit) srhs[(size_t)((n * TX + t) * VPL + h) * VB + lane] = x;
                         else if (h == 0 || two) on[h * bstride + t * SG * VB] = x;
                     }
                 }
                 if (implicit) {
                     // spectral source at the new iterate: f^{k+1} = minv (right-hand sides over the levels), per cell
-                    __syncthreads();
+                    group_sync(gi, nthreads);
 #pragma unroll
                     for (int t = 0; t < TX; ++t) {
                         if (!FULL && p0 + t >= nx) break;
@@ -649,11 +650,11 @@ __global__ void __launch_bounds__(MAXT) k4_march(Batch<T> B, int rows)
                         for (int h = 0; h < VPL; ++h)
                             if (h == 0 || two) on[h * bstride + t * SG * VB] = acc[h];
                     }
-                    __syncthreads();
+                    group_sync(gi, nthreads);
                 }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&done);
+            if (lane == 0) mbar_arrive(done);
         }
     };
     if (xneg) march(std::true_type{});
