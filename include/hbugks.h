@@ -120,7 +120,9 @@ typedef struct {
  * All cases of one handle must have the same precision.  Invalid: a non-finite or non-positive size, weight,
  * Kn, CFL, gamma, Pr, VSS alpha or speed bound; non-finite nodes or wall parameters; nodes not increasing; a
  * wall temperature <= 0 on some level; N_T > 15; or a case so large that its per-face or per-cell expm1
- * tables ((nf or 2 nc) x N_T x (nu + nv) elements) exceed 2^31 - 1 elements, the kernels' 32-bit offsets. */
+ * tables ((nf or 2 nc) x N_T x (nu + nv) elements) exceed 2^31 - 1 elements, the kernels' 32-bit offsets.
+ * An FP64 handle whose updates (cells x velocities, in blocks of 32 per sign class, x N_T) take no more than 8 GiB at 32
+ * bytes each includes that much to keep the limited slopes between two kernels of an iteration. */
 HBUGKS_API size_t hbugks_workspace_bytes(int ncases, const hbugks_case* cases);
 
 /* Create a handle for `ncases` cases (a batch of one or more uneven cases iterated together).

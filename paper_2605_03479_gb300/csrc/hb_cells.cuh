@@ -346,6 +346,9 @@ __global__ void __launch_bounds__(TX * TY * 32, CTAS) k1_cells(const __grid_cons
     // Ring of S slots: chunk k lands in slot k % S (mbarrier bars); each warp arrives on empty once it has
     // read the slot, and warp 0 refills a slot only after every warp has released it, so warps run up to
     // S - 1 chunks apart instead of meeting at a CTA barrier per chunk.
+    [[maybe_unused]] V* const slo =
+        cd.sl ? cd.sl + ((size_t)n * nc + (valid ? j * nx + i : 0)) * 2 * VB + lane : nullptr;
+    [[maybe_unused]] const size_t slstride = (size_t)nt * nc * 2 * VB;
     int k = 0, slot = 0, vb = 0;                             // chunk, its slot, its first block
     uint32_t ph = 0;                                         // phase of the slot's barrier
     for (cur = 0; cur < 4; ++cur) {
@@ -372,7 +375,7 @@ __global__ void __launch_bounds__(TX * TY * 32, CTAS) k1_cells(const __grid_cons
             const unsigned char* cb = smem_raw + (size_t)slot * SLOT;
             const int gk = min(G, vend - vb);
             // one block of the chunk; INNER: every neighbour of the warp's cell exists (no wall branches)
-            auto block = [&](auto inner_tag, const V* pc, const T* wp) {
+            auto block = [&](auto inner_tag, int g, const V* pc, const T* wp) {
                 constexpr bool INNER = decltype(inner_tag)::value;
                 const V f0 = pc[0];
                 V sxv, syv;
@@ -382,6 +385,14 @@ __global__ void __launch_bounds__(TX * TY * 32, CTAS) k1_cells(const __grid_cons
                 } else {
                     sxv = slope2(pc[-VB], f0, pc[VB], wxm, wxp, hm, hp, sx);
                     syv = slope2(pc[-PX * VB], f0, pc[PX * VB], wym, wyp, vm, vp, sy);
+                }
+                if constexpr (sizeof(T) == 8) {
+                    // kept for the micro update, which would spend a quarter of its FP64 instructions on them again
+                    if (slo) {
+                        V* o = slo + (size_t)(vb + g) * slstride;
+                        o[0] = sxv;
+                        o[VB] = syv;
+                    }
                 }
                 T a[4];
                 load_par(wp + lane * 4, a);
@@ -432,9 +443,9 @@ __global__ void __launch_bounds__(TX * TY * 32, CTAS) k1_cells(const __grid_cons
                 const T* wp = reinterpret_cast<const T*>(cb + G * blk * sizeof(V));
                 if (gk == G) {
 #pragma unroll
-                    for (int g = 0; g < G; ++g) block(inner_tag, pc + g * blk, wp + g * WT);
+                    for (int g = 0; g < G; ++g) block(inner_tag, g, pc + g * blk, wp + g * WT);
                 } else {
-                    for (int g = 0; g < gk; ++g) block(inner_tag, pc + g * blk, wp + g * WT);
+                    for (int g = 0; g < gk; ++g) block(inner_tag, g, pc + g * blk, wp + g * WT);
                 }
             };
             if (valid) {

@@ -130,6 +130,7 @@ struct CaseDev {
     const double* wconst;              // [4][nslot][WCN] reflected-half constants of each wall Maxwellian
     const double* oconst;              // [4][8]: incident and reflected flux moments of (H_ref, B_ref) per wall
     P2<T>* f[2];                       // the two state buffers (current: st->parity)
+    P2<T>* sl;                         // FP64, where it is kept: limited slopes [vb][level][cell][x, y][32] of h^k
     double* W[2];
     double* dG;
     double* hmom;                      // [nc][nt][4][NM] half-face sums of the reconstruction per sign class

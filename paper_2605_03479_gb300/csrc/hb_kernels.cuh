@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
     __syncthreads();
 
     // ---- C: velocity moments of the Maxwellian's polynomials
-    const T pref = T(rho0 * lamf / M_PI), i2l = T(i2ld);
+    const T pref = T(rho0 * lamf * M_1_PI), i2l = T(i2ld);
     // full 1-D sums of the interface Maxwellian over node subset r (0 all, 1 positive, 2 negative, 3 zero); dif: the
     // table part alone
     auto row = [&](int axis, int r, T (&o)[9]) {
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
         put(role == 2 ? F2L : F2R, o);
         if (role == 3) {
             // C1 term, Maxwellian part: moments of u_n psi (H0 - H_ref, B0 - B_ref), in FP64 from the reference sums
-            const double rr = rho0 * lamf * il0, di2l = i2ld - 0.5 * il0, fac = cd.lam0 / M_PI;
+            const double rr = rho0 * lamf * il0, di2l = i2ld - 0.5 * il0, fac = cd.lam0 * M_1_PI;
             const int rx = ax == 0 ? half : 0, ry = ax == 0 ? 0 : half;
             const double* X0 = cd.xr0 + rx * 9;
             const double* Y0 = cd.yr0 + ry * 9;

@@ -417,6 +417,14 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
         for (int k = 0; k < TX; ++k)
 #pragma unroll
             for (int h = 0; h < VPL; ++h) Fy[k][h] = bc(T(0));
+        // FP64: the slopes the face sums have kept, in mirrored direction (elsewhere they are formed here again)
+        const bool kept = sizeof(T) == 8 && cd.sl != nullptr;
+        auto kept_slopes = [&](int jr, int t, V& sx, V& sy) {                // of column p0 + t of row jr
+            const V* o = cd.sl + (((size_t)vb * nt + n) * nc + (size_t)(jr * nx + i0 + t * SG)) * 2 * VB + lane;
+            const V a = __ldg(o), b = __ldg(o + VB);
+            sx = XN ? pk(-a.x, -a.y) : a;
+            sy = yneg ? pk(-b.x, -b.y) : b;
+        };
         // differences between the rows in slots a and b (row r and r + 1) along y, of every column
         auto row_diff = [&](const char* ra, const char* rb2, int r) {
 #pragma unroll
@@ -519,12 +527,18 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
 #pragma unroll
                         for (int h = 0; h < VPL; ++h) {
                             const V fe = at(rc, t + 3, h);
-                            V dxn = pmul(psub(fe, fc[h]), bc(gxw[t + 2]));
-                            if ((!FULL || t == TX - 1) && p0 + t == nx - 1) dxn = dxp[h];
-                            const V sx = vleer2(dxp[h], dxn), sy = yslope(t + 2, h, fc[h], dyp[t + 1][h]);
+                            V sx, sy;
+                            if (kept) {
+                                kept_slopes(j, t, sx, sy);
+                            } else {
+                                V dxn = pmul(psub(fe, fc[h]), bc(gxw[t + 2]));
+                                if ((!FULL || t == TX - 1) && p0 + t == nx - 1) dxn = dxp[h];
+                                sx = vleer2(dxp[h], dxn);
+                                sy = yslope(t + 2, h, fc[h], dyp[t + 1][h]);
+                                dxp[h] = dxn;
+                            }
                             d0[h] = pfma(sy, bc(gyh[r]), fc[h]);
                             gr[h] = pfma(bc(um[h]), sx, pmul(bc(vm[h]), sy));
-                            dxp[h] = dxn;
                             fc[h] = fe;
                         }
                         face_flux(pr + FY0 + t * FS, qy_, ly_, pair_at(ahead(th, t), iu), pair_at(ahead(th, t), iv), d0,
@@ -541,10 +555,16 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
 #pragma unroll
                     for (int h = 0; h < VPL; ++h) {
                         const V fw = at(rc, 1, h);
-                        dxp[h] = pmul(psub(fc[h], fw), bc(gxw[1]));
-                        V dxm = pmul(psub(fw, at(rc, 0, h)), bc(gxw[0]));
-                        if (p0 == 1) dxm = dxp[h];           // (an overlapping strip next to the wall)
-                        const V sx = vleer2(dxm, dxp[h]), sy = yslope(1, h, fw, dyp[0][h]);
+                        V sx, sy;
+                        if (kept) {
+                            kept_slopes(j, -1, sx, sy);
+                        } else {
+                            dxp[h] = pmul(psub(fc[h], fw), bc(gxw[1]));
+                            V dxm = pmul(psub(fw, at(rc, 0, h)), bc(gxw[0]));
+                            if (p0 == 1) dxm = dxp[h];       // (an overlapping strip next to the wall)
+                            sx = vleer2(dxm, dxp[h]);
+                            sy = yslope(1, h, fw, dyp[0][h]);
+                        }
                         d0[h] = pfma(sx, bc(gxh[0]), fw);
                         gr[h] = pfma(bc(um[h]), sx, pmul(bc(vm[h]), sy));
                     }
@@ -581,13 +601,19 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
                     for (int h = 0; h < VPL; ++h) {
                         f0[h] = fc[h];
                         fc[h] = at(rc, t + 3, h);
-                        V dxn = pmul(psub(fc[h], f0[h]), bc(gxw[t + 2]));
-                        if ((!FULL || t == TX - 1) && p0 + t == nx - 1) dxn = dxp[h];
-                        const V sx = vleer2(dxp[h], dxn), sy = yslope(t + 2, h, f0[h], dyp[t + 1][h]);
+                        V sx, sy;
+                        if (kept) {
+                            kept_slopes(j, t, sx, sy);
+                        } else {
+                            V dxn = pmul(psub(fc[h], f0[h]), bc(gxw[t + 2]));
+                            if ((!FULL || t == TX - 1) && p0 + t == nx - 1) dxn = dxp[h];
+                            sx = vleer2(dxp[h], dxn);
+                            sy = yslope(t + 2, h, f0[h], dyp[t + 1][h]);
+                            dxp[h] = dxn;
+                        }
                         dx0[h] = pfma(sx, bc(gxh[t + 1]), f0[h]);
                         dy0[h] = pfma(sy, bc(gyh[r]), f0[h]);
                         gr[h] = pfma(bc(um[h]), sx, pmul(bc(vm[h]), sy));
-                        dxp[h] = dxn;
                     }
                     const bool more = t + 1 < TX && (FULL || p0 + t + 1 < nx);   // another cell in this row
                     const char* tcell = ahead(tc0, 2 * t);
