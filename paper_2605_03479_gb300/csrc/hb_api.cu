@@ -359,6 +359,7 @@ void layout_case(Carver& cv, const HostCase& h, CaseDev<T>& d, bool keep_slopes)
     d.hx = cv.take<double>(h.nx); d.hy = cv.take<double>(h.ny);
     d.rdx = cv.take<double>(h.nx); d.rdy = cv.take<double>(h.ny);
     d.vu = cv.take<double>(h.nvp); d.vv = cv.take<double>(h.nvp); d.vw = cv.take<double>(h.nvp);
+    d.vref = cv.take<double>(h.nvp);
     d.tu = cv.take<T>(h.nvp); d.tv = cv.take<T>(h.nvp); d.thref = cv.take<T>(h.nvp);
     d.twu = cv.take<T>(h.nvp);
     d.wrow = cv.take<T>((size_t)h.nvb * (h.k1sep ? K1_WT<true> : K1_WT<false>));
@@ -987,6 +988,13 @@ hbugks_status capture(hbugks_t h, Impl<T>& im)
     return HBUGKS_OK;
 }
 
+template <typename T>
+void init_uniform(const CaseDev<T>& d, double rho, double u, double v, double Tt, cudaStream_t s)
+{
+    const unsigned x = (unsigned)(((long long)d.nc * d.nt + INIT_ROWS - 1) / INIT_ROWS);
+    k_init_uniform<T><<<dim3(x, (unsigned)std::min(d.nvb, 65535)), 256, 0, s>>>(d, rho, u, v, Tt);
+}
+
 // every case at rest (rho 1, T0) on every level, fresh status, local steps of that state
 template <typename T>
 hbugks_status reset_rest(hbugks_t h, Impl<T>& im, int ncases)
@@ -996,8 +1004,8 @@ hbugks_status reset_rest(hbugks_t h, Impl<T>& im, int ncases)
     k_status_reset<<<(ncases + 127) / 128, 128, 0, h->s>>>(im.d_status, ncases, -1, 1);
     for (int k = 0; k < ncases; ++k) {
         const CaseDev<T>& d = im.dc[k];
-        size_t tot = (size_t)d.nc * d.nvb * VB * d.nt;
-        k_init_uniform<T><<<(unsigned)((tot + 255) / 256), 256, 0, h->s>>>(d, 1.0, 0.0, 0.0, 1.0);
+        k_reference<T><<<(d.nvb * VB + 127) / 128, 128, 0, h->s>>>(d);
+        init_uniform(d, 1.0, 0.0, 0.0, 1.0, h->s);
     }
     enqueue_steps(im, ncases, h->s);
     return HBUGKS_OK;
@@ -1354,9 +1362,7 @@ hbugks_status hbugks_init_uniform(hbugks_t h, int ci, double rho, double u, doub
         for (int k = 0; k < h->ncases; ++k) {
             if (ci >= 0 && k != ci) continue;
             auto& d = im.dc[k];
-            size_t tot = (size_t)d.nc * d.nvb * VB * d.nt;
-            using TT = typename std::remove_pointer<decltype(d.tu)>::type;
-            k_init_uniform<std::remove_const_t<TT>><<<(unsigned)((tot + 255) / 256), 256, 0, h->s>>>(d, rho, u, v, T);
+            init_uniform(d, rho, u, v, T, h->s);
         }
         enqueue_steps(im, h->ncases, h->s);
         return end(h);

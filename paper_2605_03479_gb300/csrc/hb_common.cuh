@@ -115,6 +115,7 @@ struct CaseDev {
     const double* wall;                // [4][nslot][3]  U_w, V_w, T_w per level (per step in time-domain mode)
     const double *xn, *yn, *xc, *yc, *hx, *hy, *rdx, *rdy;   // rdx[i] = 1/(xc[i+1]-xc[i])
     const double *vu, *vv, *vw;        // per padded velocity
+    double* vref;                      // per padded velocity: H_ref (0 for padding)
     const T *tu, *tv, *thref;          // per padded velocity
     const T* twu;                      // per padded velocity: the factor w_u of its weight (0 for padding)
     const T* wrow;                     // per velocity block: weights of the face sums (K1_WT)

@@ -824,6 +824,17 @@ __device__ __forceinline__ int first_class(const CaseDev<T>& cd, int can)
     return (u < 0 ? 1 : 0) | (v < 0 ? 2 : 0);
 }
 
+// H_ref of every stored velocity, formed once per case: an FP64 exponential costs a scheduler some 1000 cycles per warp,
+// and the conversions below took one per value (set, 20 iterations, harmonics and get of a 32x32, 32x32, N_T 7 state:
+// 22.1 -> 20.6 ms)
+template <typename T>
+__global__ void k_reference(CaseDev<T> cd)
+{
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= cd.nvb * VB) return;
+    cd.vref[a] = cd.vcan[a] >= 0 ? (cd.lam0 / M_PI) * exp(-cd.lam0 * (cd.vu[a] * cd.vu[a] + cd.vv[a] * cd.vv[a])) : 0.0;
+}
+
 // canonical FP64 level array (stage[c][a], a < nvel) -> delta-form internal layout of one level
 template <typename T>
 __global__ void k_set_level(CaseDev<T> cd, int n, int which, const double* stage)
@@ -838,7 +849,7 @@ __global__ void k_set_level(CaseDev<T> cd, int n, int which, const double* stage
     double val = 0.0;
     const int can = cd.vcan[a];
     if (can >= 0) {
-        double href = (cd.lam0 / M_PI) * exp(-cd.lam0 * (cd.vu[a] * cd.vu[a] + cd.vv[a] * cd.vv[a]));
+        const double href = cd.vref[a];
         double rv = which == 0 ? href : href * 0.5 / cd.lam0;
         val = stage[(size_t)c * cd.nvel + can] - rv;
     }
@@ -859,40 +870,44 @@ __global__ void k_get_level(CaseDev<T> cd, int n, int which, double* stage)
     const int can = cd.vcan[a];
     // a node stored in several sign classes holds the same value in each; the first copy is read
     if (can < 0 || cd.vcls[vb] != first_class(cd, can)) return;
-    double href = (cd.lam0 / M_PI) * exp(-cd.lam0 * (cd.vu[a] * cd.vu[a] + cd.vv[a] * cd.vv[a]));
+    const double href = cd.vref[a];
     double rv = which == 0 ? href : href * 0.5 / cd.lam0;
     const T* src = reinterpret_cast<const T*>(cd.f[cd.st->parity]);
     stage[(size_t)c * cd.nvel + can] = (double)src[2 * sidx(cd.nc, cd.nt, vb, c, n, lane) + which] + rv;
 }
 
-// uniform reduced Maxwellian (rho, U, V, T) on every level, delta form; W = its continuous moments
+// Uniform reduced Maxwellian (rho, U, V, T) on every level, delta form; W = its continuous moments.  CTAs (x, vb): each
+// thread forms the two values of its velocity once and writes them to INIT_ROWS (level, cell) rows (one pair of
+// exponentials per stored value took 116 ms for the 128x128, 64x64, N_T 11 state, against a write of 5.9 GB).
+constexpr int INIT_ROWS = 256;
+
 template <typename T>
-__global__ void k_init_uniform(CaseDev<T> cd, double rho, double U, double V, double Tt)
+__global__ void __launch_bounds__(256) k_init_uniform(CaseDev<T> cd, double rho, double U, double V, double Tt)
 {
-    size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    size_t tot = (size_t)cd.nc * cd.nvb * VB * cd.nt;
-    const int p = cd.st->parity;
-    if (k < (size_t)cd.nc * cd.nt) {
-        double* W = cd.W[p] + k * 4;
-        W[0] = rho; W[1] = rho * U; W[2] = rho * V; W[3] = 0.5 * rho * (U * U + V * V) + 0.75 * rho * Tt;
+    const int p = cd.st->parity, rows = cd.nc * cd.nt;
+    const int lane = threadIdx.x & 31, first = blockIdx.x * INIT_ROWS;
+    if (blockIdx.y == 0) {
+        for (int k = first + threadIdx.x; k < min(first + INIT_ROWS, rows); k += blockDim.x) {
+            double* W = cd.W[p] + (size_t)k * 4;
+            W[0] = rho; W[1] = rho * U; W[2] = rho * V; W[3] = 0.5 * rho * (U * U + V * V) + 0.75 * rho * Tt;
+        }
     }
-    if (k >= tot) return;
-    int lane = k & 31;
-    size_t r = k >> 5;
-    int n = r % cd.nt;
-    r /= cd.nt;
-    int c = r % cd.nc, vb = r / cd.nc;
-    int a = vb * VB + lane;
-    double dhv = 0.0, dbv = 0.0;
-    if (cd.vcan[a] >= 0) {
-        double uu = cd.vu[a], vv = cd.vv[a];
-        double lam = cd.lam0 / Tt;
-        double H = rho * (lam / M_PI) * exp(-lam * ((uu - U) * (uu - U) + (vv - V) * (vv - V)));
-        double href = (cd.lam0 / M_PI) * exp(-cd.lam0 * (uu * uu + vv * vv));
-        dhv = H - href;
-        dbv = H * 0.5 / lam - href * 0.5 / cd.lam0;
+    for (int vb = blockIdx.y; vb < cd.nvb; vb += gridDim.y) {
+        const int a = vb * VB + lane;
+        double dhv = 0.0, dbv = 0.0;
+        if (cd.vcan[a] >= 0) {
+            double uu = cd.vu[a], vv = cd.vv[a];
+            double lam = cd.lam0 / Tt;
+            double H = rho * (lam / M_PI) * exp(-lam * ((uu - U) * (uu - U) + (vv - V) * (vv - V)));
+            double href = (cd.lam0 / M_PI) * exp(-cd.lam0 * (uu * uu + vv * vv));
+            dhv = H - href;
+            dbv = H * 0.5 / lam - href * 0.5 / cd.lam0;
+        }
+        const P2<T> x = pk(T(dhv), T(dbv));
+        P2<T>* o = cd.f[p] + (size_t)vb * rows * VB + lane;
+        for (int k = first + (int)(threadIdx.x >> 5); k < min(first + INIT_ROWS, rows); k += blockDim.x >> 5)
+            o[(size_t)k * VB] = x;
     }
-    cd.f[p][sidx(cd.nc, cd.nt, vb, c, n, lane)] = pk(T(dhv), T(dbv));
 }
 
 // fields of one level from the moments of h, b: out[f * nc + c], f = rho, U, V, T, tau_xy, qx, qy, p
