@@ -750,13 +750,21 @@ constexpr int K5_THREADS = 128;
 template <typename T>
 __device__ __forceinline__ void finish_case(const CaseDev<T>& cd, int nb)
 {
-    CaseStatus* st = cd.st;
-    if (!st->active || *(volatile int*)cd.err) return;   // a failed wait leaves the iteration unfinished
+    // every load is issued before the first is needed: the kernel is one CTA per case and waits for little else
+    // (8.1 -> 6.1 us, 8x8 cells)
+    CaseStatus* const st = cd.st;
+    const double* __restrict__ rp = cd.rpart;
+    double* const hist = cd.rhist;
+    const double inv = rcp64((double)cd.nc);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int active = st->active, parity = st->parity, failed = *(volatile int*)cd.err;
+    const long long iters = st->iters, iters_call = st->iters_call;
+    const double tol = *cd.tol;
     // thread t sums variable t & 3 of every 32nd partial; then a fixed tree over lanes and warps
     __shared__ double part[K5_THREADS / 32][4];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double s = 0.0;
-    for (int b = threadIdx.x >> 2; b < nb; b += K5_THREADS / 4) s += cd.rpart[(size_t)b * 4 + (lane & 3)];
+    for (int b = threadIdx.x >> 2; b < nb; b += K5_THREADS / 4) s += rp[(size_t)b * 4 + (lane & 3)];
+    if (!active || failed) return;                       // a failed wait leaves the iteration unfinished
 #pragma unroll
     for (int o = 16; o >= 4; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane < 4) part[warp][lane] = s;
@@ -764,23 +772,18 @@ __device__ __forceinline__ void finish_case(const CaseDev<T>& cd, int nb)
     if (warp == 0) {
         // lanes 0..3: one variable each
         const int k = lane & 3;
-        const double R = sqrt((part[0][k] + part[1][k] + part[2][k] + part[3][k]) / cd.nc);
+        const double R = sqrt((part[0][k] + part[1][k] + part[2][k] + part[3][k]) * inv);
         const bool bad = __any_sync(0xffffffffu, !(R <= 1e10));   // also catches NaN
         if (lane < 4) {
             st->last[k] = R;
-            cd.rhist[(st->iters % RING) * 4 + k] = R;
+            hist[(iters % RING) * 4 + k] = R;
         }
-        __syncwarp();
         if (lane == 0) {
-            st->iters += 1;
-            st->iters_call += 1;
-            st->parity ^= 1;
-            if (bad) {
-                st->diverged = 1;
-                st->active = 0;
-            } else if (*cd.tol > 0.0 && st->iters >= 10 && R <= *cd.tol) {
-                st->active = 0;
-            }
+            st->iters = iters + 1;
+            st->iters_call = iters_call + 1;
+            st->parity = parity ^ 1;
+            if (bad) st->diverged = 1;
+            if (bad || (tol > 0.0 && iters + 1 >= 10 && R <= tol)) st->active = 0;
         }
     }
 }
@@ -802,10 +805,12 @@ __global__ void __launch_bounds__(K5_THREADS) k5_finish(const CaseDev<T>* cases,
     if constexpr (LOOP) {
         __syncthreads();
         if (threadIdx.x != 0) return;
-        __threadfence();
-        if (atomicAdd(loop.left + 1, 1) != ncases - 1) return;
-        __threadfence();
-        loop.left[1] = 0;
+        if (ncases > 1) {
+            __threadfence();
+            if (atomicAdd(loop.left + 1, 1) != ncases - 1) return;
+            __threadfence();
+            loop.left[1] = 0;
+        }
         const int r = loop.left[0] - 1;
         loop.left[0] = r;
         int any = 0;
