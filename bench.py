@@ -30,9 +30,9 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "HB-UGKS cell*velocity*level updates/s"
-# ncu DRAM bytes (read + write) per update of one k4_cells launch on the 64x64-cell, 64x64-velocity, N_T = 11
-# thermal cavity, by micro-update variant (tile x, tile y, velocity blocks per CTA); see profiles/
-K4_TRAFFIC_64 = {(4, 2, 2): 19.2881}
+# ncu DRAM bytes (read + write) per update of one micro-update launch on the 64x64-cell, 64x64-velocity, N_T = 11
+# thermal cavity, by micro-update variant (tile x, tile y, velocity blocks per CTA); none captured for k4_march yet
+K4_TRAFFIC_64 = {}
 UNIT = "updates/s"
 
 
@@ -609,7 +609,7 @@ def main():
     if names[top] in alg:
         ach = alg[names[top]] * upd / (kms[top] * 1e-3) / 1e9
         # DRAM bytes per update of the micro update (dram__bytes_read.sum + dram__bytes_write.sum of one ncu
-        # launch of k4_cells on the 64x64-cell thermal cavity with the 64x64 velocity grid and N_T = 11, per
+        # launch of k4_march on the 64x64-cell thermal cavity with the 64x64 velocity grid and N_T = 11, per
         # micro-update variant), scaled by updates; only where the launches match that capture: the same
         # variant, the 64x64 velocity grid, N_T = 11
         traffic = None
