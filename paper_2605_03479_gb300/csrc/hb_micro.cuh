@@ -149,12 +149,6 @@ __device__ __forceinline__ void spectral_cells(const char* row, uint32_t ls, int
     }
 }
 
-// barrier of one group's warps (named barrier 1 + group; at most 15 groups)
-__device__ __forceinline__ void group_sync(int group, int threads)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(threads) : "memory");
-}
-
 // One bulk copy of the per-row batches, formed once per warp: in batch b (lo <= b <= hi) it reads src + (b - 1) stride
 // and lands at dst, plus the slot of the row it belongs to.
 struct alignas(16) K4Copy {
@@ -177,7 +171,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
     constexpr bool FULL = TX == 4;
     constexpr int NCOPY = VPL + 3;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t full_[MAXNT][2], done_[MAXNT];       // per group
+    __shared__ uint64_t full_[MAXNT][2], done_[MAXNT], meet_[IMP ? MAXNT : 1];   // per group
     __shared__ int abort_flag;                               // set by the first warp whose wait runs out
     __shared__ K4Copy copies[MAXNT][NCOPY];                  // per warp
     int lb;
@@ -194,6 +188,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
     const int tid = (int)threadIdx.x - gi * nt * 32, nthreads = nt * 32;   // in the group
     uint64_t* const full = full_[gi];
     uint64_t* const done = &done_[gi];
+    uint64_t* const meet = &meet_[IMP ? gi : 0];             // (implicit source)
     // CTA order: velocity group fastest (the CTAs of one strip share its parameters in L2), then strips, segments
     int ng = 0;
 #pragma unroll
@@ -223,6 +218,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
         mbar_init(&full[0], nt);
         mbar_init(&full[1], nt);
         mbar_init(done, nt);
+        if (IMP) mbar_init(meet, nt);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // spacings in mirrored order: gxw[k] twice the inverse distance of columns p0 - 2 + k and p0 - 1 + k, gxh[k] half
@@ -384,6 +380,13 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
     // that none still lands in shared memory after the CTA exits
     auto give_up = [&](int b) {
         for (int k = b; k <= issued; ++k) mbar_drain(&full[k & 1], (uint32_t)((k >> 1) & 1));
+    };
+    // The group's warps meet twice per row with the implicit source, so the phases are 0 and 1 in turn.  Bounded like every
+    // wait: a warp that has given up elsewhere never arrives here.
+    auto group_meet = [&](uint32_t phase) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(meet);
+        return mbar_wait(meet, phase, err, &abort_flag);
     };
     if (!mbar_wait(&full[0], 0, err, &abort_flag)) { give_up(0); return; }
     if (expire) {
@@ -658,7 +661,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
                 }
                 if (implicit) {
                     // spectral source at the new iterate: f^{k+1} = minv (right-hand sides over the levels), per cell
-                    group_sync(gi, nthreads);
+                    if (!group_meet(0)) { give_up(r + 1); return; }
 #pragma unroll
                     for (int t = 0; t < TX; ++t) {
                         if (!FULL && p0 + t >= nx) break;
@@ -676,7 +679,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
                         for (int h = 0; h < VPL; ++h)
                             if (h == 0 || two) on[h * bstride + t * SG * VB] = acc[h];
                     }
-                    group_sync(gi, nthreads);
+                    if (!group_meet(1)) { give_up(r + 1); return; }
                 }
             }
             __syncwarp();
