@@ -153,10 +153,11 @@ __device__ __forceinline__ void spectral_cells(const char* row, uint32_t ls, int
 // and lands at dst, plus the slot of the row it belongs to.
 struct alignas(16) K4Copy {
     const char* src;
-    int stride;
+    long long stride;
     uint32_t dst, bytes;
-    int lo, hi, pad;
+    int lo, hi;
 };
+static_assert(sizeof(K4Copy) == 32);
 
 template <class P, int TX, int VPL, bool IMP, int MAXT>
 __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, int rows, int groups)
@@ -247,15 +248,14 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
     const uint32_t rb = (uint32_t)(c1 - c0) * Y::COL, xb = (uint32_t)(f1_ - f0_) * (uint32_t)(NP * sizeof(T)),
                    yb = (uint32_t)(o1 - o0) * (uint32_t)(NP * sizeof(T)),
                    cb = (uint32_t)(o1 - o0) * (uint32_t)(NCP * sizeof(T));
-    const int ysgn = yneg ? -1 : 1;
+    const long long ysgn = yneg ? -1 : 1;                    // (row strides in bytes may pass 31 bits)
     if (lane < NCOPY) {
         const int q = q0 - 1, j = yneg ? ny - 1 - q : q, fj = yneg ? ny - 1 - q : q + 1;   // stream row 1
         K4Copy c;
-        c.pad = 0;
         if (lane < VPL) {
             c.src = reinterpret_cast<const char*>(cd.f[par] + (size_t)(vb + (two ? lane : 0)) * bstride +
                                                   (size_t)n * nc * VB + ((long long)(j + ysgn) * nx + c0) * VB);
-            c.stride = ysgn * nx * (int)Y::COL;
+            c.stride = ysgn * nx * (long long)Y::COL;
             c.dst = smem_u32(srow) + n * Y::ROW + lane * Y::BLK + (uint32_t)(c0 - lowc) * Y::COL;
             c.bytes = rb;
             c.lo = 1;
@@ -264,17 +264,17 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
             const uint32_t base = smem_u32(spar) + n * Y::PAR;
             if (lane == VPL) {
                 c.src = reinterpret_cast<const char*>(cd.fpar + ((long long)n * cd.nf + (long long)j * (nx + 1) + f0_) * NP);
-                c.stride = ysgn * (nx + 1) * (int)(NP * sizeof(T));
+                c.stride = ysgn * (nx + 1) * (long long)(NP * sizeof(T));
                 c.dst = base + (uint32_t)((f0_ - lowf) * NP * sizeof(T));
                 c.bytes = xb;
             } else if (lane == VPL + 1) {
                 c.src = reinterpret_cast<const char*>(cd.fpar + ((long long)n * cd.nf + nfx + (long long)fj * nx + o0) * NP);
-                c.stride = ysgn * nx * (int)(NP * sizeof(T));
+                c.stride = ysgn * nx * (long long)(NP * sizeof(T));
                 c.dst = base + Y::PX + (uint32_t)((o0 - lowo) * NP * sizeof(T));
                 c.bytes = yb;
             } else {
                 c.src = reinterpret_cast<const char*>(cd.cpar + ((long long)n * nc + (long long)j * nx + o0) * NCP);
-                c.stride = ysgn * nx * (int)(NCP * sizeof(T));
+                c.stride = ysgn * nx * (long long)(NCP * sizeof(T));
                 c.dst = base + Y::PX + Y::PY + (uint32_t)((o0 - lowo) * NCP * sizeof(T));
                 c.bytes = cb;
             }
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
             const K4Copy c = copies[warp][lane];
             if (b >= c.lo && b <= c.hi)
                 bulk_g2s_at(c.dst + (lane < VPL ? slot * slot_b : (uint32_t)(b & 1) * pslot_b),
-                            c.src + (long long)(b - 1) * c.stride, c.bytes, bar);
+                            c.src + (b - 1) * c.stride, c.bytes, bar);
         }
     };
     if (lane == 0) {
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
         const int row = lane / VPL;
         const K4Copy c = copies[warp][lane % VPL];
         if (q0 + row >= 2)
-            bulk_g2s_at(c.dst + (uint32_t)row * slot_b, c.src + (long long)(row - 2) * c.stride, c.bytes, &full[0]);
+            bulk_g2s_at(c.dst + (uint32_t)row * slot_b, c.src + (row - 2) * c.stride, c.bytes, &full[0]);
     }
     issue(1, 2);
     int issued = 1;
