@@ -335,12 +335,12 @@ __device__ __forceinline__ void prim(const double* W, double& rho, double& U, do
     lam = 0.75 * rho * rcp64(fma(-0.5 * rho, fma(U, U, V * V), W[3]));
 }
 
-// tau = mu/p, mu = mu0 (T/T0)^w, T/T0 = lam0/lam, p = rho/(2 lam); ir = 1/rho, il0 = 1/lam0.  The power as
-// exp(-w log(lam/lam0)): both within a few ulp, for half the instructions of pow, whose extra digits of the
-// logarithm serve exponents far from the w = 0.5..1 of a viscosity law.
-__device__ __forceinline__ double relax_time(double mu0, double w, double il0, double ir, double lam)
+// tau = mu/p, mu = mu0 (T/T0)^w, T/T0 = lam0/lam, p = rho/(2 lam); ir = 1/rho, i2l = 1/(2 lam).  pow, not
+// exp(-w log(lam/lam0)): it keeps the last digits of the logarithm, and with a whole exponent it is defined for the
+// negative temperature a cell may pass through.
+__device__ __forceinline__ double relax_time(double mu0, double w, double lam0, double ir, double lam, double i2l)
 {
-    return mu0 * exp(-w * log(lam * il0)) * 2.0 * lam * ir;
+    return mu0 * pow(2.0 * lam0 * i2l, w) * 2.0 * lam * ir;
 }
 
 // Coefficients of Eq. C_coeffs: Taylor series in x = dG/tau below x = 1 (the printed forms cancel there),

@@ -72,10 +72,11 @@ __device__ __forceinline__ void heat_flux_raw(const double* A, double U, double 
 
 // A CTA takes K2_ITEMS (face, level) items with one lane each in every one of its four warps, which divide the work:
 //   A  interface state from the velocity sums (each warp for itself), then warp 0 the heat flux and Shakhov factor,
-//      1 and 2 the slopes a^L and a^R, 3 the slope a_t, the relaxation time and the weights C1..C5;
+//      1 and 2 the slopes a^L and a^R, 3 the slope a_t;
 //   B  all warps: the expm1 table of the interface Maxwellian (lanes over the nodes, one item after another) and its
 //      27 sums per axis (lanes over the items, a warp per power);
-//   C  warp 0 the compatibility condition (A), 1 the Shakhov moments, 2 and 3 the moments of the left and right slopes;
+//   C  warp 0 the compatibility condition (A), 1 the Shakhov moments, the relaxation time and the weights C1..C5, 2 and 3
+//      the moments of the left and right slopes;
 //   D  warp 0 the macro flux and the wall density, 1 and 2 the micro-flux parameters of the two upwind sides, 3 the rest.
 // On small meshes the time is the chain of one thread, in large ones FP64 instructions and latency at few warps.
 // Against one thread per item doing all of it (219 registers, nine FP64 instructions per division, polynomials in (u, v)
@@ -253,17 +254,6 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
         tco[2][lane] = T(lamf * U0 * U0);
         tco[3][lane] = T(2.0 * lamf * V0);
         tco[4][lane] = T(lamf * V0 * V0);
-        // face step (Eq. dt_face) and time-integration weights (Eq. C_coeffs)
-        double dGf;
-        if (!g.hasL) dGf = cd.dG[cR];
-        else if (!g.hasR) dGf = cd.dG[cL];
-        else if (cd.face_step == 1) dGf = 2.0 * cd.dG[cL] * cd.dG[cR] * rcp64(cd.dG[cL] + cd.dG[cR]);
-        else dGf = fmin(cd.dG[cL], cd.dG[cR]);
-        sdG[lane] = dGf;
-        T Ct[5];
-        ugks_coeffs<T>(T(dGf), T(relax_time(cd.mu0, cd.w_vss, il0, ir, lamf)), Ct);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) Cw[k][lane] = Ct[k];
     }
     __syncthreads();
 
@@ -371,6 +361,17 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
         rows(half, x, y);
         mom4<1, true>(c, shk_[10][lane], shk_[11][lane], shk_[12][lane], x, y, pref, i2l, o);
         put(F1s, o);
+        // face step (Eq. dt_face) and time-integration weights (Eq. C_coeffs), here beside warp 0's longer part
+        double dGf;
+        if (!g.hasL) dGf = cd.dG[cR];
+        else if (!g.hasR) dGf = cd.dG[cL];
+        else if (cd.face_step == 1) dGf = 2.0 * cd.dG[cL] * cd.dG[cR] * rcp64(cd.dG[cL] + cd.dG[cR]);
+        else dGf = fmin(cd.dG[cL], cd.dG[cR]);
+        sdG[lane] = dGf;
+        T Ct[5];
+        ugks_coeffs<T>(T(dGf), T(relax_time(cd.mu0, cd.w_vss, cd.lam0, ir, lamf, i2ld)), Ct);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) Cw[k][lane] = Ct[k];
     } else {
         // C2 term: u_n (u_n P(a_bar) + u_t P(a_t)), a_bar = a^L for u_n > 0 (warp 2), a^R for u_n < 0 (warp 3; at a wall
         // the incident velocities' one side is warp 2's)
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
             for (int k = 0; k < 13; ++k) A[k] = cm[k] + cd.refmom[k];
             prim(Wc, rho, U, V, lam);
             heat_flux_raw(A, U, V, qx, qy);
-            tau = relax_time(cd.mu0, cd.w_vss, il0, rcp64(rho), lam);
+            tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, rcp64(rho), lam, 0.5 * rcp64(lam));
             sq[r][0] = qx;
             sq[r][1] = qy;
         } else {
@@ -635,7 +636,7 @@ __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
 #pragma unroll
         for (int k = 0; k < 4; ++k) Wn[((size_t)n * nc + c) * 4 + k] = wn[k];
         prim(wn, rho, U, V, lam);
-        tau = relax_time(cd.mu0, cd.w_vss, il0, rcp64(rho), lam);
+        tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, rcp64(rho), lam, 0.5 * rcp64(lam));
         stau[r] = tau;
         snu[r] = nu_conv(cd, U, V, lam, idx_, idy);        // for the next local step
     }
