@@ -17,7 +17,7 @@
 // latency was 46 % of the stalls), and the x direction is a template parameter so that all offsets within a row are
 // constants.  Strips of two columns with 128 registers hold more warps per SM and win up to 7 levels (0.83 against
 // 1.02 ms, 64x64, 48x48, N_T 7), strips of four with 168 recompute less and win above (8.3 ms, 128x128, 64x64, N_T 11).
-// Bound by the FP64 pipe in FP64: everything relative to H_ref saves 9 of 178 instructions per update.  Previous kernel
+// Bound by the FP64 pipe in FP64.  Previous kernel
 // -> this one: 16.25 -> 8.27 ms (128x128, 64x64, N_T 11), 1.50 -> 0.83 ms (64x64, 48x48, N_T 7), 44.5 -> 25.8 ms (48
 // uneven cavities), 0.60 -> 0.32 ms (90x90, 28x28, N_T 3); FP64 58.1 -> 46.4 ms (twelve 64x64, 32x32, N_T 3) and 25.8 ->
 // 20.8 ms (64x64, 48x48, N_T 7).
@@ -47,12 +47,13 @@ template <> struct Lane1<float2> {
     static __device__ __forceinline__ float2 of(const float* x) { return make_float2(x[0], x[1]); }
 };
 
-// Maxwellian part of the micro flux divided by dG_f, u_n and H_ref (delta form).  With G = H/H_ref - 1 it is
-// C1' G + (1 + G) Q = Q + G (Q + C1') for h, and i2l [Qb + G (Qb + C1')] + C1' (i2l - i2l0) for b (Qb = Q + lin), from
-// the face's parameters fp (shared memory; cubic at qo, linear term at lo: the upwind side's) and the expm1 factors
-// (ex, ey) of the interface Maxwellian at the lane's velocities; c4, c5: C4', C5'
+// Maxwellian part of the micro flux divided by dG_f and u_n (delta form): C1' dH + H Q for h and i2l (C1' dH + H Qb) +
+// C1' (i2l - i2l0) H_ref for b (Qb = Q + lin), from the face's parameters fp (shared memory; cubic at qo, linear term at
+// lo: the upwind side's), the expm1 factors (ex, ey) of the interface Maxwellian and H_ref (hr) at the lane's velocities;
+// c4, c5: C4', C5'.  H/H_ref is multiplied by H_ref before anything else: far out on a wide velocity grid in hot gas it
+// nears the largest float, which its product with Q would pass.
 template <typename T, typename L>
-__device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L ey, L u, L v, L& mh, L& mb, T& c4, T& c5)
+__device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L ey, L u, L v, L hr, L& mh, L& mb, T& c4, T& c5)
 {
     using A = Lane1<L>;
     T sc[8], c[12], l[4];          // sc: r - 1, r, 1/(2 lam), 1/(2 lam) - 1/(2 lam0), C1', C4', C5', C1' times slot 3
@@ -61,41 +62,41 @@ __device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L e
     load_par(fp + lo, l);
     c4 = sc[5];
     c5 = sc[6];
-    const L G = pfma(A::all(sc[1]), pfma(ex, ey, padd(ex, ey)), A::all(sc[0]));
+    const L dH = pmul(hr, pfma(A::all(sc[1]), pfma(ex, ey, padd(ex, ey)), A::all(sc[0])));
+    const L H = padd(hr, dH), cH = pmul(A::all(sc[4]), dH);
     // Horner form of the bivariate cubic with monomials 1, u, v, u^2, uv, v^2, u^3, u^2 v, u v^2, v^3
     const L y0 = pfma(v, pfma(v, pfma(v, A::all(c[9]), A::all(c[5])), A::all(c[2])), A::all(c[0]));
     const L y1 = pfma(v, pfma(v, A::all(c[8]), A::all(c[4])), A::all(c[1]));
     const L y2 = pfma(u, A::all(c[6]), pfma(v, A::all(c[7]), A::all(c[3])));
     const L Q = pfma(u, pfma(u, y2, y1), y0);
     const L Qb = pfma(v, A::all(l[2]), pfma(u, A::all(l[1]), padd(Q, A::all(l[0]))));
-    const L c1 = A::all(sc[4]);
-    mh = pfma(G, padd(Q, c1), Q);
-    mb = pfma(A::all(sc[2]), pfma(G, padd(Qb, c1), Qb), A::all(sc[7]));
+    mh = pfma(H, Q, cH);
+    mb = pfma(A::all(sc[2]), pfma(H, Qb, cH), pmul(hr, A::all(sc[7])));
 }
 
-// Equilibrium (H+ - H_ref, B+ - B_ref) divided by H_ref of one cell-parameter slot q at the lane's velocities: G and
-// i2l G + (i2l - i2l0) of the Maxwellian (cell table factors ex, ey), and with the Shakhov model
-// G + (1 + G) sk = sk + G (1 + sk), sk = L Q, for h and the same with sk + 2 L for b (L, Q the linear and quadratic
-// factors of s (c.q)(2 lam |c|^2 - 4); r2 = u^2 + v^2)
+// Equilibrium (H+ - H_ref, B+ - B_ref) of one cell-parameter slot q at the lane's velocities: dH and i2l dH +
+// (i2l - i2l0) H_ref of the Maxwellian (cell table factors ex, ey; hr = H_ref), and with the Shakhov model dH + H sk,
+// sk = L Q, for h and the same with sk + 2 L for b (L, Q the linear and quadratic factors of s (c.q)(2 lam |c|^2 - 4);
+// r2 = u^2 + v^2)
 template <bool SHAKHOV, typename T, typename L>
-__device__ __forceinline__ void eq_core(const T* qp, L ex, L ey, L u, L v, L r2, L& mh, L& mb)
+__device__ __forceinline__ void eq_core(const T* qp, L ex, L ey, L u, L v, L r2, L hr, L& mh, L& mb)
 {
     using A = Lane1<L>;
     T q[12];
     load_par(qp, q);
-    const L G = pfma(A::all(q[E_R]), pfma(ex, ey, padd(ex, ey)), A::all(q[E_RM1]));
-    const L i2l = A::all(q[E_I2L]), di2l = A::all(q[E_DI2L]);
+    const L dH = pmul(hr, pfma(A::all(q[E_R]), pfma(ex, ey, padd(ex, ey)), A::all(q[E_RM1])));
+    const L i2l = A::all(q[E_I2L]), dB = pmul(hr, A::all(q[E_DI2L]));
     if constexpr (!SHAKHOV) {
-        mh = G;
-        mb = pfma(i2l, G, di2l);
+        mh = dH;
+        mb = pfma(i2l, dH, dB);
         return;
     }
     const L Lf = pfma(A::all(q[E_L + 2]), v, pfma(A::all(q[E_L + 1]), u, A::all(q[E_L])));
     const L Qs = pfma(A::all(q[E_Q + 3]), r2,
                       pfma(A::all(q[E_Q + 2]), v, pfma(A::all(q[E_Q + 1]), u, A::all(q[E_Q]))));
-    const L sk = pmul(Lf, Qs), sb = pfma(A::all(T(2)), Lf, sk), one = A::all(T(1));
-    mh = pfma(G, padd(one, sk), sk);
-    mb = pfma(i2l, pfma(G, padd(one, sb), sb), di2l);
+    const L sk = pmul(Lf, Qs), sb = pfma(A::all(T(2)), Lf, sk), H = padd(hr, dH);
+    mh = pfma(H, sk, dH);
+    mb = pfma(i2l, pfma(H, sb, dH), dB);
 }
 
 constexpr int K4_MAXROWS = 32;   // rows per segment
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
         iu[h] = (uint32_t)__ldg(cd.viu + av) * (uint32_t)sizeof(T);
         iv[h] = (uint32_t)(cd.nu + __ldg(cd.viv + av)) * (uint32_t)sizeof(T);
     }
-    const L uL = A::of(u), vL = A::of(v), r2L = A::of(rr2);
+    const L uL = A::of(u), vL = A::of(v), r2L = A::of(rr2), hL = A::of(hr);
     const bool shakhov = cd.shakhov != 0;
     const bool implicit = IMP && cd.spectral_implicit != 0;
     const int nh = implicit ? 0 : cd.nh;
@@ -371,10 +372,10 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
     auto face_flux = [&](const char* fp, int qo, int lo, L ex, L ey, const V (&d0)[VPL], const V (&gr)[VPL], V (&F)[VPL]) {
         L mh, mb;
         T c4, c5;
-        flux_core<T, L>(reinterpret_cast<const T*>(fp), qo, lo, ex, ey, uL, vL, mh, mb, c4, c5);
+        flux_core<T, L>(reinterpret_cast<const T*>(fp), qo, lo, ex, ey, uL, vL, hL, mh, mb, c4, c5);
 #pragma unroll
         for (int h = 0; h < VPL; ++h)
-            F[h] = pfma(bc(hr[h]), pk(A::at(mh, h), A::at(mb, h)), pfma(bc(c4), d0[h], pmul(bc(c5), gr[h])));
+            F[h] = pfma(bc(c4), d0[h], pfma(bc(c5), gr[h], pk(A::at(mh, h), A::at(mb, h))));
     };
     // a wait ran out: this warp waits (bounded) for the batches from b on that it has issued and not seen complete, so
     // that none still lands in shared memory after the CTA exits
@@ -639,11 +640,11 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
                     if (EARLY) load_c(more ? ahead(tc0, 2 * (t + 1)) : tc0);
                     L h1, b1, h0, b0;
                     if (shakhov) {
-                        eq_core<true, T, L>(cp + C_EQ1, ex1, ey1, uL, vL, r2L, h1, b1);
-                        eq_core<true, T, L>(cp + C_EQ0, ex0, ey0, uL, vL, r2L, h0, b0);
+                        eq_core<true, T, L>(cp + C_EQ1, ex1, ey1, uL, vL, r2L, hL, h1, b1);
+                        eq_core<true, T, L>(cp + C_EQ0, ex0, ey0, uL, vL, r2L, hL, h0, b0);
                     } else {
-                        eq_core<false, T, L>(cp + C_EQ1, ex1, ey1, uL, vL, r2L, h1, b1);
-                        eq_core<false, T, L>(cp + C_EQ0, ex0, ey0, uL, vL, r2L, h0, b0);
+                        eq_core<false, T, L>(cp + C_EQ1, ex1, ey1, uL, vL, r2L, hL, h1, b1);
+                        eq_core<false, T, L>(cp + C_EQ0, ex0, ey0, uL, vL, r2L, hL, h0, b0);
                     }
                     T kp[12];                                // kself, -kE, kp1, kp0, -kdx, -kdy, each twice
                     load_par(cp + C_K, kp);
@@ -653,8 +654,8 @@ __global__ void __launch_bounds__(MAXT) k4_march(const __grid_constant__ P B, in
                         x = pfma(bc(kp[8] * um[h]), dX[h], x);
                         x = pfma(bc(kp[10] * vm[h]), dY[h], x);
                         x = pfma(pk(kp[2], kp[3]), e[t & 1][h], x);
-                        x = pfma(bc(kp[4] * hr[h]), pk(A::at(h1, h), A::at(b1, h)), x);
-                        x = pfma(bc(kp[6] * hr[h]), pk(A::at(h0, h), A::at(b0, h)), x);
+                        x = pfma(pk(kp[4], kp[5]), pk(A::at(h1, h), A::at(b1, h)), x);
+                        x = pfma(pk(kp[6], kp[7]), pk(A::at(h0, h), A::at(b0, h)), x);
                         if (implicit) srhs[(size_t)((n * TX + t) * VPL + h) * VB + lane] = x;
                         else if (h == 0 || two) on[h * bstride + t * SG * VB] = x;
                     }

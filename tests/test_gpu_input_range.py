@@ -40,3 +40,26 @@ def test_negative_temperature_with_a_whole_viscosity_exponent(hb, w_vss):
     W, h, b = I.initial_state(c, seed=3)
     W[1, 7, 3] = -0.2
     compare(hb, c, (W, h, b), 1, 1e-10, 1e-13)
+
+
+@pytest.mark.parametrize("half_width", [7.8, 7.84, 7.88])
+def test_wide_velocity_grid_in_hot_gas(hb, half_width):
+    # gas at 3.8 T0 with a large heat flux on a grid so wide that H/H_ref reaches 1e37 in its corners, where H_ref lies
+    # below the smallest 32-bit value: H (1 + Shakhov factor) is finite there though (H/H_ref)(1 + factor) is not
+    c = I.make_case("hot", 6, 24, kn=10.0, st=1.0, nh=1, pr=0.3, drive="thermal", amp=0.3, precision=1,
+                    half_width=half_width)
+    for w in c.walls:
+        w[2] = 3.8
+    x, y = (0.5 * (n[1:] + n[:-1]) for n in (c.xnodes, c.ynodes))
+    X, Y = (a.ravel() for a in np.meshgrid(x, y))
+    u, v = np.tile(c.u, c.nv), np.repeat(c.v, c.nu)
+    skew = 1.0 + 0.9 * np.tanh((u + v) ** 3 / 40.0 - (u + v))
+    W, h = np.zeros((c.nt, c.nc, 4)), np.zeros((c.nt, c.nc, c.nvel))
+    b = np.zeros_like(h)
+    for n in range(c.nt):
+        T = 3.8 + 0.4 * np.cos(np.pi * X + 0.3 * n) * np.cos(np.pi * Y)
+        rho, U, V = 1.0 + 0.1 * np.sin(2 * X + n) * Y, 0.1 * np.sin(3 * Y + n), 0.1 * np.cos(2 * X)
+        H = (rho / (np.pi * T))[:, None] * np.exp(-((u - U[:, None]) ** 2 + (v - V[:, None]) ** 2) / T[:, None])
+        h[n], b[n] = H * skew, H * skew * 0.5 * T[:, None]
+        W[n] = np.stack([rho, rho * U, rho * V, 0.5 * rho * (U ** 2 + V ** 2) + 0.75 * rho * T], 1)
+    compare(hb, c, (W, h, b), 1, 2e-5, 2e-7)
