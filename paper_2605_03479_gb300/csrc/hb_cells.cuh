@@ -423,14 +423,15 @@ __global__ void __launch_bounds__(TX * TY * 32, CTAS) k1_cells(const __grid_cons
                     ys[0] = pfma(syv.x, a[3], ys[0]); ys[1] = pfma(syv.x, d[2], ys[1]); ys[2] = pfma(syv.x, d[3], ys[2]); ys[3] = pfma(syv.x, e[0], ys[3]);
                     ys[4] = pfma(syv.x, e[1], ys[4]); ys[5] = pfma(syv.x, e[3], ys[5]); ys[6] = pfma(syv.x, wr, ys[6]);
                     if constexpr (!INNER) {
-                        // a velocity parallel to a wall (u^2 w = 0) carries nothing into it
+                        // a velocity parallel to a wall (u w = 0; not u^2 w, which a small u brings below the smallest
+                        // 32-bit value) carries nothing into it
                         const bool xn = (cur & 1) != 0, yn = (cur & 2) != 0;
-                        if ((xn ? !hm : !hp) && a[3] == T(0)) {
+                        if ((xn ? !hm : !hp) && a[1] == T(0)) {
                             const V z = pfma(sxv, bc(xn ? -hxh : hxh), f0);
                             zxp[0] = pfma(z, bw, zxp[0]); zxp[1] = pfma(z, bv, zxp[1]);
                             zxs[0] = pfma(z.x, d[1], zxs[0]); zxs[1] = pfma(z.x, e[1], zxs[1]);
                         }
-                        if ((yn ? !vm : !vp) && d[1] == T(0)) {
+                        if ((yn ? !vm : !vp) && a[2] == T(0)) {
                             const V z = pfma(syv, bc(yn ? -hyh : hyh), f0);
                             zyp[0] = pfma(z, bw, zyp[0]); zyp[1] = pfma(z, bu, zyp[1]);
                             zys[0] = pfma(z.x, a[3], zys[0]); zys[1] = pfma(z.x, d[2], zys[1]);

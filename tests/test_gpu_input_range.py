@@ -63,3 +63,13 @@ def test_wide_velocity_grid_in_hot_gas(hb, half_width):
         h[n], b[n] = H * skew, H * skew * 0.5 * T[:, None]
         W[n] = np.stack([rho, rho * U, rho * V, 0.5 * rho * (U ** 2 + V ** 2) + 0.75 * rho * T], 1)
     compare(hb, c, (W, h, b), 1, 2e-5, 2e-7)
+
+
+@pytest.mark.parametrize("node", [1e-18, 1e-24, 1e-30])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_velocity_node_close_to_zero(hb, node, precision):
+    # a node whose square lies below the smallest 32-bit value still moves into the walls on its side
+    c = I.make_case("tiny", 5, 9, kn=0.3, st=1.0, nh=1, pr=2 / 3, drive="thermal", amp=0.3, precision=precision)
+    c.u, c.v = c.u.copy(), c.v.copy()
+    c.u[4], c.v[4] = node, -node
+    compare(hb, c, I.initial_state(c, seed=3), 2, *((1e-10, 1e-13) if precision == 0 else (2e-5, 2e-7)))
