@@ -318,8 +318,8 @@ std::vector<int> class_order(const std::vector<double>& x)
 }
 
 // The FP64 face sums keep their slopes for the micro update, which then takes 0 of its 45 slope instructions per update,
-// while those of all cases of a handle take at most 8 GiB (32 bytes per update beside the state's 32); larger handles
-// form them twice and need the memory they always needed.  Micro update 46.4 -> 35.5 ms (twelve 64x64, 32x32, N_T 3,
+// while those of all cases of a handle take at most 8 GiB (32 bytes per update beside the state's 32) and the caller's
+// workspace has room for them; other handles form them twice.  Micro update 46.4 -> 35.5 ms (twelve 64x64, 32x32, N_T 3,
 // FP64), 20.8 -> 16.3 ms (64x64, 48x48, N_T 7), 0.668 -> 0.479 ms (32x32, 24x24), the face sums unchanged.
 constexpr size_t KEPT_SLOPES_MAX = 8ull << 30;
 
@@ -492,8 +492,10 @@ int k4_groups_per_cta(March m, int nt, bool imp, int total)
     return 1;
 }
 
+// lays the cases out over `base` and returns the bytes they take (base null: only measures); keep_slopes: with the
+// limited slopes where KEPT_SLOPES_MAX allows
 template <typename T>
-size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
+size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base, bool keep_slopes)
 {
     Carver cv{base};
     im.hc.resize(ncases);
@@ -539,7 +541,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base)
     size_t slopes = 0;
     for (const HostCase& h : im.hc) slopes += slope_bytes<T>(h);
     for (int k = 0; k < ncases; ++k) {
-        layout_case(cv, im.hc[k], im.dc[k], slopes > 0 && slopes <= KEPT_SLOPES_MAX);
+        layout_case(cv, im.hc[k], im.dc[k], keep_slopes && slopes > 0 && slopes <= KEPT_SLOPES_MAX);
         im.dc[k].st = im.d_status + k;
         im.dc[k].tol = im.d_tol;
         im.dc[k].err = im.d_err;
@@ -1102,9 +1104,9 @@ hbugks_status autotune(hbugks_t h, Impl<T>& im, int ncases)
 }
 
 template <typename T>
-hbugks_status do_create(hbugks_t h, Impl<T>& im, int ncases, const hbugks_case* cases)
+hbugks_status do_create(hbugks_t h, Impl<T>& im, int ncases, const hbugks_case* cases, bool keep_slopes)
 {
-    plan(im, ncases, cases, h->ws);
+    plan(im, ncases, cases, h->ws, keep_slopes);
     for (auto& hc : im.hc) {
         if (hc.k4shape < 0) return HBUGKS_EINVAL;
     }
@@ -1247,24 +1249,40 @@ double* noalloc_scratch(int dev)
 
 // ====================================================================================== ABI
 
-extern "C" {
+namespace {
 
-size_t hbugks_workspace_bytes(int ncases, const hbugks_case* cases)
+// bytes a handle of these cases takes, with the slopes it would keep or without; 0 if the cases are invalid
+size_t measure(int ncases, const hbugks_case* cases, bool keep_slopes)
 {
-    Range range_("hbugks_workspace_bytes");
     if (ncases < 1 || !cases) return 0;
     for (int k = 0; k < ncases; ++k)
         if (!validate(cases[k]) || cases[k].phys.precision != cases[0].phys.precision) return 0;
     try {
         if (cases[0].phys.precision == 1) {
             Impl<float> im;
-            return plan(im, ncases, cases, nullptr);
+            return plan(im, ncases, cases, nullptr, keep_slopes);
         }
         Impl<double> im;
-        return plan(im, ncases, cases, nullptr);
+        return plan(im, ncases, cases, nullptr, keep_slopes);
     } catch (...) {
         return 0;
     }
+}
+
+}  // namespace
+
+extern "C" {
+
+size_t hbugks_workspace_bytes(int ncases, const hbugks_case* cases)
+{
+    Range range_("hbugks_workspace_bytes");
+    return measure(ncases, cases, true);
+}
+
+size_t hbugks_workspace_min_bytes(int ncases, const hbugks_case* cases)
+{
+    Range range_("hbugks_workspace_min_bytes");
+    return measure(ncases, cases, false);
 }
 
 hbugks_status hbugks_create(int ncases, const hbugks_case* cases, void* d_workspace, size_t bytes,
@@ -1274,7 +1292,8 @@ hbugks_status hbugks_create(int ncases, const hbugks_case* cases, void* d_worksp
     if (!out || !d_workspace || ((uintptr_t)d_workspace & 255)) return HBUGKS_EINVAL;
     size_t need = hbugks_workspace_bytes(ncases, cases);
     if (need == 0) return HBUGKS_EINVAL;
-    if (bytes < need) return HBUGKS_ENOMEM;
+    const bool keep_slopes = bytes >= need;
+    if (!keep_slopes && bytes < measure(ncases, cases, false)) return HBUGKS_ENOMEM;
     hbugks_t h = new (std::nothrow) hbugks_solver;
     if (!h) return HBUGKS_ENOMEM;
     h->ncases = ncases;
@@ -1294,10 +1313,10 @@ hbugks_status hbugks_create(int ncases, const hbugks_case* cases, void* d_worksp
         h->st_host.resize(ncases);
         if (h->precision == 1) {
             h->f = new Impl<float>;
-            rc = do_create(h, *h->f, ncases, cases);
+            rc = do_create(h, *h->f, ncases, cases, keep_slopes);
         } else {
             h->d = new Impl<double>;
-            rc = do_create(h, *h->d, ncases, cases);
+            rc = do_create(h, *h->d, ncases, cases, keep_slopes);
         }
     } catch (const std::bad_alloc&) {
         rc = HBUGKS_ENOMEM;

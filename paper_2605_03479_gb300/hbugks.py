@@ -63,7 +63,7 @@ EXPORTED = ("hbugks_workspace_bytes", "hbugks_create", "hbugks_destroy", "hbugks
             "hbugks_harmonic_noalloc", "hbugks_launches_per_iteration", "hbugks_get_tile_shape",
             "hbugks_set_tile_shape", "hbugks_cuda_error_string", "hbugks_test_expire_wait",
             "hbugks_copy_state", "hbugks_set_loop_mode", "hbugks_get_micro_variant",
-            "hbugks_set_micro_variant")
+            "hbugks_set_micro_variant", "hbugks_workspace_min_bytes")
 
 
 def lib():
@@ -79,6 +79,8 @@ def lib():
             pc = C.POINTER(Case)
             L.hbugks_workspace_bytes.argtypes = [i, pc]
             L.hbugks_workspace_bytes.restype = sz
+            L.hbugks_workspace_min_bytes.argtypes = [i, pc]
+            L.hbugks_workspace_min_bytes.restype = sz
             L.hbugks_create.argtypes = [i, pc, vp, sz, vp, C.POINTER(vp)]
             L.hbugks_destroy.argtypes = [vp]
             L.hbugks_destroy.restype = None
@@ -109,8 +111,8 @@ def lib():
             L.hbugks_copy_state.argtypes = [vp, i, vp, i]
             L.hbugks_set_loop_mode.argtypes = [vp, i]
             for name in EXPORTED:
-                if name not in ("hbugks_workspace_bytes", "hbugks_destroy", "hbugks_iteration_count",
-                                "hbugks_status_string", "hbugks_cuda_error_string"):
+                if name not in ("hbugks_workspace_bytes", "hbugks_workspace_min_bytes", "hbugks_destroy",
+                                "hbugks_iteration_count", "hbugks_status_string", "hbugks_cuda_error_string"):
                     getattr(L, name).restype = C.c_int
             _lib = L
     return _lib
@@ -184,7 +186,15 @@ class Solver:
         if nbytes == 0:
             raise HbugksError(EINVAL, "hbugks_workspace_bytes")
         self.device = torch.device(device)
-        self.workspace = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
+        try:
+            self.workspace = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
+        except torch.OutOfMemoryError:
+            # an FP64 handle can do without the slopes it would keep between two kernels
+            least = int(lib().hbugks_workspace_min_bytes(len(self._args), arr))
+            if least >= nbytes:
+                raise
+            nbytes = least
+            self.workspace = torch.empty(nbytes + 256, dtype=torch.uint8, device=self.device)
         if workspace_fill is not None:
             self.workspace.fill_(int(workspace_fill))
             torch.cuda.synchronize(self.device)
