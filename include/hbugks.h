@@ -224,7 +224,7 @@ HBUGKS_API hbugks_status hbugks_harmonic_noalloc(int nx, int ny, int nu, int nv,
  * (with vpl 2 two and 32), 2x2 two and 2, 8x4 four and 32 (two columns instead of four where four do not fit, or in a
  * mesh of fewer than four columns).  hbugks_create() picks one per case by timing every variant the
  * case can run on the case itself (autotuning, cached per process by mesh size, velocity grid, level count,
- * precision and SM count).  get: the variant of case `case_index`.  set: pin one, for example to reproduce a
+ * precision, spectral source, collision model, SM count, one case or several, slopes kept or not).  get: the variant of case `case_index`.  set: pin one, for example to reproduce a
  * run exactly; HBUGKS_EINVAL if it is not one of these, its tile needs more shared memory than a CTA may have, or it
  * needs what the case lacks.  Every variant gives bitwise the same iterate; the state is unchanged and the iteration
  * graphs are rebuilt.  The tile-shape pair is the same with vpl = 1 (set) or any vpl (get).  The paper has no

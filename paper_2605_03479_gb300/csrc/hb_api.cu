@@ -1026,8 +1026,9 @@ hbugks_status upload_offsets(hbugks_t h, Impl<T>& im)
 // twice against shared memory and registers per CTA, and on small meshes against the number of CTAs;
 // which wins depends on the level count, the velocity grid, the mesh and the GPU.  Each variant the case can
 // run is timed on the case itself (one warm-up launch, then three), after one iteration from rest has filled
-// the parameters the kernel reads.  Choices are cached per process by everything that sets the launch: mesh
-// size, velocity grid, blocks, levels, precision, SM count and the form of the spectral source.
+// the parameters the kernel reads.  Choices are cached per process by everything that sets the launch and its time: mesh
+// size, velocity grid, blocks, levels, precision, SM count, the form of the spectral source, whether the handle holds one
+// case (which may go as a kernel parameter), whether slopes are kept, and the collision model.
 
 struct TuneCache {
     std::mutex mu;
@@ -1051,7 +1052,8 @@ hbugks_status autotune(hbugks_t h, Impl<T>& im, int ncases)
         std::lock_guard<std::mutex> lk(tune_cache().mu);
         for (int k = 0; k < ncases; ++k) {
             const HostCase& hc = im.hc[k];
-            keys[k] = {hc.nx, hc.ny, hc.nu, hc.nv, hc.nvb, hc.nt, (int)sizeof(T), sms, im.any_implicit ? 1 : 0};
+            keys[k] = {hc.nx, hc.ny, hc.nu, hc.nv, hc.nvb, hc.nt, (int)sizeof(T), sms, im.any_implicit ? 1 : 0,
+                       ncases == 1 ? 1 : 0, im.dc[k].sl ? 1 : 0, im.dc[k].shakhov};
             auto it = tune_cache().best.find(keys[k]);
             if (it != tune_cache().best.end()) im.hc[k].k4shape = it->second;
             else need = true;
