@@ -21,7 +21,7 @@
 namespace hb {
 
 // van Leer limiter of a pair: 2 s1 s2 / (s1 + s2) where s1 s2 > 0, else 0.  Single precision: the limited slope
-// needs no correctly rounded division (approximate reciprocal, 2 ulp); double precision: rcp64
+// needs no correctly rounded division (approximate reciprocal, 2 ulp); double precision: rcp64_normal
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
@@ -39,12 +39,16 @@ __device__ __forceinline__ float2 vleer2(float2 s1, float2 s2)
     const float2 q = pmul(p, make_float2(rcp_approx(den.x), rcp_approx(den.y)));
     return make_float2(p.x > 0.f ? q.x : 0.f, p.y > 0.f ? q.y : 0.f);
 }
-// x > 0 from the high word, off the FP64 pipe (false for NaN; a positive denormal below 2^-1042 counts as zero)
-__device__ __forceinline__ bool pos64(double x) { return (unsigned)(__double2hiint(x) - 1) < 0x7ff00000u; }
+// x > 0 by integer arithmetic, off the FP64 pipe (false for NaN)
+__device__ __forceinline__ bool pos64(double x)
+{
+    return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull;
+}
 __device__ __forceinline__ double2 vleer2(double2 s1, double2 s2)
 {
     const double px = s1.x * s2.x, py = s1.y * s2.y;
-    const double qx = px * rcp64(__dadd_rn(s1.x, s2.x)), qy = py * rcp64(__dadd_rn(s1.y, s2.y));
+    // where the product is positive the sum lies above 2^-537, a normal number
+    const double qx = px * rcp64_normal(__dadd_rn(s1.x, s2.x)), qy = py * rcp64_normal(__dadd_rn(s1.y, s2.y));
     return make_double2(pos64(px) ? qx : 0.0, pos64(py) ? qy : 0.0);
 }
 

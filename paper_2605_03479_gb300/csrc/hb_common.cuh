@@ -314,14 +314,27 @@ template <> __device__ __forceinline__ float t_expm1<float>(float x) { return ex
 
 // 1 / x in double precision by Newton's iteration in its cubically convergent form r (1 + e + e^2), e = 1 - x r,
 // from the hardware's approximation (relative error about 2^-20, so e^3 lies below the last bit): 3 FMAs, within
-// 1 ulp, where a correctly rounded division costs 9.  An FP64 instruction occupies its scheduler for 64 cycles here,
-// so the per-cell and per-face arithmetic and the FP64 slopes pay for every one of them.  x = 0 or infinite gives NaN.
+// 1 ulp of the rounded quotient, where a division costs 9.  An FP64 instruction occupies its scheduler for 64 cycles here,
+// so the per-cell and per-face arithmetic and the FP64 slopes pay for every one of them.  e receives the residual.  For
+// 2^-1022 <= |x| <= 2^1021 (anything else may give NaN).
+__device__ __forceinline__ double rcp64_normal(double x, double& r, double& e)
+{
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double rcp64_normal(double x)
+{
+    double r, e;
+    return rcp64_normal(x, r, e);
+}
+// the same for every x: where the residual is not finite the approximation is the answer, infinity for 0 and denormal x,
+// 0 for infinite x (a denormal 1/x is 0); the test runs off the FP64 pipe
 __device__ __forceinline__ double rcp64(double x)
 {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
+    double r, e;
+    const double y = rcp64_normal(x, r, e);
+    return 2u * (unsigned)__double2hiint(e) < 0xffe00000u ? y : r;
 }
 
 // primitive variables from W = (rho, rho U, rho V, rho E) with D + K = 3
