@@ -221,14 +221,15 @@ HBUGKS_API hbugks_status hbugks_harmonic_noalloc(int nx, int ny, int nu, int nv,
  * The variants are 4x4, 4x2, 2x2 and 8x4 with vpl 1, and 4x2 with vpl 2, which needs single precision and sign
  * classes that each hold an even number of velocity blocks.  The kernel marches over a strip of columns on all
  * levels; a variant sets the strip and the rows it marches over: 4x4 four columns and 16 rows, 4x2 two and 16
- * (with vpl 2 two and 32), 2x2 two and 2, 8x4 four and 32 (two columns instead of four where four do not fit, or in a
- * mesh of fewer than four columns).  hbugks_create() picks one per case by timing every variant the
+ * (with vpl 2 two and 32), 2x2 two and 2, 8x4 four and 32 (two columns instead of four above 11 levels, where four do not
+ * fit, or in a mesh of fewer than four columns). hbugks_create() picks one per case by timing every variant the
  * case can run on the case itself (autotuning, cached per process by mesh size, velocity grid, level count,
- * precision, spectral source, collision model, SM count, one case or several, slopes kept or not).  get: the variant of case `case_index`.  set: pin one, for example to reproduce a
- * run exactly; HBUGKS_EINVAL if it is not one of these, its tile needs more shared memory than a CTA may have, or it
- * needs what the case lacks.  Every variant gives bitwise the same iterate; the state is unchanged and the iteration
- * graphs are rebuilt.  The tile-shape pair is the same with vpl = 1 (set) or any vpl (get).  The paper has no
- * counterpart (a GPU tuning choice). */
+ * precision, spectral source, collision model, SM count, one case or several, slopes kept or not). get: the
+ * variant of case `case_index`. set: pin one, for example to reproduce a run exactly; HBUGKS_EINVAL if it is not
+ * one of these, a tile of that size with its halo, parameters and fluxes on every level would not fit a CTA's
+ * shared memory (the limit of the names, not of the strips), or it needs what the case lacks. Every variant gives
+ * bitwise the same iterate; the state is unchanged and the iteration graphs are rebuilt. The tile-shape pair is
+ * the same with vpl = 1 (set) or any vpl (get). The paper has no counterpart (a GPU tuning choice). */
 HBUGKS_API hbugks_status hbugks_get_micro_variant(hbugks_t h, int case_index, int* tx, int* ty, int* vpl);
 HBUGKS_API hbugks_status hbugks_set_micro_variant(hbugks_t h, int case_index, int tx, int ty, int vpl);
 HBUGKS_API hbugks_status hbugks_get_tile_shape(hbugks_t h, int case_index, int* tx, int* ty);

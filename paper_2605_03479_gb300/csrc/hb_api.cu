@@ -159,8 +159,9 @@ March k4_march_of(int shape, int nx, int nt, int nuv, bool imp)
     return {s.cols == 4 && nx >= 4 && levels && k4_smem_of<T>(4, nt, imp) <= SMEM_MAX ? 4 : 2, s.rows};
 }
 
-// Bytes a tile of a variant holds: its cells on all levels, twice its halo rectangle, face and cell parameters and
-// fluxes.  A variant is offered for a case while that fits a CTA's shared memory.
+// Which variants the ABI offers a case.  The five names are tiles, and a name is accepted while a tile of its size (its cells
+// on all levels, twice its halo rectangle, face and cell parameters and fluxes) would fit a CTA's shared memory: what a
+// caller was refused stays refused.  The strip a name stands for needs less (k4_smem_of) and always fits.
 template <typename T>
 size_t k4_tile_bytes(int shape, int nt)
 {
@@ -170,7 +171,7 @@ size_t k4_tile_bytes(int shape, int nt)
     return nt * cells * pair + 2 * halo * pair + 2 * (faces * NP + cells * NCP) * sizeof(T) + 2 * faces * pair;
 }
 
-// largest tile two of which fit an SM's shared memory, else the largest that fits at all
+// the first name two of whose tiles would fit an SM's shared memory, else the first that is offered
 template <typename T>
 int pick_k4_shape(int nt)
 {
@@ -181,8 +182,8 @@ int pick_k4_shape(int nt)
     return -1;
 }
 
-// a K4 variant a case of this precision is offered: its tile fits a CTA, and two velocity blocks per CTA need single
-// precision and sign classes of an even number of blocks
+// a K4 variant a case of this precision is offered: its tile would fit a CTA, and the name with two velocity blocks needs
+// single precision and sign classes of an even number of blocks
 template <typename T>
 bool k4_shape_ok(int shape, int nt, bool pairs)
 {
@@ -529,7 +530,7 @@ size_t plan(Impl<T>& im, int ncases, const hbugks_case* cases, char* base, bool 
     std::sort(nts.begin(), nts.end());
     for (int nt : nts)
         for (int cols : {2, 4})
-            for (int rows : {2, 8, 16, 32}) {
+            for (int rows : {2, 16, 32}) {
                 add(4, 0);
                 im.specs.back().nt = nt;
                 im.specs.back().march = March{cols, rows};
@@ -904,6 +905,7 @@ void enqueue_iteration(Impl<T>& im, int ncases, cudaStream_t s, cudaEvent_t* ev 
             cudaEventRecord(ev[2 * slot], s);
             open_slot = slot;
         }
+        // stage names of the traces: k4_cells is the micro update (k4_march), k_tables a part of k3_macro's launch
         static const char* const names[5] = {"k1_cells", "k2_face_params", "k3_macro", "", "k4_cells"};
         Range r(names[sp.kind]);
         const Batch<T> b{im.d_cases, ncases, im.d_off + (size_t)sp.table * stride};

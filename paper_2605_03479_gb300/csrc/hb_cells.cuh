@@ -79,8 +79,6 @@ __device__ __forceinline__ void mbar_setup(uint64_t* bars, int n)
     __syncthreads();
 }
 
-__host__ __device__ constexpr size_t round16(size_t b) { return (b + 15) / 16 * 16; }
-
 // Sum over the 32 lanes of each of v[0..N-1] (N <= 32), recursive halving: after the step with distance d the
 // lanes with bit d set hold the upper half of the remaining values.  Returns, on lane l, the total of v[l]
 // (0 for l >= N).  v is destroyed.

@@ -450,18 +450,4 @@ __device__ inline void eq_cell(double rho, double U, double V, double lam, doubl
     o[E_Q + 3] = T(2.0 * lam);
 }
 
-// Horner evaluation of the bivariate cubic with monomials 1, u, v, u^2, uv, v^2, u^3, u^2 v, u v^2, v^3
-template <typename T>
-__device__ __forceinline__ T cubic(const T* c, T u, T v)
-{
-    T yv = c[0] + v * (c[2] + v * (c[5] + v * c[9]));
-    T ux = (c[1] + v * (c[4] + v * c[8])) + u * ((c[3] + v * c[7]) + u * c[6]);
-    return yv + u * ux;
-}
-
-// ----------------------------------------------------------------------- analytic velocity sums
-// Discrete sums of polynomial x Maxwellian over the tensor velocity grid factor into 1-D sums
-//   X[p] = sum_i wu_i u_i^p exp(-lam (u_i - U)^2)  (over u_i > 0, u_i < 0, u_i = 0 or all),
-//   Y[q] likewise in v,  so  sum_a w_a u^p v^q rho (lam/pi) e^{-lam |u - U|^2} = rho lam/pi X[p] Y[q].
-
 }  // namespace hb
