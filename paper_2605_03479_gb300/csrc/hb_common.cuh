@@ -348,12 +348,20 @@ __device__ __forceinline__ void prim(const double* W, double& rho, double& U, do
     lam = 0.75 * rho * rcp64(fma(-0.5 * rho, fma(U, U, V * V), W[3]));
 }
 
-// tau = mu/p, mu = mu0 (T/T0)^w, T/T0 = lam0/lam, p = rho/(2 lam); ir = 1/rho, i2l = 1/(2 lam).  pow, not
-// exp(-w log(lam/lam0)): it keeps the last digits of the logarithm, and with a whole exponent it is defined for the
-// negative temperature a cell may pass through.
-__device__ __forceinline__ double relax_time(double mu0, double w, double lam0, double ir, double lam, double i2l)
+// x^-w for x = lam/lam0 = T0/T, rx = 1/x.  exp(y) of the rounded y = -w log x, for half the instructions of pow, where it is
+// as exact: within 1 ulp of exp and 1.5 |y| ulp of y's roundings, at |y| <= 1/4 no more than pow (1 ulp) of a rounded
+// quotient (w/2 ulp) with the w <= 1 of a viscosity law.  pow beyond, where the lost digits of the logarithm would show, and
+// below zero temperature, where y is not a number and a whole exponent still gives one.
+__device__ __forceinline__ double temperature_power(double x, double rx, double w)
 {
-    return mu0 * pow(2.0 * lam0 * i2l, w) * 2.0 * lam * ir;
+    const double y = -w * log(x);
+    return fabs(y) <= 0.25 ? exp(y) : pow(rx, w);
+}
+
+// tau = mu/p, mu = mu0 (T/T0)^w, T/T0 = lam0/lam, p = rho/(2 lam); il0 = 1/lam0, ir = 1/rho, i2l = 1/(2 lam)
+__device__ __forceinline__ double relax_time(double mu0, double w, double lam0, double il0, double ir, double lam, double i2l)
+{
+    return mu0 * temperature_power(lam * il0, 2.0 * lam0 * i2l, w) * 2.0 * lam * ir;
 }
 
 // Coefficients of Eq. C_coeffs: Taylor series in x = dG/tau below x = 1 (the printed forms cancel there),

@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(K2_ITEMS * K2_WARPS) k2_face_params(Batch<T> B
         else dGf = fmin(cd.dG[cL], cd.dG[cR]);
         sdG[lane] = dGf;
         T Ct[5];
-        ugks_coeffs<T>(T(dGf), T(relax_time(cd.mu0, cd.w_vss, cd.lam0, ir, lamf, i2ld)), Ct);
+        ugks_coeffs<T>(T(dGf), T(relax_time(cd.mu0, cd.w_vss, cd.lam0, il0, ir, lamf, i2ld)), Ct);
 #pragma unroll
         for (int k = 0; k < 5; ++k) Cw[k][lane] = Ct[k];
     } else {
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
             for (int k = 0; k < 13; ++k) A[k] = cm[k] + cd.refmom[k];
             prim(Wc, rho, U, V, lam);
             heat_flux_raw(A, U, V, qx, qy);
-            tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, rcp64(rho), lam, 0.5 * rcp64(lam));
+            tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, il0, rcp64(rho), lam, 0.5 * rcp64(lam));
             sq[r][0] = qx;
             sq[r][1] = qy;
         } else {
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(K3_MAXTHREADS) k3_macro(Batch<T> B)
 #pragma unroll
         for (int k = 0; k < 4; ++k) Wn[((size_t)n * nc + c) * 4 + k] = wn[k];
         prim(wn, rho, U, V, lam);
-        tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, rcp64(rho), lam, 0.5 * rcp64(lam));
+        tau = relax_time(cd.mu0, cd.w_vss, cd.lam0, il0, rcp64(rho), lam, 0.5 * rcp64(lam));
         stau[r] = tau;
         snu[r] = nu_conv(cd, U, V, lam, idx_, idy);        // for the next local step
     }
