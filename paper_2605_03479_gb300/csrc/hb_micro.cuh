@@ -62,8 +62,8 @@ __device__ __forceinline__ void flux_core(const T* fp, int qo, int lo, L ex, L e
     load_par(fp + lo, l);
     c4 = sc[5];
     c5 = sc[6];
-    const L dH = pmul(hr, pfma(A::all(sc[1]), pfma(ex, ey, padd(ex, ey)), A::all(sc[0])));
-    const L H = padd(hr, dH), cH = pmul(A::all(sc[4]), dH);
+    const L G = pfma(A::all(sc[1]), pfma(ex, ey, padd(ex, ey)), A::all(sc[0]));
+    const L dH = pmul(hr, G), H = pfma(hr, G, hr), cH = pmul(A::all(sc[4]), dH);
     // Horner form of the bivariate cubic with monomials 1, u, v, u^2, uv, v^2, u^3, u^2 v, u v^2, v^3
     const L y0 = pfma(v, pfma(v, pfma(v, A::all(c[9]), A::all(c[5])), A::all(c[2])), A::all(c[0]));
     const L y1 = pfma(v, pfma(v, A::all(c[8]), A::all(c[4])), A::all(c[1]));
