@@ -47,7 +47,7 @@ typedef enum {
     HBUGKS_NOT_CONVERGED = 1,   /* warning: the iteration budget ran out before the residual target */
     HBUGKS_EINVAL = -1,         /* invalid argument (sizes, pointers, unsupported combination) */
     HBUGKS_ECUDA = -2,          /* a CUDA runtime call failed */
-    HBUGKS_ENOMEM = -3,         /* workspace smaller than hbugks_workspace_bytes(), or host memory exhausted */
+    HBUGKS_ENOMEM = -3,         /* workspace smaller than hbugks_workspace_min_bytes(), or host memory exhausted */
     HBUGKS_DIVERGED = -4,       /* a residual became NaN/Inf or exceeded 1e10 */
     HBUGKS_TIMEOUT = -5         /* a bounded device-side wait ran out (500 ms for a bulk copy); the iteration
                                    in which it happened left the state unchanged */

@@ -318,10 +318,10 @@ std::vector<int> class_order(const std::vector<double>& x)
     return o;
 }
 
-// The FP64 face sums keep their slopes for the micro update, which then takes 0 of its 45 slope instructions per update,
-// while those of all cases of a handle take at most 8 GiB (32 bytes per update beside the state's 32) and the caller's
-// workspace has room for them; other handles form them twice.  Micro update 46.4 -> 35.5 ms (twelve 64x64, 32x32, N_T 3,
-// FP64), 20.8 -> 16.3 ms (64x64, 48x48, N_T 7), 0.668 -> 0.479 ms (32x32, 24x24), the face sums unchanged.
+// The FP64 face sums keep their slopes for the micro update, which then forms none, while those of all cases of a handle
+// take at most 8 GiB (32 bytes per update beside the state's 32) and the caller's workspace has room for them; other
+// handles form them twice.  Micro update 46.4 -> 35.1 ms (twelve 64x64, 32x32, N_T 3,
+// FP64), 20.8 -> 16.2 ms (64x64, 48x48, N_T 7), 0.668 -> 0.485 ms (32x32, 24x24), the face sums unchanged.
 constexpr size_t KEPT_SLOPES_MAX = 8ull << 30;
 
 template <typename T>

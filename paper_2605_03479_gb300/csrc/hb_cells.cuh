@@ -146,7 +146,7 @@ __device__ __forceinline__ void load_par(const double* p, double (&o)[N])
 // for the staged blocks (three times the tile's own cells pass from L2) at 56 % issue.  Against 59 sums with the
 // reconstruction formed per velocity, divisions in the limiter and weights formed per lane from two loads: 36.98 ->
 // 22.2 ms (twelve 64x64 cavities, 32x32 velocities, N_T 3, FP64, SEP), 18.22 -> 11.3 ms (64x64, 48x48, N_T 7, FP64),
-// 4.83 -> 3.34 ms (128x128, 64x64, N_T 11, FP32, SEP), 0.543 -> 0.463 ms (64x64, 48x48, FP32).  Tiles of 4x2 cells:
+// 4.83 -> 3.34 ms (128x128, 64x64, N_T 11, FP32, SEP), 0.543 -> 0.457 ms (64x64, 48x48, FP32).  Tiles of 4x2 cells:
 // 4x4 4.11 ms, 6x4 3.96, 8x3 4.14 on the 128x128 case, whose larger CTAs wait for their slowest warp.
 // Weights of a velocity block in global and shared memory, T [K1_WT]: SEP four per lane (w_v v^0..3), then w_v v^4 per
 // lane; general four, four and four per lane (w times 1, u, v, uu; uv, vv, uuu, uuv; uvv, vvv, uu|u|^2, vv|u|^2), then

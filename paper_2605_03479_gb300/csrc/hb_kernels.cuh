@@ -80,9 +80,9 @@ __device__ __forceinline__ void heat_flux_raw(const double* A, double U, double 
 //   D  warp 0 the macro flux and the wall density, 1 and 2 the micro-flux parameters of the two upwind sides, 3 the rest.
 // On small meshes the time is the chain of one thread, in large ones FP64 instructions and latency at few warps.
 // Against one thread per item doing all of it (219 registers, nine FP64 instructions per division, polynomials in (u, v)
-// whose axis was known at run time only): 57 -> 29 us (8x8, N_T 3), 0.210 -> 0.139 ms (64x64, 48x48, N_T 7),
-// 5.49 -> 3.94 ms (48 uneven cavities), 1.12 -> 0.70 ms (128x128, 64x64, N_T 11); FP64 0.190 -> 0.078 ms (32x32, 24x24)
-// and 2.97 -> 2.03 ms (twelve 64x64, 32x32).  32 items fill a warp; 4 warps balance the parts of A and C.
+// whose axis was known at run time only): 57 -> 27 us (8x8, N_T 3), 0.210 -> 0.136 ms (64x64, 48x48, N_T 7),
+// 5.49 -> 3.80 ms (48 uneven cavities), 1.12 -> 0.68 ms (128x128, 64x64, N_T 11); FP64 0.190 -> 0.077 ms (32x32, 24x24)
+// and 2.97 -> 1.98 ms (twelve 64x64, 32x32).  32 items fill a warp; 4 warps balance the parts of A and C.
 constexpr int K2_ITEMS = 32, K2_WARPS = 4, K2_NODES = 32;
 
 // All polynomials are kept in the face's own velocity components, n along its normal and t along the other axis, in
@@ -534,8 +534,8 @@ __global__ void k_steps(Batch<T> B)
 // warps then write the expm1 tables of the CTA's equilibria.  Bound by FP64 instructions, and on small meshes by
 // the length of one thread's chain of them: the previous layout (a thread per cell running over its levels, then a
 // kernel of 128 cell-levels per CTA for the tables) left most of the chip idle.  Measured before -> now, both parts:
-// 115 -> 18 us (8x8 cells, N_T 3), 262 -> 57 us (64x64, N_T 7), 482 -> 255 us (128x128, N_T 11), 754 -> 49 us (32x32,
-// N_T 11, spectral source at the new iterate), 236 -> 36 us (32x32, N_T 3, FP64 tables).  8 cells per CTA give a
+// 115 -> 18 us (8x8 cells, N_T 3), 262 -> 51 us (64x64, N_T 7), 482 -> 215 us (128x128, N_T 11), 754 -> 45 us (32x32,
+// N_T 11, spectral source at the new iterate), 236 -> 35 us (32x32, N_T 3, FP64 tables).  8 cells per CTA give a
 // 32x32 mesh 128 CTAs and still fill three quarters of the lanes at N_T = 3.
 constexpr int K3_MAXTHREADS = 2 * ((MAXNT * K3_CELLS + 31) / 32) * 32;
 // warps of one half for nt levels, and threads of the launch for the largest nt of its cases (at least four warps,

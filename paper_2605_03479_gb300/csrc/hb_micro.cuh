@@ -11,16 +11,17 @@
 // with it, and u s_x, u (F_downwind - F_upwind) keep theirs, so one code serves the four sign classes.  Only the
 // strip's upwind column and the segment's upwind row are computed twice (one flux each).
 //
-// Bound by instruction issue in single precision: about 235 warp instructions per 32 updates, 130 of them floating
+// Bound by instruction issue in single precision: 232 warp instructions per 32 updates, some 130 of them floating
 // point, where the previous kernel (a tile of cells per CTA, fluxes through shared memory, one barrier per level) needed
 // 422.  The shared-memory loads serve two velocities per lane, the expm1 factors are loaded ahead of their use (their L2
 // latency was 46 % of the stalls), and the x direction is a template parameter so that all offsets within a row are
 // constants.  Strips of two columns with 128 registers hold more warps per SM and win up to 7 levels (0.83 against
-// 1.02 ms, 64x64, 48x48, N_T 7), strips of four with 168 recompute less and win above (8.3 ms, 128x128, 64x64, N_T 11).
+// 1.02 ms, 64x64, 48x48, N_T 7), strips of four with 168 recompute less and win above (8.2 ms, 128x128, 64x64, N_T 11).
 // Bound by the FP64 pipe in FP64.  Previous kernel
-// -> this one: 16.25 -> 8.27 ms (128x128, 64x64, N_T 11), 1.50 -> 0.83 ms (64x64, 48x48, N_T 7), 44.5 -> 25.8 ms (48
-// uneven cavities), 0.60 -> 0.32 ms (90x90, 28x28, N_T 3); FP64 58.1 -> 46.4 ms (twelve 64x64, 32x32, N_T 3) and 25.8 ->
-// 20.8 ms (64x64, 48x48, N_T 7).
+// -> this one: 16.25 -> 8.23 ms (128x128, 64x64, N_T 11), 1.50 -> 0.83 ms (64x64, 48x48, N_T 7), 44.5 -> 25.9 ms (48
+// uneven cavities), 0.60 -> 0.32 ms (90x90, 28x28, N_T 3), 0.56 -> 0.68 ms where a class is one block (160x160, 10x10, N_T
+// 7: the second half of every pair repeats it); FP64 with kept slopes 58.1 -> 35.1 ms (twelve 64x64, 32x32, N_T 3) and
+// 25.8 -> 16.2 ms (64x64, 48x48, N_T 7).
 #pragma once
 #include "hb_cells.cuh"
 
